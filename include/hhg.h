@@ -572,29 +572,27 @@ hhg_status hhg_learn_stats(hhg_ctx* ctx, hhg_learn_stats_report* report, int res
 hhg_status hhg_apply_host(hhg_ctx* ctx, int level, hhg_dtype dt, const void* x_host, void* y_host);
 
 /* Kernel timing.  enable != 0 starts (and resets) recording CUDA events around the
- * parts of every operator sweep: the macro-interior launches (one per macro; they
- * alternate between the context stream and a side stream, so consecutive launches
- * overlap) and the skeleton kernels (on a second side stream, concurrent with the
- * interior).  ms_host[2] and launches_host[2] (nullable) receive the accumulated span
- * of each part (first start to last end, device time) and its launch count since the
- * last call; span / launches is the interior launches' effective duration.  Waits for
+ * parts of every operator sweep: the launches that hold the macro interiors (by default one for the
+ * whole sweep; with one launch per macro they alternate between the context stream and a side
+ * stream, so consecutive launches overlap) and, where it is a launch of its own, the skeleton kernel
+ * (on another side stream, concurrent with the interior).  ms_host[2] and launches_host[2] (nullable)
+ * receive the accumulated span of each part (first start to last end, device time) and its launch
+ * count since the last call; span / launches is the interior launches' effective duration.  Waits for
  * the stream. */
 hhg_status hhg_profile(hhg_ctx* ctx, int enable, double* ms_host, int64_t* launches_host);
 
-/* Kernel of the macro-interior sweeps of the scaled-stencil variants (results equal up to
- * rounding).  The point kernels take one thread per point for FP64 and, for FP32, one thread
- * per pair of neighbouring points of a lattice row in packed two-lane FP32 arithmetic, both
- * reading the stencil neighbours straight from global memory; they run either as one launch
- * per macro (the macro's stencil a kernel parameter) or as one launch over all macros (each
- * block copies its macro's stencil to shared memory), which suits meshes of many small
- * macros.  kernel: 0 (default) the point kernels, all macros in one launch when the mesh has
- * several macros and one macro's launch would fill fewer than two waves of the GPU, else one
- * launch per macro; 1 a block per 30 x 4 x 4 box of lattice points that stages the box plus
- * its one-point halo in shared memory (asynchronous copies) and reads every neighbour from
- * there; 2 the point kernels, one launch per macro; 3 the point kernels, all macros in one
- * launch.  The Stokes sweeps follow the same choice of launch shape; the colour passes of the
- * hybrid Gauss-Seidel smoother always run as one launch over all macros.  Errors: ARG for
- * another value. */
+/* Kernel of the sweeps of the scaled-stencil variants (results equal up to rounding).  kernel: 0
+ * (default) the whole sweep in one launch, the macro interiors by a kernel whose threads march along
+ * a lattice direction (FP32: both directions of a stencil direction pair in packed two-lane
+ * arithmetic), with the skeleton rows in blocks between theirs.  The others run the interiors beside
+ * a launch of the skeleton rows: 2 the point kernels, one launch per macro (the macro's stencil a
+ * kernel parameter), with one thread per point for FP64 and, for FP32, one thread per pair of
+ * neighbouring points of a lattice row, both reading the stencil neighbours straight from global
+ * memory; 3 the point kernels, all macros in one launch (each block copies its macro's stencil to
+ * shared memory); 1 a block per 30 x 4 x 4 box of lattice points that stages the box plus its
+ * one-point halo in shared memory (asynchronous copies) and reads every neighbour from there.  The
+ * Stokes sweeps follow the same choice (1 as 3 or 2); the colour passes of the hybrid Gauss-Seidel smoother
+ * always run as one launch over all macros.  Errors: ARG for another value. */
 hhg_status hhg_set_interior_kernel(hhg_ctx* ctx, int kernel);
 
 /* FP32 FMA issue-rate probe, a measurement aid with no counterpart in the paper: the

@@ -101,7 +101,8 @@ struct KeyHash {
 struct LevelHost {
   int level = 0, n = 0;
   int64_t nt = 0, entries = 0;
-  std::vector<int32_t> tiles_int, tiles_all, tiles_lin, tiles_pair, tiles3, gs_chunks;
+  std::vector<int32_t> tiles_int, tiles_all, tiles_lin, tiles_pair, tiles3, gs_chunks, columns;
+  int32_t column_len = 1;
   int32_t gs_ptr[9] = {0};
   std::vector<int64_t> skel_entries;
   std::vector<int32_t> skel_ptr;
@@ -109,11 +110,13 @@ struct LevelHost {
   std::vector<int8_t> skel_dir;
   std::vector<int8_t> skel_support;  // number of macro vertices spanning the node's primitive
   std::vector<std::array<int64_t, 3>> skel_key;
-  std::vector<FaceItem> face_items;
-  std::vector<int32_t> face_nodes, ev_nodes, dir_nodes;
-  std::vector<FaceItem> face_items_all;
-  std::vector<int32_t> face_nodes_all, ev_all;
-  uint32_t face_mask[4] = {0, 0, 0, 0};
+  int32_t nface_nodes = 0, nev = 0;  // free nodes on macro faces; on macro edges and vertices
+  // skeleton rows and Dirichlet entries (LevelDev); [1]: the Stokes lists
+  std::vector<RowLane> row_lanes[2];
+  std::vector<int32_t> row_warps[2];
+  std::vector<FaceBlock> face_blocks[2];
+  std::vector<FacePoint> face_points[2];
+  std::vector<int64_t> dir_entries;
   std::vector<uint8_t> mask, mask_own;  // owned copy of a free node / of any node
   std::vector<double> lumped;           // lumped P1 mass of every entry's node
   std::vector<int64_t> entry_to_unique, unique_first;
@@ -124,10 +127,9 @@ struct LevelHost {
   std::vector<int64_t> rent;
   std::vector<double> rw;
   // device
-  DevMem d_tiles_pair, d_tiles3, d_gs_chunks, d_skel_entries;
+  DevMem d_columns, d_tiles_pair, d_tiles3, d_gs_chunks, d_skel_entries;
   DevMem d_tiles_int, d_tiles_all, d_tiles_lin, d_skel_ptr, d_skel_inc, d_skel_dir, d_mask, d_first, d_e2u;
-  DevMem d_face_items, d_face_nodes, d_ev_nodes, d_dir_nodes, d_acc32, d_acc64;
-  DevMem d_face_items_all, d_face_nodes_all, d_ev_all;
+  DevMem d_row_lanes[2], d_row_warps[2], d_face_blocks[2], d_face_points[2], d_dir_entries;
   DevMem d_mask_own, d_invm64, d_invm32;  // owned-node mask; inverse lumped mass
   DevMem d_mass64, d_mass32;              // lumped mass
   DevMem d_sdiag64, d_sdiag32;            // Stokes: diagonal of -C (pressure stabilisation)
@@ -259,11 +261,10 @@ struct hhg_ctx {
   hhg_mg_params mg{HHG_SMOOTH_CHEBYSHEV, 2, 2, 2.0 / 3.0, 1.0 / 8.0, 1.1, 15, HHG_COARSE_INJECT, 3, 3, 2, 2, 0.5};
   bool mg_ready = false;
   bool prof = false;
-  // side streams of a sweep: aux[0] runs the face-node skeleton kernels, aux[1] every
-  // second macro's interior launch, aux[2] the edge/vertex kernel, aux[3] the Dirichlet
-  // rows; all forked from and joined back into `stream` by events
-  cudaStream_t aux[4] = {nullptr, nullptr, nullptr, nullptr};
-  cudaEvent_t ev_fork = nullptr, ev_join[4] = {nullptr, nullptr, nullptr, nullptr};
+  // side streams of a sweep: aux[0] runs the skeleton and Dirichlet rows, aux[1] every second
+  // macro's interior launch; both forked from and joined back into `stream` by events
+  cudaStream_t aux[2] = {nullptr, nullptr};
+  cudaEvent_t ev_fork = nullptr, ev_join[2] = {nullptr, nullptr};
   // CUDA graphs of "x = 0; one V-cycle for f" per (precision, level, f, x), replayed by
   // the solvers; dropped whenever the multigrid data change (hhg_mg_setup and friends)
   std::map<std::tuple<int, int, const void*, void*>, cudaGraphExec_t> vc_graphs;
@@ -321,8 +322,9 @@ inline int64_t max_partials(hhg_ctx* c) {
   int64_t mx = 2 * 1024;
   for (int l = c->level_min; l <= c->level_max; ++l) {
     const LevelHost& L = *c->levels[l];
-    mx = std::max<int64_t>(mx, (int64_t)std::max(L.tiles_lin.size(), L.tiles3.size()) * (int64_t)c->tets.size() +
-                                   (L.face_nodes_all.size() + 127) / 128 + L.ev_all.size() + 8);
+    mx = std::max<int64_t>(mx, (int64_t)std::max({L.tiles_lin.size(), L.tiles3.size(), (L.columns.size() + 127) / 128}) * (int64_t)c->tets.size() +
+                                   (int64_t)std::max(L.row_warps[0].size() + L.face_blocks[0].size(),
+                                                     L.row_warps[1].size() + L.face_blocks[1].size()) + 8);
   }
   return mx;
 }
@@ -438,30 +440,25 @@ inline const MacroConsts<float>* consts_dev<float>(LevelHost& L) {
   return L.d_mc32.as<MacroConsts<float>>();
 }
 
-// Fork the side streams from `stream` (they start after everything issued so far).
-inline void fork_side_streams(hhg_ctx* c) {
+// Fork the first `count` side streams from `stream` (they start after everything issued so far).
+inline void fork_side_streams(hhg_ctx* c, int count) {
   if (!c->aux[0]) {
     for (auto& st : c->aux) CK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
     CK(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
     for (auto& e : c->ev_join) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
   }
   CK(cudaEventRecord(c->ev_fork, c->stream));
-  for (auto st : c->aux) CK(cudaStreamWaitEvent(st, c->ev_fork, 0));
+  for (int q = 0; q < count; ++q) CK(cudaStreamWaitEvent(c->aux[q], c->ev_fork, 0));
 }
 
-// Join the side streams back into `stream`.
-inline void join_side_streams(hhg_ctx* c) {
-  for (int q = 0; q < 4; ++q) {
+// Join them back into `stream`.
+inline void join_side_streams(hhg_ctx* c, int count) {
+  for (int q = 0; q < count; ++q) {
     CK(cudaEventRecord(c->ev_join[q], c->aux[q]));
     CK(cudaStreamWaitEvent(c->stream, c->ev_join[q], 0));
   }
 }
 
-// One operator sweep on a level.  The macro-interior launches (one per macro) alternate
-// between `stream` and aux[1] so that the tail of one overlaps the next, and the skeleton
-// kernels run concurrently on aux[0] (they write disjoint entries and their own partial-sum
-// slots); both side streams are joined back into `stream`.  With profiling on, the
-// interior span (fork to join of the interior launches) and the skeleton span are timed.
 // The stored stencil blocks of a level in precision T (STORED variant), computed on the stream
 // when the coefficient or the problem changed since they were last computed.
 template <typename T>
@@ -485,6 +482,10 @@ inline OpFlags sweep_flags(hhg_ctx* c, const LevelHost& L, bool pairs) {
   OpFlags f = c->flags;
   f.batch = 0;
   if (f.stored || f.nodal || f.tile || c->interior_kernel == 2) return f;
+  if (c->interior_kernel == 0) {
+    f.whole = 1;
+    return f;
+  }
   if (c->interior_kernel == 3) {
     f.batch = 1;
     return f;
@@ -496,6 +497,13 @@ inline OpFlags sweep_flags(hhg_ctx* c, const LevelHost& L, bool pairs) {
   return f;
 }
 
+// One operator sweep on a level.  By default one launch (k_sweep).  Else (the nodal and stored
+// variants, interior kernels chosen by hand) the macro-interior
+// rows on `stream` (all macros in one launch, or one launch per macro, every second one on aux[1]
+// so that the tail of one overlaps the next), the skeleton and Dirichlet rows beside them on
+// aux[0] (they write disjoint entries and their own partial-sum slots); the side streams are
+// joined back into `stream`.  With profiling on, the span of the launch with the interiors and, where
+// it is a launch of its own, the skeleton span are timed.
 template <typename T>
 void sweep(hhg_ctx* c, int level, OpKind op, SweepArgs<T> a, double* norm2) {
   LevelHost& L = c->lv(level);
@@ -503,58 +511,60 @@ void sweep(hhg_ctx* c, int level, OpKind op, SweepArgs<T> a, double* norm2) {
   if (c->flags.stored) a.stencil = stored_stencil<T>(c, L);
   if (std::is_same<T, float>::value && c->coeff_bf16) a.k16 = L.d_k16.as<uint16_t>();
   if (norm2) a.partial = c->scratch.as<double>();
-  if (!c->aux[0]) {
-    for (auto& st : c->aux) CK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
-    CK(cudaEventCreateWithFlags(&c->ev_fork, cudaEventDisableTiming));
-    for (auto& e : c->ev_join) CK(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-  }
-  std::array<cudaEvent_t, 2> pi{}, ps{};
-  if (c->prof) {
-    pi = {c->take_event(), c->take_event()};
-    ps = {c->take_event(), c->take_event()};
-    CK(cudaEventRecord(pi[0], c->stream));
-  }
-  CK(cudaEventRecord(c->ev_fork, c->stream));
-  for (auto st : c->aux) CK(cudaStreamWaitEvent(st, c->ev_fork, 0));
-  // interior: all macros in one launch, or macro m on stream (m even) or aux[1] (m odd); partial
-  // slots in macro order
+  int64_t np = 0;
   const OpFlags fl = sweep_flags(c, L, std::is_same<T, float>::value);
-  int64_t used = 0;
-  if (fl.batch) {
-    CK(launch_sweep_batched<T>(L.dev, consts_dev<T>(L), op, fl, a, c->stream, 0, &used));
+  if (fl.whole) {
+    std::array<cudaEvent_t, 2> pi{};
+    if (c->prof) {
+      pi = {c->take_event(), c->take_event()};
+      CK(cudaEventRecord(pi[0], c->stream));
+    }
+    CK(launch_sweep<T>(L.dev, consts_dev<T>(L), op, fl, a, c->stream, &np));
+    if (c->prof) {
+      CK(cudaEventRecord(pi[1], c->stream));
+      c->prof_ev[0].push_back(pi);
+      c->prof_launches[0] += 1;
+    }
   } else {
-    for (int m = 0; m < L.dev.nmacro; ++m) {
-      int64_t cnt = 0;
-      CK(launch_sweep_macro<T>(L.dev, stencils<T>(L), nodal_consts<T>(L), m, op, c->flags, a,
-                               m % 2 ? c->aux[1] : c->stream, used, &cnt));
-      used += cnt;
+    const int sides = fl.batch || L.dev.nmacro < 2 ? 1 : 2;
+    std::array<cudaEvent_t, 2> pi{}, ps{};
+    if (c->prof) {
+      pi = {c->take_event(), c->take_event()};
+      ps = {c->take_event(), c->take_event()};
+      CK(cudaEventRecord(pi[0], c->stream));
     }
-  }
-  if (c->prof) {
-    CK(cudaEventRecord(c->ev_join[1], c->aux[1]));
-    CK(cudaStreamWaitEvent(c->stream, c->ev_join[1], 0));
-    CK(cudaEventRecord(pi[1], c->stream));
-    CK(cudaEventRecord(ps[0], c->aux[0]));
-  }
-  int64_t used_sk = 0;
-  CK(launch_sweep<T>(L.dev, stencils<T>(L), consts_dev<T>(L), op, c->flags, a, c->aux[0], 2, used, &used_sk,
-                     c->aux[2], c->aux[3]));
-  if (c->prof) {
-    for (int q = 2; q < 4; ++q) {  // the skeleton span ends when all three skeleton streams have
-      CK(cudaEventRecord(c->ev_join[q], c->aux[q]));
-      CK(cudaStreamWaitEvent(c->aux[0], c->ev_join[q], 0));
+    fork_side_streams(c, sides);
+    // the skeleton rows first: they are few and latency-bound, and fill in beside the interior
+    int64_t used = 0;
+    if (c->prof) CK(cudaEventRecord(ps[0], c->aux[0]));
+    CK(launch_rows<T>(L.dev, consts_dev<T>(L), op, c->flags, a, c->aux[0], 0, &used));
+    if (c->prof) CK(cudaEventRecord(ps[1], c->aux[0]));
+    // interior partial slots after them, in macro order
+    if (fl.batch) {
+      CK(launch_sweep_batched<T>(L.dev, consts_dev<T>(L), op, fl, a, c->stream, used, &np));
+      used += np;
+    } else {
+      for (int m = 0; m < L.dev.nmacro; ++m) {
+        int64_t cnt = 0;
+        CK(launch_sweep_macro<T>(L.dev, stencils<T>(L), nodal_consts<T>(L), m, op, c->flags, a,
+                                 m % 2 ? c->aux[1] : c->stream, used, &cnt));
+        used += cnt;
+      }
     }
-    CK(cudaEventRecord(ps[1], c->aux[0]));
-    c->prof_ev[0].push_back(pi);
-    c->prof_ev[1].push_back(ps);
-    c->prof_launches[0] += L.dev.ntiles_lin > 0 ? (fl.batch ? (L.dev.nmacro + 65534) / 65535 : L.dev.nmacro) : 0;
-    c->prof_launches[1] += (L.dev.nface_nodes > 0) + (L.dev.nev > 0) + (L.dev.ndir > 0);
+    if (c->prof) {
+      if (sides == 2) {
+        CK(cudaEventRecord(c->ev_join[1], c->aux[1]));
+        CK(cudaStreamWaitEvent(c->stream, c->ev_join[1], 0));
+      }
+      CK(cudaEventRecord(pi[1], c->stream));
+      c->prof_ev[0].push_back(pi);
+      c->prof_ev[1].push_back(ps);
+      c->prof_launches[0] += L.dev.ntiles_lin > 0 ? (fl.batch ? (L.dev.nmacro + 65534) / 65535 : L.dev.nmacro) : 0;
+      c->prof_launches[1] += 1;
+    }
+    join_side_streams(c, sides);
+    np = used;
   }
-  for (int q = 0; q < 4; ++q) {
-    CK(cudaEventRecord(c->ev_join[q], c->aux[q]));
-    CK(cudaStreamWaitEvent(c->stream, c->ev_join[q], 0));
-  }
-  const int64_t np = used + used_sk;
   if (norm2) {
     CK(launch_reduce(c->scratch.as<double>(), np, c->scalar.as<double>(), c->stream));
     CK(cudaMemcpyAsync(c->pinned, c->scalar.p, sizeof(double), cudaMemcpyDeviceToHost, c->stream));

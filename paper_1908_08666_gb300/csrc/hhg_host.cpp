@@ -229,6 +229,33 @@ void macro_constants(const MacroGeom& G, int n, double c_eps, double c_div, Macr
           }
       }
     }
+    // the elements of the edge in cyclic order of its ring
+    {
+      for (int e = 0; e < 6; ++e)
+        for (int q = 0; q < 16; ++q) out.el[d][e][q] = 0;
+      for (const PatchEl& e : patch) {
+        int P[4][3], other[2], no = 0;
+        kuhn_vertices(e.p, P);
+        for (int v = 0; v < 4; ++v) {
+          if (v == e.a || v == e.b) continue;
+          const int off[3] = {e.c[0] + P[v][0], e.c[1] + P[v][1], e.c[2] + P[v][2]};
+          other[no++] = node_of(off);
+        }
+        int at = -1;
+        for (int q = 0; q < count; ++q)
+          if ((ring_cyc(d, q) == other[0] && ring_cyc(d, q + 1) == other[1]) ||
+              (ring_cyc(d, q) == other[1] && ring_cyc(d, q + 1) == other[0]))
+            at = q;
+        if (at < 0) THROW(HHG_ERR_STATE, "element outside the ring of direction %d", d);
+        double* el = out.el[d][at];
+        for (int q = 0; q < 9; ++q) el[q] = KE[e.p][e.a][e.b][q];
+        for (int l = 0; l < 3; ++l) {
+          el[9 + l] = BD[e.p][e.a][e.b][l];
+          el[12 + l] = BD[e.p][e.b][e.a][l];
+        }
+        el[15] = LC[e.p][e.a][e.b];
+      }
+    }
     // checks: Shat symmetric, khat weights, ring structure, pair antisymmetry
     for (int m = 0; m < 3; ++m)
       for (int l = 0; l < 3; ++l) {
@@ -287,7 +314,39 @@ void macro_constants(const MacroGeom& G, int n, double c_eps, double c_div, Macr
         if (std::fabs(S[r] - want[r]) > 1e-12 * (1 + std::fabs(want[r])))
           THROW(HHG_ERR_STATE, "Shat(-d) != Shat(d) for direction %d", d);
     }
+    if (d < 7) {
+      // axial vector of the ring pair (cyc[q], cyc[q + nr]), and its dependency on a red edge
+      const int nr = dir_red(d) ? 3 : 2;
+      auto axial = [&](int q, int r) {
+        for (int c = 0; c < ring_count(d); ++c) {
+          if (ring_a(d, c) == ring_cyc(d, q)) return out.st.s[d][c][r];
+          if (ring_b(d, c) == ring_cyc(d, q)) return -out.st.s[d][c][r];
+        }
+        THROW(HHG_ERR_STATE, "ring pair of direction %d not found", d);
+      };
+      for (int r = 0; r < 6; ++r) out.mar[d][r] = out.st.S[d][r];
+      for (int r = 0; r < 3; ++r) {
+        out.mar[d][6 + r] = axial(0, r);
+        out.mar[d][9 + r] = axial(nr - 1, r);
+        if (nr == 3 && std::fabs(axial(1, r) - axial(0, r) - axial(2, r)) > 1e-10 * (cmax + 1e-300))
+          THROW(HHG_ERR_STATE, "correction stencils of direction %d are not dependent", d);
+        out.mar[d][12 + r] = out.st.B[d][r];
+        out.mar[d][15 + r] = out.st.G[d][r];
+      }
+      out.mar[d][18] = out.st.C[d];
+      out.mar[d][19] = 0;
+    }
+    for (int r = 0; r < 6; ++r) out.sc[d][r] = out.st.S[d < 7 ? d : d - 7][r];
+    for (int r = 0; r < 9; ++r) out.sc[d][6 + r] = out.st.s[d][r / 3][r % 3];
+    out.sc[d][15] = 0;
+    for (int l = 0; l < 3; ++l) {
+      out.sb[d][l] = out.st.B[d][l];
+      out.sb[d][3 + l] = out.st.G[d][l];
+    }
+    out.sb[d][6] = out.st.C[d];
+    out.sb[d][7] = 0;
   }
+  out.pad[0] = out.pad[1] = 0;
 }
 
 // the centre terms of B, B^T and C at a macro-interior node, from the 24 elements around it
@@ -325,6 +384,98 @@ MacroConsts<T> cast_consts(const MacroConsts<double>& c) {
 
 
 
+// Lanes, warps and face blocks of the skeleton rows (LevelDev).  Nodes on macro edges and vertices:
+// the incidences of a node take a power of two of lanes, spread over the warp (lane = incidence *
+// nodes per warp + node), more than 32 of them several rounds.  Nodes are ordered by how many lanes they take (most first, they run
+// longest), then by macros and the faces or edges they lie on, so that the lanes of a warp read
+// the same constants and neighbouring points.
+void build_rows(LevelHost& L) {
+  const int n = L.n;
+  const int64_t nskel = (int64_t)L.skel_dir.size();
+  auto primitive = [&](const SkelInc& I) {
+    return (I.i + I.j + I.k == n ? 1 : 0) | (I.i == 0 ? 2 : 0) | (I.j == 0 ? 4 : 0) | (I.k == 0 ? 8 : 0);
+  };
+  struct Key {
+    int32_t rounds, lg, near, m0, p0, m1, p1;
+    int64_t s;
+    bool operator<(const Key& o) const {
+      return std::make_tuple(-rounds, -lg, -near, m0, p0, m1, p1, s) <
+             std::make_tuple(-o.rounds, -o.lg, -o.near, o.m0, o.p0, o.m1, o.p1, o.s);
+    }
+  };
+  for (int stk = 0; stk < 2; ++stk) {
+    std::vector<RowLane>& lanes = L.row_lanes[stk];
+    std::vector<int32_t>& warps = L.row_warps[stk];
+    std::vector<Key> keys, faces;
+    for (int64_t s = 0; s < nskel; ++s) {
+      if (L.skel_dir[s] && !stk) continue;
+      const int b0 = L.skel_ptr[s], ni = L.skel_ptr[s + 1] - b0;
+      Key q{(ni + 31) / 32, 0, 0, L.skel_inc[b0].macro, primitive(L.skel_inc[b0]), -1, 0, s};
+      while ((1 << q.lg) < std::min(ni, 32)) ++q.lg;
+      if (ni > 1) {
+        q.m1 = L.skel_inc[b0 + 1].macro;
+        q.p1 = primitive(L.skel_inc[b0 + 1]);
+      }
+      if (q.rounds > 255) THROW(HHG_ERR_UNSUPPORTED, "a node lies in %d macros (at most %d)", ni, 255 * 32);
+      // next to a face's edges one of the three non-zero barycentric weights is 1
+      const SkelInc& I = L.skel_inc[b0];
+      if (L.skel_support[s] == 3)
+        for (const int w : {n - I.i - I.j - I.k, (int)I.i, (int)I.j, (int)I.k}) q.near |= w == 1;
+      (L.skel_support[s] == 3 ? faces : keys).push_back(q);
+    }
+    std::sort(keys.begin(), keys.end());
+    std::sort(faces.begin(), faces.end());
+    for (size_t q0 = 0; q0 < faces.size();) {
+      const Key& K = faces[q0];
+      size_t q1 = q0;
+      while (q1 < faces.size() && q1 - q0 < 32 && faces[q1].lg == K.lg && faces[q1].near == K.near && faces[q1].m0 == K.m0 && faces[q1].p0 == K.p0 &&
+             faces[q1].m1 == K.m1 && faces[q1].p1 == K.p1)
+        ++q1;
+      auto face_of = [](int p) { return p == 1 ? 0 : p == 2 ? 1 : p == 4 ? 2 : 3; };
+      FaceBlock F{{K.m0, K.m1}, {(int16_t)face_of(K.p0), (int16_t)face_of(K.p1)}, (int16_t)(q1 - q0), L.skel_dir[K.s], (int16_t)K.near, 0};
+      L.face_blocks[stk].push_back(F);
+      for (int side = 0; side < 2; ++side)
+        for (int lane = 0; lane < 32; ++lane) {
+          FacePoint P{0, 0, 0, 0};
+          if (q0 + lane < q1 && (side == 0 || K.m1 >= 0)) {
+            const SkelInc& I = L.skel_inc[L.skel_ptr[faces[q0 + lane].s] + side];
+            P = FacePoint{I.i, I.j, I.k, 0};
+          }
+          L.face_points[stk].push_back(P);
+        }
+      q0 = q1;
+    }
+    for (size_t q0 = 0; q0 < keys.size();) {
+      const Key& K = keys[q0];
+      const int per = 32 >> K.lg;
+      size_t q1 = q0;
+      while (q1 < keys.size() && q1 - q0 < (size_t)per && keys[q1].lg == K.lg && keys[q1].rounds == K.rounds) ++q1;
+      warps.push_back((int32_t)(lanes.size() / 32));
+      const uint16_t common = (uint16_t)(K.lg | (K.rounds << ROW_ROUNDS_SHIFT));
+      for (int r = 0; r < K.rounds; ++r)
+        for (int lane = 0; lane < 32; ++lane) {
+          const size_t q = q0 + lane % per;
+          const int inc = 32 * r + lane / per;
+          RowLane R{-1, 0, 0, 0, common};
+          if (q < q1) {
+            const int64_t s = keys[q].s;
+            if (L.skel_ptr[s] + inc < L.skel_ptr[s + 1]) {
+              const SkelInc& I = L.skel_inc[L.skel_ptr[s] + inc];
+              R.macro = I.macro;
+              R.i = I.i;
+              R.j = I.j;
+              R.k = I.k;
+              if (L.skel_dir[s]) R.flags |= ROW_VDIR;
+              if (inc == 0) R.flags |= ROW_FIRST;
+            }
+          }
+          lanes.push_back(R);
+        }
+      q0 = q1;
+    }
+  }
+}
+
 void build_level(hhg_ctx* c, int level) {
   auto L = std::make_unique<LevelHost>();
   const int n = 1 << level;
@@ -346,6 +497,21 @@ void build_level(hhg_ctx* c, int level) {
     const int M = n - 1 - k;
     const int count = M * M / 4;
     for (int start = 0; start < count; start += INTERIOR_BLOCK) L->tiles_pair.push_back((k << 20) | start);
+  }
+  // columns of the marching kernel
+  {
+    const int64_t points = (int64_t)M * (n >= 4 ? tetnum(n - 3) : 0);
+    // length: the longer, the less the loads before a column's first point weigh (44 of 28 per
+    // point), but the fewer columns there are; about 3.5 columns per thread that fits the GPU (152
+    // SMs x 512) leave no large last wave.  FP32 apply on 129^3 / 257^3 nodes: length 4 61 / 432
+    // us, 8 61 / 405, 16 67 / 391; FP64 residual on 129^3: 4 1.76 ms, 8 1.83; V-cycle: at least 2
+    // on its coarse levels (1.01 ms; 1: 1.02, 4: 1.03)
+    int len = 2;
+    while (len < 16 && 2 * points > 7 * (2 * len) * (int64_t)152 * 512) len *= 2;
+    L->column_len = len;
+    for (int cc = 2; cc <= n - 2; ++cc)
+      for (int k0 = 1; k0 <= cc - 1; k0 += len)
+        for (int i = 1; i <= n - 1 - cc; ++i) L->columns.push_back((cc << 20) | (k0 << 10) | i);
   }
   // boxes of TILE3_I x TILE3_J x TILE3_K lattice points (i, j, k) with at least one
   // macro-interior point, for the shared-memory tile kernel
@@ -502,104 +668,14 @@ void build_level(hhg_ctx* c, int level) {
     L->lumped.resize(L->entries);
     for (int64_t e = 0; e < L->entries; ++e) L->lumped[e] = mu[L->entry_to_unique[e]];
   }
-  // skeleton split for the kernels: free face-interior nodes, free edge/vertex nodes and
-  // Dirichlet nodes; and the same face/edge-vertex split including Dirichlet nodes
-  auto add_face = [&](int64_t s, std::vector<int32_t>& nodes, std::vector<FaceItem>& items) {
-    const int32_t fid = (int32_t)nodes.size();
-    nodes.push_back((int32_t)s);
-    for (int q = L->skel_ptr[s]; q < L->skel_ptr[s + 1]; ++q) {
-      const SkelInc& I = L->skel_inc[q];
-      const int w[4] = {n - I.i - I.j - I.k, I.i, I.j, I.k};
-      int f = -1, zeros = 0;
-      for (int cc = 0; cc < 4; ++cc)
-        if (w[cc] == 0) {
-          f = cc;
-          ++zeros;
-        }
-      if (zeros != 1) THROW(HHG_ERR_STATE, "face node with %d zero barycentric weights", zeros);
-      FaceItem it;
-      it.macro = I.macro;
-      it.node = fid;
-      it.i = I.i;
-      it.j = I.j;
-      it.k = I.k;
-      it.f = (int16_t)f;
-      items.push_back(it);
-    }
-  };
-  std::vector<int64_t> free_face;
   for (int64_t s = 0; s < nskel; ++s) {
-    if (L->skel_dir[s])
-      L->dir_nodes.push_back((int32_t)s);
-    else if (L->skel_support[s] == 3)
-      free_face.push_back(s);
-    else
-      L->ev_nodes.push_back((int32_t)s);
-    if (L->skel_support[s] == 3)
-      add_face(s, L->face_nodes_all, L->face_items_all);
-    else
-      L->ev_all.push_back((int32_t)s);
-  }
-  // free face nodes ordered by their incidences (macro and face type of each), so that the
-  // lanes of a warp of the face-row kernel take the same face types
-  {
-    auto face_type = [&](const SkelInc& I) {
-      return (I.i + I.j + I.k == n) ? 0 : (I.i == 0) ? 1 : (I.j == 0) ? 2 : 3;
-    };
-    auto key = [&](int64_t s) {
-      std::array<int64_t, 5> kk{};
-      const int b0 = L->skel_ptr[s], b1 = L->skel_ptr[s + 1];
-      for (int q = 0; q < 2; ++q) {
-        if (b0 + q < b1) {
-          kk[2 * q] = L->skel_inc[b0 + q].macro;
-          kk[2 * q + 1] = face_type(L->skel_inc[b0 + q]);
-        } else {
-          kk[2 * q] = -1;
-        }
-      }
-      kk[4] = s;
-      return kk;
-    };
-    std::sort(free_face.begin(), free_face.end(), [&](int64_t a, int64_t b) { return key(a) < key(b); });
-    for (int64_t s : free_face) add_face(s, L->face_nodes, L->face_items);
-  }
-  // group the face items by macro and face type so that the lanes of a warp share the
-  // candidate set (the unrolled candidate loop then does not diverge)
-  auto item_order = [](const FaceItem& a, const FaceItem& b) {
-    if (a.macro != b.macro) return a.macro < b.macro;
-    if (a.f != b.f) return a.f < b.f;
-    if (a.k != b.k) return a.k < b.k;
-    if (a.j != b.j) return a.j < b.j;
-    return a.i < b.i;
-  };
-  std::stable_sort(L->face_items.begin(), L->face_items.end(), item_order);
-  std::stable_sort(L->face_items_all.begin(), L->face_items_all.end(), item_order);
-  // candidate elements around a face-interior point that lie inside the macro (per face
-  // type); checked against every face item of this level
-  auto cand_inside = [](int nn, int i, int j, int k, int bit) {
-    const int p = bit >> 2, av = bit & 3;
-    int P[4][3];
-    kuhn_vertices(p, P);
-    const int X = i + j + k, Y = j + k, Z = k;
-    for (int v = 0; v < 4; ++v) {
-      const int VX = X - P[av][0] + P[v][0], VY = Y - P[av][1] + P[v][1], VZ = Z - P[av][2] + P[v][2];
-      if (!(0 <= VZ && VZ <= VY && VY <= VX && VX <= nn)) return false;
+    if (L->skel_dir[s]) {
+      for (int q = L->skel_ptr[s]; q < L->skel_ptr[s + 1]; ++q) L->dir_entries.push_back(L->skel_entries[q]);
+    } else {
+      ++(L->skel_support[s] == 3 ? L->nface_nodes : L->nev);
     }
-    return true;
-  };
-  {
-    const int nn = 16;
-    const int rep[4][3] = {{5, 5, 6}, {0, 5, 5}, {5, 0, 5}, {5, 5, 0}};
-    for (int f = 0; f < 4; ++f) {
-      L->face_mask[f] = 0;
-      for (int bit = 0; bit < 24; ++bit)
-        if (cand_inside(nn, rep[f][0], rep[f][1], rep[f][2], bit)) L->face_mask[f] |= 1u << bit;
-    }
-    for (const FaceItem& it : L->face_items_all)
-      for (int bit = 0; bit < 24; ++bit)
-        if (cand_inside(n, it.i, it.j, it.k, bit) != (((L->face_mask[it.f] >> bit) & 1u) != 0))
-          THROW(HHG_ERR_STATE, "face candidate mask mismatch");
   }
+  build_rows(*L);
   for (int64_t e = 0; e < L->entries; ++e)
     if (L->entry_to_unique[e] < 0) THROW(HHG_ERR_STATE, "entry without node");
   c->levels[level] = std::move(L);
@@ -643,6 +719,7 @@ void upload_level(hhg_ctx* c, LevelHost& L) {
   upload(L.d_tiles_int, L.tiles_int);
   upload(L.d_tiles_all, L.tiles_all);
   upload(L.d_tiles_lin, L.tiles_lin);
+  upload(L.d_columns, L.columns);
   upload(L.d_tiles_pair, L.tiles_pair);
   upload(L.d_tiles3, L.tiles3);
   upload(L.d_gs_chunks, L.gs_chunks);
@@ -665,17 +742,13 @@ void upload_level(hhg_ctx* c, LevelHost& L) {
     upload(L.d_mass64, L.lumped);
     upload(L.d_mass32, m32);
   }
-  upload(L.d_face_items, L.face_items);
-  upload(L.d_face_items_all, L.face_items_all);
-  upload(L.d_face_nodes_all, L.face_nodes_all);
-  upload(L.d_ev_all, L.ev_all);
-  upload(L.d_face_nodes, L.face_nodes);
-  upload(L.d_ev_nodes, L.ev_nodes);
-  upload(L.d_dir_nodes, L.dir_nodes);
-  CK(L.d_acc32.alloc(std::max<size_t>(1, L.face_nodes_all.size()) * 8 * sizeof(float)));
-  CK(L.d_acc64.alloc(std::max<size_t>(1, L.face_nodes_all.size()) * 8 * sizeof(double)));
-  CK(cudaMemset(L.d_acc32.p, 0, L.d_acc32.bytes));
-  CK(cudaMemset(L.d_acc64.p, 0, L.d_acc64.bytes));
+  for (int q = 0; q < 2; ++q) {
+    upload(L.d_row_lanes[q], L.row_lanes[q]);
+    upload(L.d_row_warps[q], L.row_warps[q]);
+    upload(L.d_face_blocks[q], L.face_blocks[q]);
+    upload(L.d_face_points[q], L.face_points[q]);
+  }
+  upload(L.d_dir_entries, L.dir_entries);
   upload(L.d_first, L.unique_first);
   upload(L.d_e2u, L.entry_to_unique);
   if (!L.rptr.empty()) {
@@ -698,6 +771,9 @@ void upload_level(hhg_ctx* c, LevelHost& L) {
   D.tiles_all = L.d_tiles_all.as<int32_t>();
   D.ntiles_lin = (int32_t)L.tiles_lin.size();
   D.tiles_lin = L.d_tiles_lin.as<int32_t>();
+  D.ncolumns = (int32_t)L.columns.size();
+  D.column_len = L.column_len;
+  D.columns = L.d_columns.as<int32_t>();
   D.ntiles_pair = (int32_t)L.tiles_pair.size();
   D.tiles_pair = L.d_tiles_pair.as<int32_t>();
   D.ntiles3 = (int32_t)L.tiles3.size();
@@ -711,23 +787,21 @@ void upload_level(hhg_ctx* c, LevelHost& L) {
   D.skel_inc = L.d_skel_inc.as<SkelInc>();
   D.skel_dir = L.d_skel_dir.as<int8_t>();
   D.mask = L.d_mask.as<uint8_t>();
-  D.nface_items = (int32_t)L.face_items.size();
-  D.nface_nodes = (int32_t)L.face_nodes.size();
-  D.nev = (int32_t)L.ev_nodes.size();
-  D.ndir = (int32_t)L.dir_nodes.size();
-  D.face_items = L.d_face_items.as<FaceItem>();
-  D.face_nodes = L.d_face_nodes.as<int32_t>();
-  D.ev_nodes = L.d_ev_nodes.as<int32_t>();
-  D.dir_nodes = L.d_dir_nodes.as<int32_t>();
-  for (int f = 0; f < 4; ++f) D.face_mask[f] = L.face_mask[f];
-  D.nface_items_all = (int32_t)L.face_items_all.size();
-  D.nface_nodes_all = (int32_t)L.face_nodes_all.size();
-  D.nev_all = (int32_t)L.ev_all.size();
-  D.face_items_all = L.d_face_items_all.as<FaceItem>();
-  D.face_nodes_all = L.d_face_nodes_all.as<int32_t>();
-  D.ev_all = L.d_ev_all.as<int32_t>();
-  D.acc32 = L.d_acc32.as<float>();
-  D.acc64 = L.d_acc64.as<double>();
+  D.nface_nodes = L.nface_nodes;
+  D.nev = L.nev;
+  D.nrow_skel = (int32_t)L.row_warps[0].size();
+  D.row_lanes = L.d_row_lanes[0].as<RowLane>();
+  D.row_warps = L.d_row_warps[0].as<int32_t>();
+  D.nrow_stk = (int32_t)L.row_warps[1].size();
+  D.row_lanes_stk = L.d_row_lanes[1].as<RowLane>();
+  D.row_warps_stk = L.d_row_warps[1].as<int32_t>();
+  for (int q = 0; q < 2; ++q) {
+    D.nface_blocks[q] = (int32_t)L.face_blocks[q].size();
+    D.face_blocks[q] = L.d_face_blocks[q].as<FaceBlock>();
+    D.face_points[q] = L.d_face_points[q].as<FacePoint>();
+  }
+  D.ndir_entries = (int64_t)L.dir_entries.size();
+  D.dir_entries = L.d_dir_entries.as<int64_t>();
 }
 
 }  // namespace

@@ -55,6 +55,17 @@ HHG_HD int ring_b(int d, int c) {
   return d < 7 ? t[d][c] : dir_neg(t[d - 7][c]);
 }
 
+// The ring of the edge (0, d) in cyclic order: consecutive ring nodes are the other two vertices of
+// one of the edge's elements; ring_cyc(d, 6) (red) resp. ring_cyc(d, 4) is ring_cyc(d, 0) again.
+HHG_HD constexpr int ring_cyc(int d, int q) {
+  const int8_t t[NDIR][7] = {{3, 6, 5, 8, 11, 9, 3},      {7, 4, 6, 3, 9, 12, 7},      {10, 8, 5, 6, 4, 7, 10},
+                             {0, 6, 1, 9, 0, 0, 0},       {7, 1, 6, 2, 7, 7, 7},       {0, 6, 2, 8, 0, 0, 0},
+                             {0, 3, 1, 4, 2, 5, 0},       {1, 4, 2, 10, 13, 12, 1},    {10, 2, 5, 0, 11, 13, 10},
+                             {13, 11, 0, 3, 1, 12, 13},   {8, 2, 7, 13, 8, 8, 8},      {13, 9, 0, 8, 13, 13, 13},
+                             {9, 1, 7, 13, 9, 9, 9},      {11, 9, 12, 7, 10, 8, 11}};
+  return t[d][q];
+}
+
 // direction index of the corner offset (di, dj, dk), -1 if it is not a stencil direction
 HHG_HD int dir_of_offset(int di, int dj, int dk) {
   int r = -1;
@@ -155,13 +166,25 @@ struct NodalConsts {
   T ke[6][4][4][9];
 };
 
+// el[d][e]: element e of the edge (0, d), the one whose other two vertices are the ring nodes e and
+// e + 1 of the edge in cyclic order (ring_cyc), as seen by the row of point 0: the 3x3 block
+// (test vertex 0, trial vertex d), then bd(0, d), bd(d, 0) and lc(0, d).
 template <typename T>
-struct MacroConsts {
+struct alignas(16) MacroConsts {
+  T el[NDIR][6][16];
+  T sc[NDIR][16];  // the scaled block of direction d: S (6 values) and s (3 x 3) of the interior stencil
+  T sb[NDIR][8];   // its Stokes blocks: B, G (3 values each), C
+  // the marching kernel's constants per direction pair: S, the axial vectors of the ring pairs
+  // (ring_cyc 0 and 2; 0 and 1 of a four-element edge), B, G, C
+  T mar[7][20];
   MacroStencil<T> st;
   T ke[6][4][4][9];
   T bd[6][4][4][3];
   T lc[6][4][4];
+  T pad[2];  // a whole number of 16-byte words in FP32 as in FP64
 };
+static_assert(sizeof(MacroConsts<float>) % 16 == 0 && sizeof(MacroConsts<double>) == 2 * sizeof(MacroConsts<float>),
+              "el is read in 16-byte words, and both precisions have the same layout");
 
 // one incidence of a skeleton node in a macro
 struct SkelInc {
@@ -170,14 +193,30 @@ struct SkelInc {
   int16_t pad;
 };
 
-// one incidence of a node on a macro face (face-interior node) in a macro;
-// f = which barycentric coordinate vanishes (0: i+j+k = n, 1: i = 0, 2: j = 0, 3: k = 0)
-struct FaceItem {
+// one lane of the edge and vertex rows: an incidence of a node (macro < 0: idle), and what the warp does with it
+struct RowLane {
   int32_t macro;
-  int32_t node;  // index into the face-node list
   int16_t i, j, k;
-  int16_t f;
+  uint16_t flags;
 };
+// A block of 32 nodes in the interior of one macro face, seen from the
+// macros on its sides (the second < 0 on an outer face); face F of the macro: 0 is i + j + k = n,
+// 1 i = 0, 2 j = 0, 3 k = 0.
+struct FaceBlock {
+  int32_t macro[2];
+  int16_t face[2];
+  int16_t count;  // nodes
+  int16_t vdir;   // velocity-Dirichlet nodes (Stokes lists)
+  int16_t near;   // nodes next to the face's edges
+  int16_t pad;
+};
+struct FacePoint {
+  int16_t i, j, k, pad;
+};
+constexpr int ROW_LG = 7;       // log2 of the lanes that share a node (the same in the whole warp)
+constexpr int ROW_VDIR = 8;     // velocity-Dirichlet node (Stokes lists)
+constexpr int ROW_FIRST = 32;   // the node's first incidence (counts in norms)
+constexpr int ROW_ROUNDS_SHIFT = 8;  // rounds of 32 lanes of the warp (the same in the whole warp)
 
 // device view of one level
 struct LevelDev {
@@ -191,6 +230,10 @@ struct LevelDev {
   const int32_t* tiles_lin;
   int32_t ntiles_pair;  // 128-pair chunks of the point pairs of each slice (FP32 sweeps): (k << 20) | start
   const int32_t* tiles_pair;
+  // columns of the marching kernel: (c << 20) | (k0 << 10) | i, the points (i, c - k, k), k = k0 ..
+  // min(k0 + column_len, c) - 1
+  int32_t ncolumns, column_len;
+  const int32_t* columns;
   int32_t ntiles3;      // boxes of the shared-memory tile kernel: (k0 << 20) | (j0 << 10) | i0
   const int32_t* tiles3;
   // hybrid Gauss-Seidel: chunks of up to 32 macro-interior points of one colour along a row,
@@ -207,22 +250,21 @@ struct LevelDev {
   const SkelInc* skel_inc;   // incidences
   const int8_t* skel_dir;    // Dirichlet flag per skeleton node
   const uint8_t* mask;       // [entries] 1 = owned copy of a free node (dot products)
-  // skeleton split: free face-interior nodes (per-incidence items + accumulator),
-  // free edge/vertex nodes (warp kernel), Dirichlet nodes
-  int32_t nface_items, nface_nodes, nev, ndir;
-  const FaceItem* face_items;
-  const int32_t* face_nodes;  // skeleton id of each face node
-  const int32_t* ev_nodes;    // skeleton ids
-  const int32_t* dir_nodes;   // skeleton ids
-  uint32_t face_mask[4];      // candidate elements (bit 4p+av) inside the macro, per face type
-  float* acc32;               // [nface_nodes_all * 8] accumulators, zero between sweeps
-  double* acc64;
-  // the same split including Dirichlet skeleton nodes (the Stokes pressure rows of
-  // velocity-Dirichlet nodes are free)
-  int32_t nface_items_all, nface_nodes_all, nev_all;
-  const FaceItem* face_items_all;
-  const int32_t* face_nodes_all;
-  const int32_t* ev_all;
+  int32_t nface_nodes, nev;  // free nodes in the interior of macro faces; on macro edges and vertices
+  // skeleton rows (hhg_rows.cuh).  Nodes on macro edges and vertices: lanes in units of 32, the first
+  // unit of every warp; _stk: with the velocity-Dirichlet nodes (their pressure rows are free)
+  int32_t nrow_skel, nrow_stk;
+  const RowLane* row_lanes;
+  const int32_t* row_warps;
+  const RowLane* row_lanes_stk;
+  const int32_t* row_warps_stk;
+  // nodes in the interior of macro faces: points of block b from its side q at
+  // face_points[64 b + 32 q ..]; [1]: the Stokes lists
+  int32_t nface_blocks[2];
+  const FaceBlock* face_blocks[2];
+  const FacePoint* face_points[2];
+  int64_t ndir_entries;  // entries of Dirichlet nodes (every copy)
+  const int64_t* dir_entries;
 };
 
 constexpr int INTERIOR_BLOCK = 128;

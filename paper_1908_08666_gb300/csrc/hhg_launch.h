@@ -16,6 +16,7 @@ struct OpFlags {
   int nodal = 0;  // 1: macro-interior rows by nodal integration a_h (the NODAL variant)
   int stored = 0; // 1: macro-interior rows from the stored stencil blocks (the STORED variant)
   int tile = 0;   // 1: macro-interior sweeps by the shared-memory tile kernel (k_interior_tile)
+  int whole = 0;  // 1: the whole sweep in one launch (k_sweep)
   int batch = 0;  // 1: the macro-interior sweeps of all macros in one launch (stencils staged in shared memory)
 };
 
@@ -49,15 +50,25 @@ template <typename T>
 int launch_store_stencil(const LevelDev& L, const MacroStencil<double>* st_host, const OpFlags& fl, const double* k64,
                          T* out, void* stream);
 
-// parts: 1 = macro-interior kernels (one launch per macro), 2 = skeleton kernel, 3 = both.
-// partial_offset: first partial slot used (the interior launches take ntiles_lin slots per
-// macro, then the skeleton kernel one per block); *partial_count returns the slots used.
-// stream_ev / stream_dir (nullable: `stream`): streams of the edge/vertex and Dirichlet
-// skeleton kernels, which write disjoint entries and may run concurrently.
+// The rows of the free skeleton nodes and the Dirichlet rows (k_rows).  partial_offset: first
+// partial slot used; *partial_count returns the slots used, one per block of rows.
 template <typename T>
-int launch_sweep(const LevelDev& L, const MacroStencil<T>* st_host, const MacroConsts<T>* mc_dev, OpKind op,
-                 const OpFlags& fl, const SweepArgs<T>& a, void* stream, int parts, int64_t partial_offset,
-                 int64_t* partial_count, void* stream_ev = nullptr, void* stream_dir = nullptr);
+int launch_rows(const LevelDev& L, const MacroConsts<T>* mc_dev, OpKind op, const OpFlags& fl, const SweepArgs<T>& a,
+                void* stream, int64_t partial_offset, int64_t* partial_count);
+// the Stokes rows (apply or residual) of all skeleton nodes
+template <typename T>
+int launch_rows_stokes(const LevelDev& L, const MacroConsts<T>* mc_dev, OpKind op, const OpFlags& fl,
+                       const SweepArgs<T>& a, void* stream, int64_t partial_offset, int64_t* partial_count);
+
+// A whole sweep (macro interiors, skeleton and Dirichlet rows) of a scaled-stencil variant in one
+// launch (k_sweep); partial slots from 0.
+template <typename T>
+int launch_sweep(const LevelDev& L, const MacroConsts<T>* mc_dev, OpKind op, const OpFlags& fl, const SweepArgs<T>& a,
+                 void* stream, int64_t* partial_count);
+// the same for the Stokes saddle operator (apply or residual)
+template <typename T>
+int launch_sweep_stokes(const LevelDev& L, const MacroConsts<T>* mc_dev, OpKind op, const OpFlags& fl,
+                        const SweepArgs<T>& a, void* stream, int64_t* partial_count);
 
 // The macro-interior sweeps of all macros of the level in one launch (k_interior_pair_batched for
 // FP32, k_interior_batched for FP64; each block stages its macro's stencil from mc_dev in shared
@@ -95,12 +106,17 @@ int launch_gs_colour(const LevelDev& L, const MacroStencil<T>* st_host, const Ma
 template <typename T>
 int launch_copy_entries(int64_t count, const int64_t* idx, int comps, int64_t E, const T* src, T* dst, void* stream);
 
-// constant-memory direction tables of the skeleton kernels (once per device)
+// constant-memory direction tables of the skeleton kernel (once per device)
 int upload_direction_tables();
+// its parts, one for every translation unit with skeleton rows
+int upload_tables_f32();
+int upload_tables_f64();
+int upload_tables_stokes_f32();
+int upload_tables_stokes_f64();
 
 // Stokes saddle operator on (u, v, w, p) vectors (4 components): apply or residual
-// side (nullable): three side streams for the face-node chain, every second macro's
-// interior launch and the edge/vertex nodes (they write disjoint entries).
+// side (nullable): two side streams for the skeleton rows and every second macro's interior launch
+// (they write disjoint entries).
 template <typename T>
 int launch_stokes_sweep(const LevelDev& L, const MacroStencil<T>* st_host, const MacroConsts<T>* mc_dev, OpKind op,
                         const OpFlags& fl, const SweepArgs<T>& a, void* stream, int64_t* partial_count,

@@ -282,7 +282,7 @@ void smooth(hhg_ctx* c, int l, int steps, const T* f, T* x) {
       a.k = kptr<T>(L);
       a.out = oth;
       a.omega = c->mg.omega;
-      CK(launch_sweep<T>(L.dev, stencils<T>(L), consts_dev<T>(L), OP_JACOBI, c->flags, a, c->stream, 2, 0, nullptr));
+      CK(launch_rows<T>(L.dev, consts_dev<T>(L), OP_JACOBI, c->flags, a, c->stream, 0, nullptr));
       CK(launch_copy_entries<T>(L.dev.nskel_entries, L.dev.skel_entries, 3, L.entries, oth, x, c->stream));
       SweepArgs<T> g{};
       g.x = x;
@@ -524,11 +524,16 @@ double stokes_sweep(hhg_ctx* c, int l, OpKind op, const T* f, const T* x, T* out
   a.k = kptr<T>(L);
   if (norm) a.partial = c->scratch.as<double>();
   int64_t np = 0;
-  fork_side_streams(c);
-  void* side[3] = {c->aux[0], c->aux[1], c->aux[2]};
-  CK(launch_stokes_sweep<T>(L.dev, stencils<T>(L), consts_dev<T>(L), op, sweep_flags(c, L, false), a, c->stream, &np,
-                            side));
-  join_side_streams(c);
+  const OpFlags fl = sweep_flags(c, L, false);
+  if (fl.whole) {
+    CK(launch_sweep_stokes<T>(L.dev, consts_dev<T>(L), op, fl, a, c->stream, &np));
+  } else {
+    const int sides = fl.batch ? 1 : 2;
+    fork_side_streams(c, sides);
+    void* side[2] = {c->aux[0], c->aux[1]};
+    CK(launch_stokes_sweep<T>(L.dev, stencils<T>(L), consts_dev<T>(L), op, fl, a, c->stream, &np, side));
+    join_side_streams(c, sides);
+  }
   if (!norm) return 0.0;
   CK(launch_reduce(c->scratch.as<double>(), np, c->scalar.as<double>(), c->stream));
   CK(cudaMemcpyAsync(c->pinned, c->scalar.p, sizeof(double), cudaMemcpyDeviceToHost, c->stream));

@@ -26,63 +26,11 @@
 
 #include "hhg_internal.h"
 #include "hhg_launch.h"
+#include "hhg_row.cuh"
 
 namespace hhg {
 
 namespace {
-
-template <typename T>
-__device__ __forceinline__ void block_sum_store(double v, double* out) {
-  __shared__ double red[32];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-  const int nw = (blockDim.x * blockDim.y + 31) / 32;
-  if ((tid & 31) == 0) red[tid >> 5] = v;
-  __syncthreads();
-  if (tid < 32) {
-    double s = tid < nw ? red[tid] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (tid == 0) *out = s;
-  }
-}
-
-template <typename T, int OP>
-__device__ __forceinline__ void epilogue(const SweepArgs<T>& a, int64_t e, int64_t E, T ax, T ay, T az, T dgx, T dgy,
-                                         T dgz, T x0, T y0, T z0, double& r2) {
-  if (OP == OP_APPLY) {
-    a.out[e] = ax;
-    a.out[e + E] = ay;
-    a.out[e + 2 * E] = az;
-  } else if (OP == OP_DIAG) {
-    a.out[e] = dgx;
-    a.out[e + E] = dgy;
-    a.out[e + 2 * E] = dgz;
-  } else {
-    const T rx = a.f[e] - ax, ry = a.f[e + E] - ay, rz = a.f[e + 2 * E] - az;
-    if (OP == OP_RESID) {
-      a.out[e] = rx;
-      a.out[e + E] = ry;
-      a.out[e + 2 * E] = rz;
-      r2 += (double)rx * rx + (double)ry * ry + (double)rz * rz;
-    } else if (OP == OP_JACOBI) {
-      const T om = (T)a.omega;
-      a.out[e] = x0 + om * rx / dgx;
-      a.out[e + E] = y0 + om * ry / dgy;
-      a.out[e + 2 * E] = z0 + om * rz / dgz;
-    } else if (OP == OP_CHEBY) {
-      const T r1 = (T)a.rho1, r2c = (T)a.rho2;
-      const T ux = (a.d ? r1 * a.d[e] : (T)0) + r2c * rx / dgx;
-      const T uy = (a.d ? r1 * a.d[e + E] : (T)0) + r2c * ry / dgy;
-      const T uz = (a.d ? r1 * a.d[e + 2 * E] : (T)0) + r2c * rz / dgz;
-      a.dout[e] = ux;
-      a.dout[e + E] = uy;
-      a.dout[e + 2 * E] = uz;
-      a.out[e] = x0 + ux;
-      a.out[e + E] = y0 + uy;
-      a.out[e + 2 * E] = z0 + uz;
-    }
-  }
-}
 
 // (j, i) of the t-th interior point of a slice with M = n-1-k: rows j = 1..M-1 hold
 // M-j points; C(j) = (j-1)(2M-j)/2 points precede row j.
@@ -235,27 +183,6 @@ __device__ __forceinline__ void interior_row(const MacroStencil<C>& st, const Op
       dgy = fma(nks, S[1], dgy);
       dgz = fma(nks, S[2], dgz);
     }
-  }
-}
-
-// Stokes epilogue (apply / residual) for one copy: velocity rows (identity on
-// velocity-Dirichlet nodes) and the pressure row.
-template <typename T, int OP>
-__device__ __forceinline__ void stokes_epilogue(const SweepArgs<T>& a, int64_t e, int64_t E, T ax, T ay, T az, T yp,
-                                                T x0, T y0, T z0, bool vdir, double& r2) {
-  if (OP == OP_APPLY) {
-    a.out[e] = vdir ? x0 : ax;
-    a.out[e + E] = vdir ? y0 : ay;
-    a.out[e + 2 * E] = vdir ? z0 : az;
-    a.out[e + 3 * E] = yp;
-  } else {
-    const T rx = vdir ? (T)0 : a.f[e] - ax, ry = vdir ? (T)0 : a.f[e + E] - ay, rz = vdir ? (T)0 : a.f[e + 2 * E] - az;
-    const T rp = a.f[e + 3 * E] - yp;
-    a.out[e] = rx;
-    a.out[e + E] = ry;
-    a.out[e + 2 * E] = rz;
-    a.out[e + 3 * E] = rp;
-    r2 += (double)rx * rx + (double)ry * ry + (double)rz * rz + (double)rp * rp;
   }
 }
 
@@ -967,652 +894,6 @@ __global__ void __launch_bounds__(INTERIOR_BLOCK) k_interior_stored(const LevelD
   if (OP == OP_RESID && a.partial != nullptr) block_sum_store<T>(r2, a.partial + blockIdx.x);
 }
 
-// Kuhn coordinates of corner (i, j, k): X = i+j+k, Y = j+k, Z = k.
-__device__ __forceinline__ bool kuhn_inside(int n, int X, int Y, int Z) {
-  return 0 <= Z && Z <= Y && Y <= X && X <= n;
-}
-__device__ __forceinline__ bool kuhn_interior(int n, int X, int Y, int Z) {
-  return 1 <= Z && Z < Y && Y < X && X <= n - 1;
-}
-
-// Contribution of one incident macro to the row of a skeleton node at corner
-// (i, j, k) of that macro: a_h terms over the candidate elements `cand` (bit
-// 4p+av: Kuhn permutation p, node at vertex av) for partner vertices on the
-// skeleton (every partner with the practical rule), and the scaled blocks of
-// the directions that end at a macro-interior node (symmetric rule).
-// Candidates bit in [B0, B1) and directions in [D0, D1) only (a part of the row).
-template <typename T, int B0 = 0, int B1 = 24, int D0 = 0, int D1 = NDIR>
-__device__ __forceinline__ void incidence_row(const MacroConsts<T>& C, const T* __restrict__ px,
-                                              const T* __restrict__ pk, int64_t E, int n, int i, int j, int k,
-                                              uint32_t cand, uint32_t dirs, T x0, T y0, T z0, const OpFlags& fl,
-                                              T& ax, T& ay, T& az, T& dgx, T& dgy, T& dgz) {
-  const int X = i + j + k, Y = j + k, Z = k;
-  int nb[NDIR];
-  lattice_neighbours(n, i, j, k, nb);
-  const int c0 = lattice_index32(n, i, j, k);
-  // fully unrolled over the 24 candidates so that permutation, vertex offsets, the
-  // neighbour direction of every vertex and stiffness offsets are compile-time constants
-#pragma unroll
-  for (int bit = B0; bit < B1; ++bit) {
-    if (!((cand >> bit) & 1u)) continue;
-    const int p = bit >> 2, av = bit & 3;
-    int a0, a1, a2;
-    kuhn_perm(p, a0, a1, a2);
-    int PX[4], PY[4], PZ[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      PX[v] = (v >= 1 && a0 == 0) + (v >= 2 && a1 == 0) + (v >= 3 && a2 == 0);
-      PY[v] = (v >= 1 && a0 == 1) + (v >= 2 && a1 == 1) + (v >= 3 && a2 == 1);
-      PZ[v] = (v >= 1 && a0 == 2) + (v >= 2 && a1 == 2) + (v >= 3 && a2 == 2);
-    }
-    const int cX = X - PX[av], cY = Y - PY[av], cZ = Z - PZ[av];
-    bool ok = true;
-    int idx[4];
-    bool inner[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int VX = cX + PX[v], VY = cY + PY[v], VZ = cZ + PZ[v];
-      ok = ok && kuhn_inside(n, VX, VY, VZ);
-      // Kuhn offset of vertex v from the node, as a corner offset -> stencil direction
-      const int oX = PX[v] - PX[av], oY = PY[v] - PY[av], oZ = PZ[v] - PZ[av];
-      idx[v] = v == av ? c0 : nb[dir_of_offset(oX - oY, oY - oZ, oZ)];
-      inner[v] = kuhn_interior(n, VX, VY, VZ);
-    }
-    if (!ok) continue;
-    const T kb = (T)0.25 * (pk[idx[0]] + pk[idx[1]] + pk[idx[2]] + pk[idx[3]]);
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      if (v == av) continue;
-      if (!fl.practical && inner[v]) continue;
-      const T* K = C.ke[p][av][v];
-      const T ddx = px[idx[v]] - x0, ddy = px[idx[v] + E] - y0, ddz = px[idx[v] + 2 * E] - z0;
-      ax += kb * (K[0] * ddx + K[1] * ddy + K[2] * ddz);
-      ay += kb * (K[3] * ddx + K[4] * ddy + K[5] * ddz);
-      az += kb * (K[6] * ddx + K[7] * ddy + K[8] * ddz);
-      dgx -= kb * K[0];
-      dgy -= kb * K[4];
-      dgz -= kb * K[8];
-    }
-  }
-  if (fl.practical || !dirs) return;
-  const T k0 = pk[c0];
-#pragma unroll
-  for (int d = D0; d < D1; ++d) {
-    if (!((dirs >> d) & 1u)) continue;
-    const int qi = i + dir_di(d), qj = j + dir_dj(d), qk = k + dir_dk(d);
-    if (!lattice_interior(n, qi, qj, qk)) continue;
-    const int qe = nb[d];
-    T rs = 0, wx = 0, wy = 0, wz = 0;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      if (c >= ring_count(d)) continue;
-      const T ka = pk[nb[ring_a(d, c)]];
-      const T kb = pk[nb[ring_b(d, c)]];
-      rs += ka + kb;
-      const T dk = ka - kb;
-      wx += dk * C.st.s[d][c][0];
-      wy += dk * C.st.s[d][c][1];
-      wz += dk * C.st.s[d][c][2];
-    }
-    const T kq = pk[qe];
-    const T kh = fl.khat_edge ? (T)0.5 * (k0 + kq)
-                              : (T)0.25 * (k0 + kq) + (dir_red(d) ? (T)(1.0 / 12.0) : (T)0.125) * rs;
-    const T* S = C.st.S[d < 7 ? d : d - 7];
-    const T ddx = px[qe] - x0, ddy = px[qe + E] - y0, ddz = px[qe + 2 * E] - z0;
-    ax += kh * (S[0] * ddx + S[3] * ddy + S[4] * ddz);
-    ay += kh * (S[3] * ddx + S[1] * ddy + S[5] * ddz);
-    az += kh * (S[4] * ddx + S[5] * ddy + S[2] * ddz);
-    if (fl.physical) {
-      ax += wy * ddz - wz * ddy;
-      ay += wz * ddx - wx * ddz;
-      az += wx * ddy - wy * ddx;
-    }
-    dgx -= kh * S[0];
-    dgy -= kh * S[1];
-    dgz -= kh * S[2];
-  }
-}
-
-__constant__ int c_dir[NDIR][3];
-__constant__ int c_ring[NDIR][3][2];
-__constant__ int c_ring_n[NDIR];
-
-// Lane version of incidence_row for the block kernels: lane l evaluates candidate
-// element l (l < 24) and stencil direction l (l < 14) with run-time indices, so
-// the lanes of a warp run the same element/direction body concurrently.
-template <typename T>
-__device__ __forceinline__ void incidence_lane(const MacroConsts<T>& C, const T* __restrict__ px,
-                                               const T* __restrict__ pk, int64_t E, int n, int i, int j, int k,
-                                               int lane, T x0, T y0, T z0, const OpFlags& fl, T& ax, T& ay, T& az,
-                                               T& dgx, T& dgy, T& dgz) {
-  if (lane < 24) {
-    const int X = i + j + k, Y = j + k, Z = k;
-    const int p = lane >> 2, av = lane & 3;
-    // Kuhn permutation p (lexicographic order 012 021 102 120 201 210)
-    const int a0 = p >> 1;
-    const int lo = a0 == 0 ? 1 : 0, hi = a0 == 2 ? 1 : 2;
-    const int a1 = (p & 1) ? hi : lo, a2 = (p & 1) ? lo : hi;
-    const int oX = (av >= 1 && a0 == 0) + (av >= 2 && a1 == 0) + (av >= 3 && a2 == 0);
-    const int oY = (av >= 1 && a0 == 1) + (av >= 2 && a1 == 1) + (av >= 3 && a2 == 1);
-    const int oZ = (av >= 1 && a0 == 2) + (av >= 2 && a1 == 2) + (av >= 3 && a2 == 2);
-    bool ok = true;
-    int idx[4];
-    bool inner[4];
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int VX = X - oX + (v >= 1 && a0 == 0) + (v >= 2 && a1 == 0) + (v >= 3 && a2 == 0);
-      const int VY = Y - oY + (v >= 1 && a0 == 1) + (v >= 2 && a1 == 1) + (v >= 3 && a2 == 1);
-      const int VZ = Z - oZ + (v >= 1 && a0 == 2) + (v >= 2 && a1 == 2) + (v >= 3 && a2 == 2);
-      ok = ok && kuhn_inside(n, VX, VY, VZ);
-      idx[v] = ok ? lattice_index32(n, VX - VY, VY - VZ, VZ) : 0;
-      inner[v] = kuhn_interior(n, VX, VY, VZ);
-    }
-    if (ok) {
-      const T kb = (T)0.25 * (pk[idx[0]] + pk[idx[1]] + pk[idx[2]] + pk[idx[3]]);
-#pragma unroll
-      for (int v = 0; v < 4; ++v) {
-        if (v == av) continue;
-        if (!fl.practical && inner[v]) continue;
-        const T* K = C.ke[p][av][v];
-        const T ddx = px[idx[v]] - x0, ddy = px[idx[v] + E] - y0, ddz = px[idx[v] + 2 * E] - z0;
-        ax += kb * (K[0] * ddx + K[1] * ddy + K[2] * ddz);
-        ay += kb * (K[3] * ddx + K[4] * ddy + K[5] * ddz);
-        az += kb * (K[6] * ddx + K[7] * ddy + K[8] * ddz);
-        dgx -= kb * K[0];
-        dgy -= kb * K[4];
-        dgz -= kb * K[8];
-      }
-    }
-  }
-  if (fl.practical || lane >= NDIR) return;
-  const int d = lane;
-  const int qi = i + c_dir[d][0], qj = j + c_dir[d][1], qk = k + c_dir[d][2];
-  if (!lattice_interior(n, qi, qj, qk)) return;
-  const T k0 = pk[lattice_index32(n, i, j, k)];
-  const int qe = lattice_index32(n, qi, qj, qk);
-  T rs = 0, wx = 0, wy = 0, wz = 0;
-  for (int c = 0; c < c_ring_n[d]; ++c) {
-    const int ra = c_ring[d][c][0], rb = c_ring[d][c][1];
-    const T ka = pk[lattice_index32(n, i + c_dir[ra][0], j + c_dir[ra][1], k + c_dir[ra][2])];
-    const T kb = pk[lattice_index32(n, i + c_dir[rb][0], j + c_dir[rb][1], k + c_dir[rb][2])];
-    rs += ka + kb;
-    const T dk = ka - kb;
-    wx += dk * C.st.s[d][c][0];
-    wy += dk * C.st.s[d][c][1];
-    wz += dk * C.st.s[d][c][2];
-  }
-  const T kq = pk[qe];
-  const T kh = fl.khat_edge ? (T)0.5 * (k0 + kq)
-                            : (T)0.25 * (k0 + kq) + (c_ring_n[d] == 3 ? (T)(1.0 / 12.0) : (T)0.125) * rs;
-  const T* S = C.st.S[d < 7 ? d : d - 7];
-  const T ddx = px[qe] - x0, ddy = px[qe + E] - y0, ddz = px[qe + 2 * E] - z0;
-  ax += kh * (S[0] * ddx + S[3] * ddy + S[4] * ddz);
-  ay += kh * (S[3] * ddx + S[1] * ddy + S[5] * ddz);
-  az += kh * (S[4] * ddx + S[5] * ddy + S[2] * ddz);
-  if (fl.physical) {
-    ax += wy * ddz - wz * ddy;
-    ay += wz * ddx - wx * ddz;
-    az += wx * ddy - wy * ddx;
-  }
-  dgx -= kh * S[0];
-  dgy -= kh * S[1];
-  dgz -= kh * S[2];
-}
-
-template <typename T>
-__device__ __forceinline__ T* acc_of(const LevelDev& L);
-template <>
-__device__ __forceinline__ float* acc_of<float>(const LevelDev& L) {
-  return L.acc32;
-}
-template <>
-__device__ __forceinline__ double* acc_of<double>(const LevelDev& L) {
-  return L.acc64;
-}
-
-// ---------------------------------------------------------------------------
-// Free face-interior skeleton nodes, one thread per node (k_face_rows).  A node on a macro
-// face has one incidence per macro sharing the face (two on an interior face); in macro T
-// the node sits on face F of T's lattice (F = 0: i + j + k = n, 1: i = 0, 2: j = 0,
-// 3: k = 0), so the elements of T around it, the stencil directions that stay in T and
-// those that can end at a macro-interior node are fixed by F.  face_incidence<F> evaluates
-// T's part of the row with those sets fixed at compile time (the representative
-// face-interior point of each face type, on a lattice with 16 intervals, decides them);
-// only whether a neighbour is macro-interior (next to the face's edges it is not) is
-// decided at run time.  The symmetric interface rule of Sec. 2.2: pairs of skeleton nodes
-// by nodal integration a_h over T's elements, pairs with a macro-interior neighbour by T's
-// scaled block; the practical rule: a_h for every pair.  Rows are in difference form, so
-// the centre block is minus the sum of the off-diagonal blocks.
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ void face_rep(int F, int& i, int& j, int& k) {
-  i = F == 1 ? 0 : 5;
-  j = F == 2 ? 0 : 5;
-  k = F == 3 ? 0 : (F == 0 ? 6 : 5);
-}
-// direction d stays in the macro's closed lattice from a face-interior point of face F
-__device__ __forceinline__ bool face_dir_valid(int F, int d) {
-  int i, j, k;
-  face_rep(F, i, j, k);
-  return lattice_inside(16, i + dir_di(d), j + dir_dj(d), k + dir_dk(d));
-}
-// direction d can end at a macro-interior point
-__device__ __forceinline__ bool face_dir_inward(int F, int d) {
-  int i, j, k;
-  face_rep(F, i, j, k);
-  return lattice_interior(16, i + dir_di(d), j + dir_dj(d), k + dir_dk(d));
-}
-// candidate element (bit 4 p + av: Kuhn permutation p, the point at vertex av) lies in the macro
-__device__ __forceinline__ bool face_cand_inside(int F, int bit) {
-  int i, j, k;
-  face_rep(F, i, j, k);
-  const int p = bit >> 2, av = bit & 3;
-  int a0, a1, a2;
-  kuhn_perm(p, a0, a1, a2);
-  const int X = i + j + k, Y = j + k, Z = k;
-  bool ok = true;
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const int VX = X + ((v >= 1 && a0 == 0) + (v >= 2 && a1 == 0) + (v >= 3 && a2 == 0)) -
-                   ((av >= 1 && a0 == 0) + (av >= 2 && a1 == 0) + (av >= 3 && a2 == 0));
-    const int VY = Y + ((v >= 1 && a0 == 1) + (v >= 2 && a1 == 1) + (v >= 3 && a2 == 1)) -
-                   ((av >= 1 && a0 == 1) + (av >= 2 && a1 == 1) + (av >= 3 && a2 == 1));
-    const int VZ = Z + ((v >= 1 && a0 == 2) + (v >= 2 && a1 == 2) + (v >= 3 && a2 == 2)) -
-                   ((av >= 1 && a0 == 2) + (av >= 2 && a1 == 2) + (av >= 3 && a2 == 2));
-    ok = ok && kuhn_inside(16, VX, VY, VZ);
-  }
-  return ok;
-}
-
-template <typename T, int F, bool DIAG>
-__device__ __forceinline__ void face_incidence(const MacroConsts<T>& C, const T* __restrict__ px,
-                                               const T* __restrict__ pk, int64_t E, int n, int i, int j, int k,
-                                               const OpFlags& fl, T x0, T y0, T z0, T& ax, T& ay, T& az, T& dgx,
-                                               T& dgy, T& dgz) {
-  int nb[NDIR];
-  lattice_neighbours(n, i, j, k, nb);
-  const T k0 = pk[lattice_index32(n, i, j, k)];
-  T kv[NDIR], dx[NDIR], dy[NDIR], dz[NDIR];
-  bool in[NDIR];
-#pragma unroll
-  for (int d = 0; d < NDIR; ++d) {
-    kv[d] = dx[d] = dy[d] = dz[d] = (T)0;
-    in[d] = false;
-    if (face_dir_valid(F, d)) {
-      const int q = nb[d];
-      kv[d] = pk[q];
-      dx[d] = px[q] - x0;
-      dy[d] = px[q + E] - y0;
-      dz[d] = px[q + 2 * E] - z0;
-      in[d] = face_dir_inward(F, d) && lattice_interior(n, i + dir_di(d), j + dir_dj(d), k + dir_dk(d));
-    }
-  }
-  // nodal-integration terms over the macro's elements around the point
-#pragma unroll
-  for (int bit = 0; bit < 24; ++bit) {
-    if (!face_cand_inside(F, bit)) continue;
-    const int p = bit >> 2, av = bit & 3;
-    int a0, a1, a2;
-    kuhn_perm(p, a0, a1, a2);
-    int dv[4];
-    T ks = k0;
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      const int oX = ((v >= 1 && a0 == 0) + (v >= 2 && a1 == 0) + (v >= 3 && a2 == 0)) -
-                     ((av >= 1 && a0 == 0) + (av >= 2 && a1 == 0) + (av >= 3 && a2 == 0));
-      const int oY = ((v >= 1 && a0 == 1) + (v >= 2 && a1 == 1) + (v >= 3 && a2 == 1)) -
-                     ((av >= 1 && a0 == 1) + (av >= 2 && a1 == 1) + (av >= 3 && a2 == 1));
-      const int oZ = ((v >= 1 && a0 == 2) + (v >= 2 && a1 == 2) + (v >= 3 && a2 == 2)) -
-                     ((av >= 1 && a0 == 2) + (av >= 2 && a1 == 2) + (av >= 3 && a2 == 2));
-      dv[v] = v == av ? -1 : dir_of_offset(oX - oY, oY - oZ, oZ);
-      if (v != av) ks += kv[dv[v]];
-    }
-    const T kb = (T)0.25 * ks;
-#pragma unroll
-    for (int v = 0; v < 4; ++v) {
-      if (v == av) continue;
-      const int d = dv[v];
-      if (!fl.practical && in[d]) continue;
-      const T* K = C.ke[p][av][v];
-      ax = fma(kb, fma(K[0], dx[d], fma(K[1], dy[d], K[2] * dz[d])), ax);
-      ay = fma(kb, fma(K[3], dx[d], fma(K[4], dy[d], K[5] * dz[d])), ay);
-      az = fma(kb, fma(K[6], dx[d], fma(K[7], dy[d], K[8] * dz[d])), az);
-      if (DIAG) {
-        dgx = fma(-kb, K[0], dgx);
-        dgy = fma(-kb, K[4], dgy);
-        dgz = fma(-kb, K[8], dgz);
-      }
-    }
-  }
-  if (fl.practical) return;
-  // scaled blocks of the directions that end at a macro-interior point (their ring nodes
-  // are neighbours of that point, so they lie in the macro)
-#pragma unroll
-  for (int d = 0; d < NDIR; ++d) {
-    if (!face_dir_inward(F, d)) continue;
-    if (!in[d]) continue;
-    T rs = 0, wx = 0, wy = 0, wz = 0;
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      if (c >= ring_count(d)) continue;
-      const T ka = kv[ring_a(d, c)], kb = kv[ring_b(d, c)];
-      rs += ka + kb;
-      const T dk = ka - kb;
-      wx = fma(dk, C.st.s[d][c][0], wx);
-      wy = fma(dk, C.st.s[d][c][1], wy);
-      wz = fma(dk, C.st.s[d][c][2], wz);
-    }
-    const T kh = fl.khat_edge ? (T)0.5 * (k0 + kv[d])
-                              : fma((dir_red(d) ? (T)(1.0 / 12.0) : (T)0.125), rs, (T)0.25 * (k0 + kv[d]));
-    const T* S = C.st.S[d < 7 ? d : d - 7];
-    const T vx = kh * dx[d], vy = kh * dy[d], vz = kh * dz[d];
-    ax = fma(S[0], vx, fma(S[3], vy, fma(S[4], vz, ax)));
-    ay = fma(S[3], vx, fma(S[1], vy, fma(S[5], vz, ay)));
-    az = fma(S[4], vx, fma(S[5], vy, fma(S[2], vz, az)));
-    if (fl.physical) {
-      ax = fma(wy, dz[d], fma(-wz, dy[d], ax));
-      ay = fma(wz, dx[d], fma(-wx, dz[d], ay));
-      az = fma(wx, dy[d], fma(-wy, dx[d], az));
-    }
-    if (DIAG) {
-      dgx = fma(-kh, S[0], dgx);
-      dgy = fma(-kh, S[1], dgy);
-      dgz = fma(-kh, S[2], dgz);
-    }
-  }
-}
-
-template <typename T, int OP>
-__global__ void __launch_bounds__(128) k_face_rows(const LevelDev L, const MacroConsts<T>* __restrict__ mc,
-                                                    const OpFlags fl, const SweepArgs<T> a) {
-  constexpr bool DIAG = OP == OP_JACOBI || OP == OP_CHEBY || OP == OP_DIAG;
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  double r2 = 0.0;
-  if (t < L.nface_nodes) {
-    const int n = L.n;
-    const int64_t E = L.entries;
-    const int s = L.face_nodes[t];
-    const int b0 = L.skel_ptr[s], b1 = L.skel_ptr[s + 1];
-    const SkelInc I0 = L.skel_inc[b0];
-    const int64_t e0 = (int64_t)I0.macro * L.nt + lattice_index32(n, I0.i, I0.j, I0.k);
-    const T x0 = a.x[e0], y0 = a.x[e0 + E], z0 = a.x[e0 + 2 * E];
-    T ax = 0, ay = 0, az = 0, dgx = 0, dgy = 0, dgz = 0;
-    for (int q = b0; q < b1; ++q) {
-      const SkelInc I = L.skel_inc[q];
-      const int64_t base = (int64_t)I.macro * L.nt;
-      const T* px = a.x + base;
-      const T* pk = a.k + base;
-      const MacroConsts<T>& C = mc[I.macro];
-      const int f = (I.i + I.j + I.k == n) ? 0 : (I.i == 0) ? 1 : (I.j == 0) ? 2 : 3;
-      switch (f) {
-        case 0: face_incidence<T, 0, DIAG>(C, px, pk, E, n, I.i, I.j, I.k, fl, x0, y0, z0, ax, ay, az, dgx, dgy, dgz); break;
-        case 1: face_incidence<T, 1, DIAG>(C, px, pk, E, n, I.i, I.j, I.k, fl, x0, y0, z0, ax, ay, az, dgx, dgy, dgz); break;
-        case 2: face_incidence<T, 2, DIAG>(C, px, pk, E, n, I.i, I.j, I.k, fl, x0, y0, z0, ax, ay, az, dgx, dgy, dgz); break;
-        default: face_incidence<T, 3, DIAG>(C, px, pk, E, n, I.i, I.j, I.k, fl, x0, y0, z0, ax, ay, az, dgx, dgy, dgz); break;
-      }
-    }
-    for (int q = b0; q < b1; ++q) {
-      const SkelInc I = L.skel_inc[q];
-      const int64_t e = (int64_t)I.macro * L.nt + lattice_index32(n, I.i, I.j, I.k);
-      double tmp = 0.0;
-      epilogue<T, OP>(a, e, E, ax, ay, az, dgx, dgy, dgz, x0, y0, z0, tmp);
-      if (q == b0) r2 = tmp;
-    }
-  }
-  if (OP == OP_RESID && a.partial != nullptr) block_sum_store<T>(r2, a.partial + blockIdx.x);
-}
-
-// Dirichlet skeleton nodes: identity rows (residual 0), every copy.
-template <typename T, int OP>
-__global__ void __launch_bounds__(128) k_dirichlet(const LevelDev L, const SweepArgs<T> a) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= L.ndir) return;
-  const int n = L.n;
-  const int64_t E = L.entries;
-  const int s = L.dir_nodes[t];
-  const int b0 = L.skel_ptr[s], b1 = L.skel_ptr[s + 1];
-  const SkelInc I0 = L.skel_inc[b0];
-  const int64_t e0 = (int64_t)I0.macro * L.nt + lattice_index32(n, I0.i, I0.j, I0.k);
-  const T x0 = a.x[e0], y0 = a.x[e0 + E], z0 = a.x[e0 + 2 * E];
-  for (int q = b0; q < b1; ++q) {
-    const SkelInc I = L.skel_inc[q];
-    const int64_t e = (int64_t)I.macro * L.nt + lattice_index32(n, I.i, I.j, I.k);
-    if (OP == OP_RESID) {
-      a.out[e] = 0;
-      a.out[e + E] = 0;
-      a.out[e + 2 * E] = 0;
-    } else if (OP == OP_DIAG) {
-      a.out[e] = 1;
-      a.out[e + E] = 1;
-      a.out[e + 2 * E] = 1;
-    } else {
-      a.out[e] = x0;
-      a.out[e + E] = y0;
-      a.out[e + 2 * E] = z0;
-      if (OP == OP_CHEBY) {
-        a.dout[e] = 0;
-        a.dout[e + E] = 0;
-        a.dout[e + 2 * E] = 0;
-      }
-    }
-  }
-}
-
-// Free nodes on macro edges and vertices: one 128-thread block per node; warp w
-// takes incidences w, w+4, ...; lanes take candidate elements and directions
-// (incidence_lane).  Warp sums are combined in a fixed order, so the row is
-// deterministic, and it is written to every copy of the node.
-template <typename T, int OP>
-__global__ void __launch_bounds__(128) k_skeleton_ev(const LevelDev L, const MacroConsts<T>* __restrict__ mc,
-                                                      const OpFlags fl, const SweepArgs<T> a) {
-  __shared__ T part[4][6];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double r2 = 0.0;
-  const int s = L.ev_nodes[blockIdx.x];
-  const int n = L.n;
-  const int64_t E = L.entries;
-  const int b0 = L.skel_ptr[s], b1 = L.skel_ptr[s + 1];
-  const SkelInc I0 = L.skel_inc[b0];
-  const int64_t e0 = (int64_t)I0.macro * L.nt + lattice_index32(n, I0.i, I0.j, I0.k);
-  const T x0 = a.x[e0], y0 = a.x[e0 + E], z0 = a.x[e0 + 2 * E];
-  T ax = 0, ay = 0, az = 0, dgx = 0, dgy = 0, dgz = 0;
-  for (int q = b0 + warp; q < b1; q += 4) {
-    const SkelInc I = L.skel_inc[q];
-    const int64_t base = (int64_t)I.macro * L.nt;
-    incidence_lane<T>(mc[I.macro], a.x + base, a.k + base, E, n, I.i, I.j, I.k, lane, x0, y0, z0, fl, ax, ay, az,
-                      dgx, dgy, dgz);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    ax += __shfl_xor_sync(0xffffffffu, ax, o);
-    ay += __shfl_xor_sync(0xffffffffu, ay, o);
-    az += __shfl_xor_sync(0xffffffffu, az, o);
-    dgx += __shfl_xor_sync(0xffffffffu, dgx, o);
-    dgy += __shfl_xor_sync(0xffffffffu, dgy, o);
-    dgz += __shfl_xor_sync(0xffffffffu, dgz, o);
-  }
-  if (lane == 0) {
-    part[warp][0] = ax;
-    part[warp][1] = ay;
-    part[warp][2] = az;
-    part[warp][3] = dgx;
-    part[warp][4] = dgy;
-    part[warp][5] = dgz;
-  }
-  __syncthreads();
-  ax = (part[0][0] + part[1][0]) + (part[2][0] + part[3][0]);
-  ay = (part[0][1] + part[1][1]) + (part[2][1] + part[3][1]);
-  az = (part[0][2] + part[1][2]) + (part[2][2] + part[3][2]);
-  dgx = (part[0][3] + part[1][3]) + (part[2][3] + part[3][3]);
-  dgy = (part[0][4] + part[1][4]) + (part[2][4] + part[3][4]);
-  dgz = (part[0][5] + part[1][5]) + (part[2][5] + part[3][5]);
-  for (int q = b0 + threadIdx.x; q < b1; q += blockDim.x) {
-    const SkelInc I = L.skel_inc[q];
-    const int64_t e = (int64_t)I.macro * L.nt + lattice_index32(n, I.i, I.j, I.k);
-    double tmp = 0.0;
-    epilogue<T, OP>(a, e, E, ax, ay, az, dgx, dgy, dgz, x0, y0, z0, tmp);
-    if (q == b0) r2 = tmp;
-  }
-  if (OP == OP_RESID && a.partial != nullptr) block_sum_store<T>(r2, a.partial + blockIdx.x);
-}
-
-// Stokes element terms of one candidate element (permutation p, node at vertex av)
-// of one incident macro for the skeleton node at Kuhn coordinates (X, Y, Z): full
-// element sums of B u, C p (pressure row) and B^T p (velocity rows) -- no interface
-// rule applies to these coefficient-free blocks.
-template <typename T>
-__device__ __forceinline__ void stokes_candidate(const MacroConsts<T>& C, const T* __restrict__ px, int64_t E, int n,
-                                                 int X, int Y, int Z, int p, int av, T& ax, T& ay, T& az, T& yp) {
-  const int a0 = p >> 1;
-  const int lo = a0 == 0 ? 1 : 0, hi = a0 == 2 ? 1 : 2;
-  const int a1 = (p & 1) ? hi : lo, a2 = (p & 1) ? lo : hi;
-  const int oX = (av >= 1 && a0 == 0) + (av >= 2 && a1 == 0) + (av >= 3 && a2 == 0);
-  const int oY = (av >= 1 && a0 == 1) + (av >= 2 && a1 == 1) + (av >= 3 && a2 == 1);
-  const int oZ = (av >= 1 && a0 == 2) + (av >= 2 && a1 == 2) + (av >= 3 && a2 == 2);
-  bool ok = true;
-  int idx[4];
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const int VX = X - oX + (v >= 1 && a0 == 0) + (v >= 2 && a1 == 0) + (v >= 3 && a2 == 0);
-    const int VY = Y - oY + (v >= 1 && a0 == 1) + (v >= 2 && a1 == 1) + (v >= 3 && a2 == 1);
-    const int VZ = Z - oZ + (v >= 1 && a0 == 2) + (v >= 2 && a1 == 2) + (v >= 3 && a2 == 2);
-    ok = ok && kuhn_inside(n, VX, VY, VZ);
-    idx[v] = ok ? lattice_index32(n, VX - VY, VY - VZ, VZ) : 0;
-  }
-  if (!ok) return;
-#pragma unroll
-  for (int v = 0; v < 4; ++v) {
-    const T ux = px[idx[v]], uy = px[idx[v] + E], uz = px[idx[v] + 2 * E], pv = px[idx[v] + 3 * E];
-    const T* b = C.bd[p][av][v];
-    yp = fma(b[0], ux, yp);
-    yp = fma(b[1], uy, yp);
-    yp = fma(b[2], uz, yp);
-    yp = fma(C.lc[p][av][v], pv, yp);
-    const T* g = C.bd[p][v][av];
-    ax = fma(g[0], pv, ax);
-    ay = fma(g[1], pv, ay);
-    az = fma(g[2], pv, az);
-  }
-}
-
-// Stokes: face-interior skeleton nodes (Dirichlet ones included), one thread per
-// (node, incident macro); velocity part as in k_face_items unless the node is
-// velocity-Dirichlet, plus the element terms of B, B^T and C.
-template <typename T>
-__global__ void __launch_bounds__(128) k_face_items_stk(const LevelDev L, const MacroConsts<T>* __restrict__ mc,
-                                                         const OpFlags fl, const T* __restrict__ x,
-                                                         const T* __restrict__ kc) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= L.nface_items_all) return;
-  const FaceItem it = L.face_items_all[t];
-  const int n = L.n;
-  const int64_t E = L.entries;
-  const int64_t base = (int64_t)it.macro * L.nt;
-  const T* px = x + base;
-  const T* pk = kc + base;
-  const int c0 = lattice_index32(n, it.i, it.j, it.k);
-  const T x0 = px[c0], y0 = px[c0 + E], z0 = px[c0 + 2 * E];
-  T ax = 0, ay = 0, az = 0, dgx = 0, dgy = 0, dgz = 0, yp = 0;
-  const bool vdir = L.skel_dir[L.face_nodes_all[it.node]] != 0;
-  const MacroConsts<T>& C = mc[it.macro];
-  if (!vdir)
-    incidence_row<T>(C, px, pk, E, n, it.i, it.j, it.k, L.face_mask[it.f], (1u << NDIR) - 1u, x0, y0, z0, fl, ax, ay,
-                     az, dgx, dgy, dgz);
-  const uint32_t cand = L.face_mask[it.f];
-  const int X = it.i + it.j + it.k, Y = it.j + it.k, Z = it.k;
-#pragma unroll
-  for (int bit = 0; bit < 24; ++bit)
-    if ((cand >> bit) & 1u) stokes_candidate<T>(C, px, E, n, X, Y, Z, bit >> 2, bit & 3, ax, ay, az, yp);
-  T* acc = acc_of<T>(L) + 8 * (int64_t)it.node;
-  atomicAdd(acc + 0, ax);
-  atomicAdd(acc + 1, ay);
-  atomicAdd(acc + 2, az);
-  atomicAdd(acc + 6, yp);
-}
-
-template <typename T, int OP>
-__global__ void __launch_bounds__(128) k_face_finalize_stk(const LevelDev L, const SweepArgs<T> a) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  double r2 = 0.0;
-  if (t < L.nface_nodes_all) {
-    const int n = L.n;
-    const int64_t E = L.entries;
-    T* acc = acc_of<T>(L) + 8 * (int64_t)t;
-    const T ax = acc[0], ay = acc[1], az = acc[2], yp = acc[6];
-    acc[0] = 0;
-    acc[1] = 0;
-    acc[2] = 0;
-    acc[6] = 0;
-    const int s = L.face_nodes_all[t];
-    const bool vdir = L.skel_dir[s] != 0;
-    const int b0 = L.skel_ptr[s], b1 = L.skel_ptr[s + 1];
-    const SkelInc I0 = L.skel_inc[b0];
-    const int64_t e0 = (int64_t)I0.macro * L.nt + lattice_index32(n, I0.i, I0.j, I0.k);
-    const T x0 = a.x[e0], y0 = a.x[e0 + E], z0 = a.x[e0 + 2 * E];
-    for (int q = b0; q < b1; ++q) {
-      const SkelInc I = L.skel_inc[q];
-      const int64_t e = (int64_t)I.macro * L.nt + lattice_index32(n, I.i, I.j, I.k);
-      double tmp = 0.0;
-      stokes_epilogue<T, OP>(a, e, E, ax, ay, az, yp, x0, y0, z0, vdir, tmp);
-      if (q == b0) r2 = tmp;
-    }
-  }
-  if (OP == OP_RESID && a.partial != nullptr) block_sum_store<T>(r2, a.partial + blockIdx.x);
-}
-
-// Stokes: macro edge/vertex skeleton nodes (Dirichlet ones included), one block per node.
-template <typename T, int OP>
-__global__ void __launch_bounds__(128) k_skeleton_ev_stk(const LevelDev L, const MacroConsts<T>* __restrict__ mc,
-                                                          const OpFlags fl, const SweepArgs<T> a) {
-  __shared__ T part[4][4];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  double r2 = 0.0;
-  const int s = L.ev_all[blockIdx.x];
-  const bool vdir = L.skel_dir[s] != 0;
-  const int n = L.n;
-  const int64_t E = L.entries;
-  const int b0 = L.skel_ptr[s], b1 = L.skel_ptr[s + 1];
-  const SkelInc I0 = L.skel_inc[b0];
-  const int64_t e0 = (int64_t)I0.macro * L.nt + lattice_index32(n, I0.i, I0.j, I0.k);
-  const T x0 = a.x[e0], y0 = a.x[e0 + E], z0 = a.x[e0 + 2 * E];
-  T ax = 0, ay = 0, az = 0, dgx = 0, dgy = 0, dgz = 0, yp = 0;
-  for (int q = b0 + warp; q < b1; q += 4) {
-    const SkelInc I = L.skel_inc[q];
-    const int64_t base = (int64_t)I.macro * L.nt;
-    if (!vdir)
-      incidence_lane<T>(mc[I.macro], a.x + base, a.k + base, E, n, I.i, I.j, I.k, lane, x0, y0, z0, fl, ax, ay, az,
-                        dgx, dgy, dgz);
-    if (lane < 24)
-      stokes_candidate<T>(mc[I.macro], a.x + base, E, n, I.i + I.j + I.k, I.j + I.k, I.k, lane >> 2, lane & 3, ax, ay,
-                          az, yp);
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    ax += __shfl_xor_sync(0xffffffffu, ax, o);
-    ay += __shfl_xor_sync(0xffffffffu, ay, o);
-    az += __shfl_xor_sync(0xffffffffu, az, o);
-    yp += __shfl_xor_sync(0xffffffffu, yp, o);
-  }
-  if (lane == 0) {
-    part[warp][0] = ax;
-    part[warp][1] = ay;
-    part[warp][2] = az;
-    part[warp][3] = yp;
-  }
-  __syncthreads();
-  ax = (part[0][0] + part[1][0]) + (part[2][0] + part[3][0]);
-  ay = (part[0][1] + part[1][1]) + (part[2][1] + part[3][1]);
-  az = (part[0][2] + part[1][2]) + (part[2][2] + part[3][2]);
-  yp = (part[0][3] + part[1][3]) + (part[2][3] + part[3][3]);
-  for (int q = b0 + threadIdx.x; q < b1; q += blockDim.x) {
-    const SkelInc I = L.skel_inc[q];
-    const int64_t e = (int64_t)I.macro * L.nt + lattice_index32(n, I.i, I.j, I.k);
-    double tmp = 0.0;
-    stokes_epilogue<T, OP>(a, e, E, ax, ay, az, yp, x0, y0, z0, vdir, tmp);
-    if (q == b0) r2 = tmp;
-  }
-  if (OP == OP_RESID && a.partial != nullptr) block_sum_store<T>(r2, a.partial + blockIdx.x);
-}
-
 }  // namespace
 
 // one macro's interior launch: the BF16-coefficient kernel for FP32 sweeps of the default
@@ -1763,85 +1044,12 @@ int launch_sweep_macro(const LevelDev& L, const MacroStencil<T>* st_host, const 
   return (int)cudaGetLastError();
 }
 
-template <typename T>
-int launch_sweep(const LevelDev& L, const MacroStencil<T>* st_host, const MacroConsts<T>* mc_dev, OpKind op,
-                 const OpFlags& fl, const SweepArgs<T>& a, void* stream, int parts, int64_t partial_offset,
-                 int64_t* partial_count, void* stream_ev, void* stream_dir) {
-  cudaStream_t s = (cudaStream_t)stream;
-  cudaStream_t s_ev = stream_ev ? (cudaStream_t)stream_ev : s;
-  cudaStream_t s_dir = stream_dir ? (cudaStream_t)stream_dir : s;
-  const dim3 blk(TILE_I, TILE_J);
-  int64_t used = partial_offset;
-  const bool gen = !(fl.physical == 1 && fl.khat_edge == 0);
-  if ((parts & 1) && fl.batch && !fl.tile) {
-    int64_t nb = 0;
-    const int e = launch_sweep_batched<T>(L, mc_dev, op, fl, a, stream, used, &nb);
-    if (e != 0) return e;
-    used += nb;
-    parts &= ~1;
-  }
-  for (int m = 0; m < L.nmacro && (parts & 1); ++m) {
-    SweepArgs<T> am = a;
-    if (a.partial) am.partial = a.partial + used;
-    int nb = 0;
-    switch (op) {
-      case OP_APPLY: nb = launch_interior<T, OP_APPLY>(gen, L, st_host[m], m, fl, am, s); break;
-      case OP_RESID: nb = launch_interior<T, OP_RESID>(gen, L, st_host[m], m, fl, am, s); break;
-      case OP_JACOBI: nb = launch_interior<T, OP_JACOBI>(gen, L, st_host[m], m, fl, am, s); break;
-      case OP_CHEBY: nb = launch_interior<T, OP_CHEBY>(gen, L, st_host[m], m, fl, am, s); break;
-      case OP_DIAG: nb = launch_interior<T, OP_DIAG>(gen, L, st_host[m], m, fl, am, s); break;
-    }
-    used += nb;
-  }
-  if (parts & 2) {
-    if (L.nface_nodes > 0) {
-      const int nb = (L.nface_nodes + 127) / 128;
-      SweepArgs<T> am = a;
-      if (a.partial) am.partial = a.partial + used;
-      switch (op) {
-        case OP_APPLY: k_face_rows<T, OP_APPLY><<<nb, 128, 0, s>>>(L, mc_dev, fl, am); break;
-        case OP_RESID: k_face_rows<T, OP_RESID><<<nb, 128, 0, s>>>(L, mc_dev, fl, am); break;
-        case OP_JACOBI: k_face_rows<T, OP_JACOBI><<<nb, 128, 0, s>>>(L, mc_dev, fl, am); break;
-        case OP_CHEBY: k_face_rows<T, OP_CHEBY><<<nb, 128, 0, s>>>(L, mc_dev, fl, am); break;
-        case OP_DIAG: k_face_rows<T, OP_DIAG><<<nb, 128, 0, s>>>(L, mc_dev, fl, am); break;
-      }
-      used += nb;
-    }
-    if (L.nev > 0) {
-      const int nb = L.nev;
-      SweepArgs<T> am = a;
-      if (a.partial) am.partial = a.partial + used;
-      switch (op) {
-        case OP_APPLY: k_skeleton_ev<T, OP_APPLY><<<nb, 128, 0, s_ev>>>(L, mc_dev, fl, am); break;
-        case OP_RESID: k_skeleton_ev<T, OP_RESID><<<nb, 128, 0, s_ev>>>(L, mc_dev, fl, am); break;
-        case OP_JACOBI: k_skeleton_ev<T, OP_JACOBI><<<nb, 128, 0, s_ev>>>(L, mc_dev, fl, am); break;
-        case OP_CHEBY: k_skeleton_ev<T, OP_CHEBY><<<nb, 128, 0, s_ev>>>(L, mc_dev, fl, am); break;
-        case OP_DIAG: k_skeleton_ev<T, OP_DIAG><<<nb, 128, 0, s_ev>>>(L, mc_dev, fl, am); break;
-      }
-      used += nb;
-    }
-    if (L.ndir > 0) {
-      const int nb = (L.ndir + 127) / 128;
-      switch (op) {
-        case OP_APPLY: k_dirichlet<T, OP_APPLY><<<nb, 128, 0, s_dir>>>(L, a); break;
-        case OP_RESID: k_dirichlet<T, OP_RESID><<<nb, 128, 0, s_dir>>>(L, a); break;
-        case OP_JACOBI: k_dirichlet<T, OP_JACOBI><<<nb, 128, 0, s_dir>>>(L, a); break;
-        case OP_CHEBY: k_dirichlet<T, OP_CHEBY><<<nb, 128, 0, s_dir>>>(L, a); break;
-        case OP_DIAG: k_dirichlet<T, OP_DIAG><<<nb, 128, 0, s_dir>>>(L, a); break;
-      }
-    }
-  }
-  if (partial_count) *partial_count = used - partial_offset;
-  return (int)cudaGetLastError();
-}
-
 // ---------------------------------------------------------------------------
 // Residual with norm that allocates nothing.  Its scratch (per-block partial
 // sums of |r|^2 and the reduced result) lives in this file-scope device array,
 // which every GPU that loads the library holds until the process exits.  Host
 // code never uses the array's name as an address: the device address is looked
-// up once per device with cudaGetSymbolAddress.  Face-interior skeleton nodes
-// go through the warp-per-node kernel here, so no accumulator is needed.
+// up once per device with cudaGetSymbolAddress.
 // Calls that overlap on the GPU share the array and race.
 // ---------------------------------------------------------------------------
 __device__ __align__(256) static double g_noalloc_scratch[NOALLOC_SLOTS + 32];
@@ -1880,24 +1088,11 @@ int launch_residual_noalloc(const LevelDev& L, const MacroStencil<T>* st_host, c
     (gen ? k_interior<T, OP_RESID, 1> : k_interior<T, OP_RESID, 0>)<<<L.ntiles_lin, INTERIOR_BLOCK, 0, s>>>(L, st_host[m], m, fl, am, 0);
     used += L.ntiles_lin;
   }
-  if (L.nface_nodes > 0) {
-    LevelDev Lf = L;  // face-interior nodes through the warp-per-node path
-    Lf.ev_nodes = L.face_nodes;
-    Lf.nev = L.nface_nodes;
-    const int nb = L.nface_nodes;
-    SweepArgs<T> am = a;
-    am.partial = scratch + used;
-    k_skeleton_ev<T, OP_RESID><<<nb, 128, 0, s>>>(Lf, mc_dev, fl, am);
-    used += nb;
-  }
-  if (L.nev > 0) {
-    const int nb = L.nev;
-    SweepArgs<T> am = a;
-    am.partial = scratch + used;
-    k_skeleton_ev<T, OP_RESID><<<nb, 128, 0, s>>>(L, mc_dev, fl, am);
-    used += nb;
-  }
-  if (L.ndir > 0) k_dirichlet<T, OP_RESID><<<(L.ndir + 127) / 128, 128, 0, s>>>(L, a);
+  int64_t rows = 0;
+  a.partial = scratch;
+  const int er = launch_rows<T>(L, mc_dev, OP_RESID, fl, a, stream, used, &rows);
+  if (er != 0) return er;
+  used += rows;
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return (int)e;
   return launch_reduce(scratch, used, scratch + NOALLOC_SLOTS, stream);
@@ -1915,11 +1110,11 @@ int launch_stokes_sweep(const LevelDev& L, const MacroStencil<T>* st_host, const
                         void* const* side) {
   if (op != OP_APPLY && op != OP_RESID) return (int)cudaErrorInvalidValue;
   cudaStream_t s = (cudaStream_t)stream;
-  // side streams (nullable): [0] face chain, [1] every second macro, [2] edge/vertex nodes
-  cudaStream_t s_face = side ? (cudaStream_t)side[0] : s;
+  // side streams (nullable): [0] skeleton rows, [1] every second macro
   cudaStream_t s_odd = side ? (cudaStream_t)side[1] : s;
-  cudaStream_t s_ev = side ? (cudaStream_t)side[2] : s;
   int64_t used = 0;
+  const int er = launch_rows_stokes<T>(L, mc_dev, op, fl, a, side ? side[0] : stream, 0, &used);
+  if (er != 0) return er;
   const bool gen = !(fl.physical == 1 && fl.khat_edge == 0);
   if (fl.batch && L.ntiles_lin > 0) {
     for (int m0 = 0; m0 < L.nmacro; m0 += BATCH_MAX_MACROS) {
@@ -1949,27 +1144,6 @@ int launch_stokes_sweep(const LevelDev& L, const MacroStencil<T>* st_host, const
           L, st_host[m], m, fl, am, 0);
     used += L.ntiles_lin;
   }
-  if (L.nface_items_all > 0)
-    k_face_items_stk<T><<<(L.nface_items_all + 127) / 128, 128, 0, s_face>>>(L, mc_dev, fl, a.x, a.k);
-  if (L.nface_nodes_all > 0) {
-    const int nb = (L.nface_nodes_all + 127) / 128;
-    SweepArgs<T> am = a;
-    if (a.partial) am.partial = a.partial + used;
-    if (op == OP_APPLY)
-      k_face_finalize_stk<T, OP_APPLY><<<nb, 128, 0, s_face>>>(L, am);
-    else
-      k_face_finalize_stk<T, OP_RESID><<<nb, 128, 0, s_face>>>(L, am);
-    used += nb;
-  }
-  if (L.nev_all > 0) {
-    SweepArgs<T> am = a;
-    if (a.partial) am.partial = a.partial + used;
-    if (op == OP_APPLY)
-      k_skeleton_ev_stk<T, OP_APPLY><<<L.nev_all, 128, 0, s_ev>>>(L, mc_dev, fl, am);
-    else
-      k_skeleton_ev_stk<T, OP_RESID><<<L.nev_all, 128, 0, s_ev>>>(L, mc_dev, fl, am);
-    used += L.nev_all;
-  }
   if (partial_count) *partial_count = used;
   return (int)cudaGetLastError();
 }
@@ -1979,27 +1153,6 @@ template int launch_stokes_sweep<float>(const LevelDev&, const MacroStencil<floa
 template int launch_stokes_sweep<double>(const LevelDev&, const MacroStencil<double>*, const MacroConsts<double>*,
                                          OpKind, const OpFlags&, const SweepArgs<double>&, void*, int64_t*,
                                          void* const*);
-
-// fills the direction / ring tables used with run-time indices
-int upload_direction_tables() {
-  int dir[NDIR][3], ring[NDIR][3][2], rn[NDIR];
-  for (int d = 0; d < NDIR; ++d) {
-    dir[d][0] = dir_di(d);
-    dir[d][1] = dir_dj(d);
-    dir[d][2] = dir_dk(d);
-    rn[d] = ring_count(d);
-    for (int c = 0; c < 3; ++c) {
-      ring[d][c][0] = c < rn[d] ? ring_a(d, c) : 0;
-      ring[d][c][1] = c < rn[d] ? ring_b(d, c) : 0;
-    }
-  }
-  cudaError_t e = cudaMemcpyToSymbol(c_dir, dir, sizeof(dir));
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_ring, ring, sizeof(ring));
-  if (e == cudaSuccess) e = cudaMemcpyToSymbol(c_ring_n, rn, sizeof(rn));
-  // the copies may still be landing on the legacy stream, which library streams do not wait for
-  if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
-  return (int)e;
-}
 
 template <typename T>
 int launch_gs_colour(const LevelDev& L, const MacroStencil<T>* st_host, const MacroConsts<T>* mc_dev, const OpFlags& fl,
@@ -2054,9 +1207,4 @@ template int launch_sweep_macro<float>(const LevelDev&, const MacroStencil<float
 template int launch_sweep_macro<double>(const LevelDev&, const MacroStencil<double>*, const NodalConsts<double>*,
                                         int, OpKind, const OpFlags&, const SweepArgs<double>&, void*, int64_t,
                                         int64_t*);
-template int launch_sweep<float>(const LevelDev&, const MacroStencil<float>*, const MacroConsts<float>*, OpKind,
-                                 const OpFlags&, const SweepArgs<float>&, void*, int, int64_t, int64_t*, void*, void*);
-template int launch_sweep<double>(const LevelDev&, const MacroStencil<double>*, const MacroConsts<double>*, OpKind,
-                                  const OpFlags&, const SweepArgs<double>&, void*, int, int64_t, int64_t*, void*, void*);
-
 }  // namespace hhg
