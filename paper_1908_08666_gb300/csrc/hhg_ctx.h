@@ -101,7 +101,7 @@ struct KeyHash {
 struct LevelHost {
   int level = 0, n = 0;
   int64_t nt = 0, entries = 0;
-  std::vector<int32_t> tiles_int, tiles_all, tiles_lin, tiles_pair, tiles3, gs_chunks, columns;
+  std::vector<int32_t> tiles_int, tiles_all, tiles_lin, tiles_pair, tiles3, gs_points, columns;
   int32_t column_len = 1;
   int32_t gs_ptr[9] = {0};
   std::vector<int64_t> skel_entries;
@@ -127,7 +127,7 @@ struct LevelHost {
   std::vector<int64_t> rent;
   std::vector<double> rw;
   // device
-  DevMem d_columns, d_tiles_pair, d_tiles3, d_gs_chunks, d_skel_entries;
+  DevMem d_columns, d_tiles_pair, d_tiles3, d_gs_points, d_skel_entries;
   DevMem d_tiles_int, d_tiles_all, d_tiles_lin, d_skel_ptr, d_skel_inc, d_skel_dir, d_mask, d_first, d_e2u;
   DevMem d_row_lanes[2], d_row_warps[2], d_face_blocks[2], d_face_points[2], d_dir_entries;
   DevMem d_mask_own, d_invm64, d_invm32;  // owned-node mask; inverse lumped mass

@@ -518,21 +518,15 @@ void build_level(hhg_ctx* c, int level) {
   for (int k0 = 1; k0 <= n - 3; k0 += TILE3_K)
     for (int j0 = 1; j0 <= n - 2 - k0; j0 += TILE3_J)
       for (int i0 = 1; i0 <= n - 1 - k0 - j0; i0 += TILE3_I) L->tiles3.push_back((k0 << 20) | (j0 << 10) | i0);
-  // hybrid Gauss-Seidel colour chunks: for colour (ci, cj, ck) the rows j = cj (mod 2) of the
-  // slices k = ck (mod 2), split into chunks of 32 points i = ci (mod 2)
+  // hybrid Gauss-Seidel: the points of every colour (ci, cj, ck)
   for (int col = 0; col < 8; ++col) {
     const int ci = col >> 2, cj = (col >> 1) & 1, ck = col & 1;
-    L->gs_ptr[col] = (int32_t)L->gs_chunks.size();
-    for (int k = 1; k <= n - 3; ++k) {
-      if ((k & 1) != ck) continue;
-      for (int j = 1; j <= n - 2 - k; ++j) {
-        if ((j & 1) != cj) continue;
-        const int last = n - 1 - j - k;
-        for (int i0 = ci ? 1 : 2; i0 <= last; i0 += 64) L->gs_chunks.push_back((k << 20) | (j << 10) | i0);
-      }
-    }
+    L->gs_ptr[col] = (int32_t)L->gs_points.size();
+    for (int k = ck ? 1 : 2; k <= n - 3; k += 2)
+      for (int j = cj ? 1 : 2; j <= n - 2 - k; j += 2)
+        for (int i = ci ? 1 : 2; i <= n - 1 - j - k; i += 2) L->gs_points.push_back((k << 20) | (j << 10) | i);
   }
-  L->gs_ptr[8] = (int32_t)L->gs_chunks.size();
+  L->gs_ptr[8] = (int32_t)L->gs_points.size();
   // interior points of slice k, enumerated row by row (j = 1..M-1, i = 1..M-j, M = n-1-k),
   // in chunks of INTERIOR_BLOCK
   for (int k = 1; k <= n - 3; ++k) {
@@ -722,7 +716,7 @@ void upload_level(hhg_ctx* c, LevelHost& L) {
   upload(L.d_columns, L.columns);
   upload(L.d_tiles_pair, L.tiles_pair);
   upload(L.d_tiles3, L.tiles3);
-  upload(L.d_gs_chunks, L.gs_chunks);
+  upload(L.d_gs_points, L.gs_points);
   upload(L.d_skel_entries, L.skel_entries);
   upload(L.d_skel_ptr, L.skel_ptr);
   upload(L.d_skel_inc, L.skel_inc);
@@ -779,7 +773,7 @@ void upload_level(hhg_ctx* c, LevelHost& L) {
   D.ntiles3 = (int32_t)L.tiles3.size();
   D.tiles3 = L.d_tiles3.as<int32_t>();
   for (int q = 0; q < 9; ++q) D.gs_ptr[q] = L.gs_ptr[q];
-  D.gs_chunks = L.d_gs_chunks.as<int32_t>();
+  D.gs_points = L.d_gs_points.as<int32_t>();
   D.nskel_entries = (int64_t)L.skel_entries.size();
   D.skel_entries = L.d_skel_entries.as<int64_t>();
   D.nskel = (int32_t)L.skel_dir.size();
@@ -828,6 +822,7 @@ hhg_status hhg_create(hhg_ctx** out, int device, void* stream) {
     CK(c->scalar.alloc(64 * sizeof(double)));
     CK(cudaMallocHost((void**)&c->pinned, 64 * sizeof(double)));
     CK(upload_direction_tables());
+    CK(upload_gs_tables());
   });
   if (st != HHG_OK) {
     delete c;

@@ -236,11 +236,10 @@ struct LevelDev {
   const int32_t* columns;
   int32_t ntiles3;      // boxes of the shared-memory tile kernel: (k0 << 20) | (j0 << 10) | i0
   const int32_t* tiles3;
-  // hybrid Gauss-Seidel: chunks of up to 32 macro-interior points of one colour along a row,
-  // (k << 20) | (j << 10) | i0 (points i0, i0 + 2, ...), colour c's at [gs_ptr[c], gs_ptr[c+1]);
-  // colour = 4 (i % 2) + 2 (j % 2) + (k % 2) of the point's lattice coordinates
+  // hybrid Gauss-Seidel: the macro-interior points (k << 20) | (j << 10) | i of each colour
+  // 4 (i % 2) + 2 (j % 2) + (k % 2), colour c's at [gs_ptr[c], gs_ptr[c+1])
   int32_t gs_ptr[9];
-  const int32_t* gs_chunks;
+  const int32_t* gs_points;
   int64_t nskel_entries;           // entries of skeleton nodes (every copy)
   const int64_t* skel_entries;
   const int32_t* tiles_int;  // packed (k << 20) | (j0 << 10) | i0

@@ -95,13 +95,12 @@ template <typename T>
 int launch_residual_noalloc(const LevelDev& L, const MacroStencil<T>* st_host, const MacroConsts<T>* mc_dev,
                             const OpFlags& fl, SweepArgs<T> a, double* scratch, void* stream);
 
-// One colour pass of the hybrid Gauss-Seidel smoother on the macro interiors: every
-// macro-interior point of the colour, x_i += D_ii^-1 (f - A x)_i in place (a.x == a.out, a.omega
-// = 1); points of one colour are never neighbours.  mc_dev non-null: one launch for all macros
-// (stencils staged in shared memory); null: one launch per macro with st_host[m].
+// The Gauss-Seidel passes of the hybrid smoother over the macro interiors, all eight colours in place:
+// x_i += D_ii^-1 (f - A x)_i at every macro-interior point, colour by colour.
 template <typename T>
-int launch_gs_colour(const LevelDev& L, const MacroStencil<T>* st_host, const MacroConsts<T>* mc_dev, const OpFlags& fl,
-                     const SweepArgs<T>& a, int colour, void* stream);
+int launch_gs(const LevelDev& L, const MacroConsts<T>* mc_dev, const OpFlags& fl, const T* f, const T* k, T* x,
+              void* stream);
+int upload_gs_tables();  // its constant-memory tables (once per device)
 // dst[c * E + idx[u]] = src[c * E + idx[u]] for u < count, c < comps
 template <typename T>
 int launch_copy_entries(int64_t count, const int64_t* idx, int comps, int64_t E, const T* src, T* dst, void* stream);

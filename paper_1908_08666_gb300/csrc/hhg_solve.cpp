@@ -284,14 +284,7 @@ void smooth(hhg_ctx* c, int l, int steps, const T* f, T* x) {
       a.omega = c->mg.omega;
       CK(launch_rows<T>(L.dev, consts_dev<T>(L), OP_JACOBI, c->flags, a, c->stream, 0, nullptr));
       CK(launch_copy_entries<T>(L.dev.nskel_entries, L.dev.skel_entries, 3, L.entries, oth, x, c->stream));
-      SweepArgs<T> g{};
-      g.x = x;
-      g.f = f;
-      g.k = kptr<T>(L);
-      g.out = x;
-      g.omega = 1.0;
-      for (int col = 0; col < 8; ++col)
-        CK(launch_gs_colour<T>(L.dev, stencils<T>(L), consts_dev<T>(L), c->flags, g, col, c->stream));
+      CK(launch_gs<T>(L.dev, consts_dev<T>(L), c->flags, f, kptr<T>(L), x, c->stream));
     }
   } else {
     for (int s = 0; s < steps; ++s) {

@@ -189,29 +189,16 @@ __device__ __forceinline__ void interior_row(const MacroStencil<C>& st, const Op
 // STK = 1: the Stokes saddle operator [[A(mu), B^T], [B, C]] on (u, v, w, p) (Sec. 5.2),
 // the velocity block being the scaled-stencil operator of the 2 mu eps(u) form.
 // KB = 1 (FP32, default operator only): the coefficient is read as BF16 bits from a.k16.
-// GS = 1 (a colour pass of the hybrid Gauss-Seidel smoother): the block takes four chunks of
-// colour `colour`'s list (a warp each; lane l the point i0 + 2 l of the chunk's row) instead
-// of a slice chunk.
 // The body takes its block's index among the macro's blocks (`block`) and the slot of its
 // partial sum (`partial`, nullable) from the kernel around it.
-template <typename T, int OP, int GEN, int STK, int KB, int GS>
+template <typename T, int OP, int GEN, int STK, int KB>
 __device__ __forceinline__ void interior_point_body(const LevelDev& L, const MacroStencil<T>& st, const int macro,
                                                     const int block, double* partial, const OpFlags& fl,
-                                                    const SweepArgs<T>& a, const int colour) {
+                                                    const SweepArgs<T>& a) {
   const int n = L.n;
   int i = 0, j = 0, k = 0;
   bool valid;
-  if constexpr (GS) {
-    const int q = block * (INTERIOR_BLOCK / 32) + (threadIdx.x >> 5);
-    valid = q < L.gs_ptr[colour + 1] - L.gs_ptr[colour];
-    if (valid) {
-      const int32_t ch = L.gs_chunks[L.gs_ptr[colour] + q];
-      k = ch >> 20;
-      j = (ch >> 10) & 0x3FF;
-      i = (ch & 0x3FF) + 2 * (threadIdx.x & 31);
-      valid = i + j + k <= n - 1;
-    }
-  } else {
+  {
     const int32_t tile = L.tiles_lin[block];
     k = tile >> 20;
     const int M = n - 1 - k;
@@ -319,12 +306,12 @@ __device__ __forceinline__ void interior_point_body(const LevelDev& L, const Mac
 }
 
 // one launch per macro: the stencil is a kernel parameter
-template <typename T, int OP, int GEN, int STK = 0, int KB = 0, int GS = 0>
+template <typename T, int OP, int GEN, int STK = 0, int KB = 0>
 __global__ void __launch_bounds__(INTERIOR_BLOCK) k_interior(const LevelDev L, const MacroStencil<T> st,
                                                               const int macro, const OpFlags fl,
-                                                              const SweepArgs<T> a, const int colour) {
-  interior_point_body<T, OP, GEN, STK, KB, GS>(L, st, macro, blockIdx.x, a.partial ? a.partial + blockIdx.x : nullptr,
-                                               fl, a, colour);
+                                                              const SweepArgs<T> a) {
+  interior_point_body<T, OP, GEN, STK, KB>(L, st, macro, blockIdx.x, a.partial ? a.partial + blockIdx.x : nullptr,
+                                           fl, a);
 }
 
 // The interior stencil of one macro copied into shared memory by the whole block, each value
@@ -353,7 +340,7 @@ __global__ void __launch_bounds__(INTERIOR_BLOCK) k_interior_batched(const Level
   const int m = macro0 + blockIdx.y;
   stage_stencil(sst, &mc[m].st);
   double* partial = a.partial ? a.partial + (int64_t)blockIdx.y * gridDim.x + blockIdx.x : nullptr;
-  interior_point_body<T, OP, GEN, STK, KB, 0>(L, sst, m, blockIdx.x, partial, fl, a, 0);
+  interior_point_body<T, OP, GEN, STK, KB>(L, sst, m, blockIdx.x, partial, fl, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -525,19 +512,6 @@ __global__ void __launch_bounds__(INTERIOR_BLOCK, 4) k_interior_pair(const Level
                                                                    const int macro, const OpFlags fl,
                                                                    const SweepArgs<float> a) {
   interior_pair_body<OP, GEN, KB>(L, st, macro, blockIdx.x, a.partial ? a.partial + blockIdx.x : nullptr, fl, a);
-}
-
-// a colour pass of the hybrid Gauss-Seidel smoother over all macros (grid.y), each block staging
-// its macro's stencil in shared memory
-template <typename T, int GEN>
-__global__ void __launch_bounds__(INTERIOR_BLOCK) k_gs_colour_batched(const LevelDev L,
-                                                                       const MacroConsts<T>* __restrict__ mc,
-                                                                       const int macro0, const OpFlags fl,
-                                                                       const SweepArgs<T> a, const int colour) {
-  __shared__ MacroStencil<T> sst;
-  const int m = macro0 + blockIdx.y;
-  stage_stencil(sst, &mc[m].st);
-  interior_point_body<T, OP_JACOBI, GEN, 0, 0, 1>(L, sst, m, blockIdx.x, nullptr, fl, a, colour);
 }
 
 // all macros in one launch, as k_interior_batched: the block stages its macro's stencil as lane
@@ -937,9 +911,9 @@ int launch_interior(bool gen, const LevelDev& L, const MacroStencil<T>& st, int 
   } else {
     if (L.ntiles_lin == 0) return 0;
     if (gen)
-      k_interior<T, OP, 1><<<L.ntiles_lin, INTERIOR_BLOCK, 0, s>>>(L, st, m, fl, am, 0);
+      k_interior<T, OP, 1><<<L.ntiles_lin, INTERIOR_BLOCK, 0, s>>>(L, st, m, fl, am);
     else
-      k_interior<T, OP, 0><<<L.ntiles_lin, INTERIOR_BLOCK, 0, s>>>(L, st, m, fl, am, 0);
+      k_interior<T, OP, 0><<<L.ntiles_lin, INTERIOR_BLOCK, 0, s>>>(L, st, m, fl, am);
     return L.ntiles_lin;
   }
 }
@@ -1085,7 +1059,7 @@ int launch_residual_noalloc(const LevelDev& L, const MacroStencil<T>* st_host, c
   for (int m = 0; m < L.nmacro && L.ntiles_lin > 0; ++m) {
     SweepArgs<T> am = a;
     am.partial = scratch + used;
-    (gen ? k_interior<T, OP_RESID, 1> : k_interior<T, OP_RESID, 0>)<<<L.ntiles_lin, INTERIOR_BLOCK, 0, s>>>(L, st_host[m], m, fl, am, 0);
+    (gen ? k_interior<T, OP_RESID, 1> : k_interior<T, OP_RESID, 0>)<<<L.ntiles_lin, INTERIOR_BLOCK, 0, s>>>(L, st_host[m], m, fl, am);
     used += L.ntiles_lin;
   }
   int64_t rows = 0;
@@ -1138,10 +1112,10 @@ int launch_stokes_sweep(const LevelDev& L, const MacroStencil<T>* st_host, const
     cudaStream_t sm = m % 2 ? s_odd : s;
     if (op == OP_APPLY)
       (gen ? k_interior<T, OP_APPLY, 1, 1> : k_interior<T, OP_APPLY, 0, 1>)<<<L.ntiles_lin, INTERIOR_BLOCK, 0, sm>>>(
-          L, st_host[m], m, fl, am, 0);
+          L, st_host[m], m, fl, am);
     else
       (gen ? k_interior<T, OP_RESID, 1, 1> : k_interior<T, OP_RESID, 0, 1>)<<<L.ntiles_lin, INTERIOR_BLOCK, 0, sm>>>(
-          L, st_host[m], m, fl, am, 0);
+          L, st_host[m], m, fl, am);
     used += L.ntiles_lin;
   }
   if (partial_count) *partial_count = used;
@@ -1153,41 +1127,6 @@ template int launch_stokes_sweep<float>(const LevelDev&, const MacroStencil<floa
 template int launch_stokes_sweep<double>(const LevelDev&, const MacroStencil<double>*, const MacroConsts<double>*,
                                          OpKind, const OpFlags&, const SweepArgs<double>&, void*, int64_t*,
                                          void* const*);
-
-template <typename T>
-int launch_gs_colour(const LevelDev& L, const MacroStencil<T>* st_host, const MacroConsts<T>* mc_dev, const OpFlags& fl,
-                     const SweepArgs<T>& a, int colour, void* stream) {
-  const int count = L.gs_ptr[colour + 1] - L.gs_ptr[colour];
-  if (count == 0) return 0;
-  const int per = INTERIOR_BLOCK / 32;
-  const bool gen = !(fl.physical == 1 && fl.khat_edge == 0);
-  // all macros of the level in one launch per colour (grid.y: macros), or one launch per macro
-  // when only the stencil-parameter kernel applies (mc_dev null)
-  if (mc_dev) {
-    for (int m0 = 0; m0 < L.nmacro; m0 += BATCH_MAX_MACROS) {
-      const dim3 g((count + per - 1) / per, std::min(BATCH_MAX_MACROS, L.nmacro - m0));
-      if (gen)
-        k_gs_colour_batched<T, 1><<<g, INTERIOR_BLOCK, 0, (cudaStream_t)stream>>>(L, mc_dev, m0, fl, a, colour);
-      else
-        k_gs_colour_batched<T, 0><<<g, INTERIOR_BLOCK, 0, (cudaStream_t)stream>>>(L, mc_dev, m0, fl, a, colour);
-    }
-    return (int)cudaGetLastError();
-  }
-  const dim3 g((count + per - 1) / per);
-  for (int m = 0; m < L.nmacro; ++m) {
-    if (gen)
-      k_interior<T, OP_JACOBI, 1, 0, 0, 1><<<g, INTERIOR_BLOCK, 0, (cudaStream_t)stream>>>(L, st_host[m], m, fl, a,
-                                                                                            colour);
-    else
-      k_interior<T, OP_JACOBI, 0, 0, 0, 1><<<g, INTERIOR_BLOCK, 0, (cudaStream_t)stream>>>(L, st_host[m], m, fl, a,
-                                                                                            colour);
-  }
-  return (int)cudaGetLastError();
-}
-template int launch_gs_colour<float>(const LevelDev&, const MacroStencil<float>*, const MacroConsts<float>*,
-                                     const OpFlags&, const SweepArgs<float>&, int, void*);
-template int launch_gs_colour<double>(const LevelDev&, const MacroStencil<double>*, const MacroConsts<double>*,
-                                      const OpFlags&, const SweepArgs<double>&, int, void*);
 
 template <typename T>
 int launch_store_stencil(const LevelDev& L, const MacroStencil<double>* st_host, const OpFlags& fl, const double* k64,
