@@ -14,10 +14,10 @@ OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libhhgs.so")
 
 SOURCES = ["hhg_host.cpp", "hhg_solve.cpp", "hhg_learn.cpp", "hhg_sweep.cu", "hhg_sweep_f32.cu", "hhg_sweep_f64.cu", "hhg_stokes_f32.cu", "hhg_stokes_f64.cu",
-           "hhg_rows.cu", "hhg_gs.cu", "hhg_vec.cu", "hhg_learn.cu",
+           "hhg_rows_f32.cu", "hhg_rows_f64.cu", "hhg_gs.cu", "hhg_vec.cu", "hhg_learn.cu",
            "hhg_twod.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC,-O2",
+FLAGS = ["-O3", "--split-compile", "0", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC,-O2",
          "-I" + os.path.join(os.path.dirname(HERE), "include")]
 
 

@@ -112,8 +112,9 @@ struct LevelHost {
   std::vector<std::array<int64_t, 3>> skel_key;
   int32_t nface_nodes = 0, nev = 0;  // free nodes on macro faces; on macro edges and vertices
   // skeleton rows and Dirichlet entries (LevelDev); [1]: the Stokes lists
-  std::vector<RowLane> row_lanes[2];
-  std::vector<int32_t> row_warps[2];
+  std::vector<EvWarp> ev_warps[2];
+  std::vector<EdgeBlock> edge_blocks[2];
+  std::vector<EdgeSide> edge_sides[2];
   std::vector<FaceBlock> face_blocks[2];
   std::vector<FacePoint> face_points[2];
   std::vector<int64_t> dir_entries;
@@ -129,7 +130,7 @@ struct LevelHost {
   // device
   DevMem d_columns, d_tiles_pair, d_tiles3, d_gs_points, d_skel_entries;
   DevMem d_tiles_int, d_tiles_all, d_tiles_lin, d_skel_ptr, d_skel_inc, d_skel_dir, d_mask, d_first, d_e2u;
-  DevMem d_row_lanes[2], d_row_warps[2], d_face_blocks[2], d_face_points[2], d_dir_entries;
+  DevMem d_ev_warps[2], d_edge_blocks[2], d_edge_sides[2], d_face_blocks[2], d_face_points[2], d_dir_entries;
   DevMem d_mask_own, d_invm64, d_invm32;  // owned-node mask; inverse lumped mass
   DevMem d_mass64, d_mass32;              // lumped mass
   DevMem d_sdiag64, d_sdiag32;            // Stokes: diagonal of -C (pressure stabilisation)
@@ -323,8 +324,8 @@ inline int64_t max_partials(hhg_ctx* c) {
   for (int l = c->level_min; l <= c->level_max; ++l) {
     const LevelHost& L = *c->levels[l];
     mx = std::max<int64_t>(mx, (int64_t)std::max({L.tiles_lin.size(), L.tiles3.size(), (L.columns.size() + 127) / 128}) * (int64_t)c->tets.size() +
-                                   (int64_t)std::max(L.row_warps[0].size() + L.face_blocks[0].size(),
-                                                     L.row_warps[1].size() + L.face_blocks[1].size()) + 8);
+                                   (int64_t)std::max(L.ev_warps[0].size() / 4 + L.edge_blocks[0].size() + L.face_blocks[0].size(),
+                                                     L.ev_warps[1].size() / 4 + L.edge_blocks[1].size() + L.face_blocks[1].size()) + 8);
   }
   return mx;
 }

@@ -277,7 +277,8 @@ int launch_gs(const LevelDev& L, const MacroConsts<T>* mc, const OpFlags& fl, co
   for (int m0 = 0; m0 < L.nmacro; m0 += GS_MAX_MACROS) {
     const int nm = std::min(GS_MAX_MACROS, L.nmacro - m0);
     if ((int64_t)most * L.nmacro <= GS_MACRO_MAX_POINTS) {
-      // blocks per macro: enough for the largest colour, no more than share the SMs, at most 8
+      // blocks per macro: enough for the largest colour, no more than share the SMs, a power of two up
+      // to 8 (three blocks per macro were slower than two: 118 against 73 us on 48 macros)
       int parts = 1;
       while (parts < 8 && parts * (GSM_BLOCK / 8) < most && 2 * parts * L.nmacro <= 152) parts *= 2;
       cudaLaunchConfig_t cfg = {};

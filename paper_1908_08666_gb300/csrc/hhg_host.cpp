@@ -314,16 +314,16 @@ void macro_constants(const MacroGeom& G, int n, double c_eps, double c_div, Macr
         if (std::fabs(S[r] - want[r]) > 1e-12 * (1 + std::fabs(want[r])))
           THROW(HHG_ERR_STATE, "Shat(-d) != Shat(d) for direction %d", d);
     }
+    // axial vector of the ring pair (cyc[q], cyc[q + nr]), and its dependency on a red edge
+    const int nr = dir_red(d) ? 3 : 2;
+    auto axial = [&](int q, int r) {
+      for (int c = 0; c < ring_count(d); ++c) {
+        if (ring_a(d, c) == ring_cyc(d, q)) return out.st.s[d][c][r];
+        if (ring_b(d, c) == ring_cyc(d, q)) return -out.st.s[d][c][r];
+      }
+      THROW(HHG_ERR_STATE, "ring pair of direction %d not found", d);
+    };
     if (d < 7) {
-      // axial vector of the ring pair (cyc[q], cyc[q + nr]), and its dependency on a red edge
-      const int nr = dir_red(d) ? 3 : 2;
-      auto axial = [&](int q, int r) {
-        for (int c = 0; c < ring_count(d); ++c) {
-          if (ring_a(d, c) == ring_cyc(d, q)) return out.st.s[d][c][r];
-          if (ring_b(d, c) == ring_cyc(d, q)) return -out.st.s[d][c][r];
-        }
-        THROW(HHG_ERR_STATE, "ring pair of direction %d not found", d);
-      };
       for (int r = 0; r < 6; ++r) out.mar[d][r] = out.st.S[d][r];
       for (int r = 0; r < 3; ++r) {
         out.mar[d][6 + r] = axial(0, r);
@@ -337,7 +337,7 @@ void macro_constants(const MacroGeom& G, int n, double c_eps, double c_div, Macr
       out.mar[d][19] = 0;
     }
     for (int r = 0; r < 6; ++r) out.sc[d][r] = out.st.S[d < 7 ? d : d - 7][r];
-    for (int r = 0; r < 9; ++r) out.sc[d][6 + r] = out.st.s[d][r / 3][r % 3];
+    for (int r = 0; r < 9; ++r) out.sc[d][6 + r] = r / 3 < ring_count(d) ? axial(r / 3, r % 3) : 0;
     out.sc[d][15] = 0;
     for (int l = 0; l < 3; ++l) {
       out.sb[d][l] = out.st.B[d][l];
@@ -384,11 +384,9 @@ MacroConsts<T> cast_consts(const MacroConsts<double>& c) {
 
 
 
-// Lanes, warps and face blocks of the skeleton rows (LevelDev).  Nodes on macro edges and vertices:
-// the incidences of a node take a power of two of lanes, spread over the warp (lane = incidence *
-// nodes per warp + node), more than 32 of them several rounds.  Nodes are ordered by how many lanes they take (most first, they run
-// longest), then by macros and the faces or edges they lie on, so that the lanes of a warp read
-// the same constants and neighbouring points.
+// Blocks of the skeleton rows (LevelDev).  Macro vertices take 1, 2 or 4 warps of a block by their number
+// of incidences (two per warp and round, two rounds), the widest first (they run longest); nodes inside a
+// macro edge lie in the same macros and are numbered along it; nodes inside faces are ordered by macros and face types, those next to the face's edges apart.
 void build_rows(LevelHost& L) {
   const int n = L.n;
   const int64_t nskel = (int64_t)L.skel_dir.size();
@@ -396,39 +394,68 @@ void build_rows(LevelHost& L) {
     return (I.i + I.j + I.k == n ? 1 : 0) | (I.i == 0 ? 2 : 0) | (I.j == 0 ? 4 : 0) | (I.k == 0 ? 8 : 0);
   };
   struct Key {
-    int32_t rounds, lg, near, m0, p0, m1, p1;
+    int32_t rounds, warps, near, m0, p0, m1, p1;
     int64_t s;
     bool operator<(const Key& o) const {
-      return std::make_tuple(-rounds, -lg, -near, m0, p0, m1, p1, s) <
-             std::make_tuple(-o.rounds, -o.lg, -o.near, o.m0, o.p0, o.m1, o.p1, o.s);
+      return std::make_tuple(-rounds, -warps, -near, m0, p0, m1, p1, s) <
+             std::make_tuple(-o.rounds, -o.warps, -o.near, o.m0, o.p0, o.m1, o.p1, o.s);
     }
   };
   for (int stk = 0; stk < 2; ++stk) {
-    std::vector<RowLane>& lanes = L.row_lanes[stk];
-    std::vector<int32_t>& warps = L.row_warps[stk];
     std::vector<Key> keys, faces;
+    std::map<std::array<int64_t, 2>, std::vector<std::pair<int64_t, int64_t>>> edges;  // vertices -> (weight, node)
     for (int64_t s = 0; s < nskel; ++s) {
       if (L.skel_dir[s] && !stk) continue;
+      if (L.skel_support[s] == 2) {
+        const std::array<int64_t, 3>& key = L.skel_key[s];
+        edges[{key[0] / 4096, key[1] / 4096}].push_back({key[0] % 4096, s});
+        continue;
+      }
       const int b0 = L.skel_ptr[s], ni = L.skel_ptr[s + 1] - b0;
-      Key q{(ni + 31) / 32, 0, 0, L.skel_inc[b0].macro, primitive(L.skel_inc[b0]), -1, 0, s};
-      while ((1 << q.lg) < std::min(ni, 32)) ++q.lg;
+      Key q{(ni + 15) / 16, ni > 8 ? 4 : ni > 4 ? 2 : 1, 0, L.skel_inc[b0].macro, primitive(L.skel_inc[b0]), -1, 0, s};
       if (ni > 1) {
         q.m1 = L.skel_inc[b0 + 1].macro;
         q.p1 = primitive(L.skel_inc[b0 + 1]);
       }
-      if (q.rounds > 255) THROW(HHG_ERR_UNSUPPORTED, "a node lies in %d macros (at most %d)", ni, 255 * 32);
       // next to a face's edges one of the three non-zero barycentric weights is 1
       const SkelInc& I = L.skel_inc[b0];
       if (L.skel_support[s] == 3)
         for (const int w : {n - I.i - I.j - I.k, (int)I.i, (int)I.j, (int)I.k}) q.near |= w == 1;
       (L.skel_support[s] == 3 ? faces : keys).push_back(q);
     }
+    for (auto& ed : edges) {
+      std::sort(ed.second.begin(), ed.second.end());
+      for (size_t q0 = 0; q0 < ed.second.size(); q0 += 32) {
+        const size_t count = std::min<size_t>(32, ed.second.size() - q0);
+        const int64_t s = ed.second[q0].second, t = count > 1 ? ed.second[q0 + 1].second : s;
+        const int b0 = L.skel_ptr[s], ni = L.skel_ptr[s + 1] - b0;
+        L.edge_blocks[stk].push_back(
+            EdgeBlock{(int32_t)L.edge_sides[stk].size(), ni, (int16_t)count, L.skel_dir[s]});
+        for (int q = 0; q < ni; ++q) {
+          const SkelInc &I = L.skel_inc[b0 + q], &J = L.skel_inc[L.skel_ptr[t] + q];
+          const int p = primitive(I);  // bit f: on face f
+          const int edge = p == 3 ? 4 : p == 5 ? 5 : p == 9 ? 6 : p == 6 ? 7 : p == 10 ? 8 : p == 12 ? 9 : -1;
+          if (edge < 0 || I.macro != J.macro) THROW(HHG_ERR_STATE, "macro edge node off its edge");
+          L.edge_sides[stk].push_back(EdgeSide{
+              I.macro, {I.i, I.j, I.k}, {(int8_t)(J.i - I.i), (int8_t)(J.j - I.j), (int8_t)(J.k - I.k)}, (int8_t)edge});
+          // the points of the block in this macro
+          const EdgeSide& S = L.edge_sides[stk].back();
+          for (size_t r = 0; r < count; ++r) {
+            const int64_t u = ed.second[q0 + r].second;
+            const SkelInc& U = L.skel_inc[L.skel_ptr[u] + q];
+            if (L.skel_ptr[u + 1] - L.skel_ptr[u] != ni || U.macro != I.macro || U.i != I.i + (int)r * S.step[0] ||
+                U.j != I.j + (int)r * S.step[1] || U.k != I.k + (int)r * S.step[2])
+              THROW(HHG_ERR_STATE, "macro edge nodes are not in line");
+          }
+        }
+      }
+    }
     std::sort(keys.begin(), keys.end());
     std::sort(faces.begin(), faces.end());
     for (size_t q0 = 0; q0 < faces.size();) {
       const Key& K = faces[q0];
       size_t q1 = q0;
-      while (q1 < faces.size() && q1 - q0 < 32 && faces[q1].lg == K.lg && faces[q1].near == K.near && faces[q1].m0 == K.m0 && faces[q1].p0 == K.p0 &&
+      while (q1 < faces.size() && q1 - q0 < 32 && faces[q1].near == K.near && faces[q1].m0 == K.m0 && faces[q1].p0 == K.p0 &&
              faces[q1].m1 == K.m1 && faces[q1].p1 == K.p1)
         ++q1;
       auto face_of = [](int p) { return p == 1 ? 0 : p == 2 ? 1 : p == 4 ? 2 : 3; };
@@ -445,34 +472,15 @@ void build_rows(LevelHost& L) {
         }
       q0 = q1;
     }
-    for (size_t q0 = 0; q0 < keys.size();) {
-      const Key& K = keys[q0];
-      const int per = 32 >> K.lg;
-      size_t q1 = q0;
-      while (q1 < keys.size() && q1 - q0 < (size_t)per && keys[q1].lg == K.lg && keys[q1].rounds == K.rounds) ++q1;
-      warps.push_back((int32_t)(lanes.size() / 32));
-      const uint16_t common = (uint16_t)(K.lg | (K.rounds << ROW_ROUNDS_SHIFT));
-      for (int r = 0; r < K.rounds; ++r)
-        for (int lane = 0; lane < 32; ++lane) {
-          const size_t q = q0 + lane % per;
-          const int inc = 32 * r + lane / per;
-          RowLane R{-1, 0, 0, 0, common};
-          if (q < q1) {
-            const int64_t s = keys[q].s;
-            if (L.skel_ptr[s] + inc < L.skel_ptr[s + 1]) {
-              const SkelInc& I = L.skel_inc[L.skel_ptr[s] + inc];
-              R.macro = I.macro;
-              R.i = I.i;
-              R.j = I.j;
-              R.k = I.k;
-              if (L.skel_dir[s]) R.flags |= ROW_VDIR;
-              if (inc == 0) R.flags |= ROW_FIRST;
-            }
-          }
-          lanes.push_back(R);
-        }
-      q0 = q1;
+    for (const Key& K : keys) {
+      std::vector<EvWarp>& W = L.ev_warps[stk];
+      // keys are ordered by width, so a node's warps never straddle two blocks
+      const int16_t w0 = (int16_t)(W.size() % 4);
+      for (int w = 0; w < K.warps; ++w)
+        W.push_back(EvWarp{L.skel_ptr[K.s], L.skel_ptr[K.s + 1] - L.skel_ptr[K.s], L.skel_dir[K.s], (int16_t)w, w0,
+                           (int16_t)K.warps});
     }
+    while (L.ev_warps[stk].size() % 4) L.ev_warps[stk].push_back(EvWarp{-1, 0, 0, 0, 0, 1});
   }
 }
 
@@ -737,8 +745,9 @@ void upload_level(hhg_ctx* c, LevelHost& L) {
     upload(L.d_mass32, m32);
   }
   for (int q = 0; q < 2; ++q) {
-    upload(L.d_row_lanes[q], L.row_lanes[q]);
-    upload(L.d_row_warps[q], L.row_warps[q]);
+    upload(L.d_ev_warps[q], L.ev_warps[q]);
+    upload(L.d_edge_blocks[q], L.edge_blocks[q]);
+    upload(L.d_edge_sides[q], L.edge_sides[q]);
     upload(L.d_face_blocks[q], L.face_blocks[q]);
     upload(L.d_face_points[q], L.face_points[q]);
   }
@@ -783,13 +792,12 @@ void upload_level(hhg_ctx* c, LevelHost& L) {
   D.mask = L.d_mask.as<uint8_t>();
   D.nface_nodes = L.nface_nodes;
   D.nev = L.nev;
-  D.nrow_skel = (int32_t)L.row_warps[0].size();
-  D.row_lanes = L.d_row_lanes[0].as<RowLane>();
-  D.row_warps = L.d_row_warps[0].as<int32_t>();
-  D.nrow_stk = (int32_t)L.row_warps[1].size();
-  D.row_lanes_stk = L.d_row_lanes[1].as<RowLane>();
-  D.row_warps_stk = L.d_row_warps[1].as<int32_t>();
   for (int q = 0; q < 2; ++q) {
+    D.nev_blocks[q] = (int32_t)(L.ev_warps[q].size() / 4);
+    D.ev_warps[q] = L.d_ev_warps[q].as<EvWarp>();
+    D.nedge_blocks[q] = (int32_t)L.edge_blocks[q].size();
+    D.edge_blocks[q] = L.d_edge_blocks[q].as<EdgeBlock>();
+    D.edge_sides[q] = L.d_edge_sides[q].as<EdgeSide>();
     D.nface_blocks[q] = (int32_t)L.face_blocks[q].size();
     D.face_blocks[q] = L.d_face_blocks[q].as<FaceBlock>();
     D.face_points[q] = L.d_face_points[q].as<FacePoint>();

@@ -172,7 +172,9 @@ struct NodalConsts {
 template <typename T>
 struct alignas(16) MacroConsts {
   T el[NDIR][6][16];
-  T sc[NDIR][16];  // the scaled block of direction d: S (6 values) and s (3 x 3) of the interior stencil
+  // the scaled block of direction d: S (6 values) and the axial vectors of the ring pairs
+  // (ring_cyc q, q + 3 resp. q + 2)
+  T sc[NDIR][16];
   T sb[NDIR][8];   // its Stokes blocks: B, G (3 values each), C
   // the marching kernel's constants per direction pair: S, the axial vectors of the ring pairs
   // (ring_cyc 0 and 2; 0 and 1 of a four-element edge), B, G, C
@@ -193,12 +195,27 @@ struct SkelInc {
   int16_t pad;
 };
 
-// one lane of the edge and vertex rows: an incidence of a node (macro < 0: idle), and what the warp does with it
-struct RowLane {
-  int32_t macro;
-  int16_t i, j, k;
-  uint16_t flags;
+// Rows of macro vertices: half a warp takes an incidence, `warps` warps of a block a
+// node.  EvWarp: what a warp of a block does (first < 0: nothing): `count` incidences of the node from
+// skel_inc[first] on, of which it takes 2 w, 2 w + 1, 2 (w + warps), ...; the block's warps
+// w0 .. w0 + warps - 1 share the node.
+struct EvWarp {
+  int32_t first, count;
+  int16_t vdir, w, w0, warps;
 };
+
+// A block of up to 32 nodes of one macro edge, in `macros` macros: edge_sides[first ..]; in each the
+// points at + lane * step, on the macro's edge 4 .. 9 (hhg_rows.cuh)
+struct EdgeBlock {
+  int32_t first, macros;
+  int16_t count, vdir;
+};
+struct EdgeSide {
+  int32_t macro;
+  int16_t at[3];
+  int8_t step[3], edge;
+};
+
 // A block of 32 nodes in the interior of one macro face, seen from the
 // macros on its sides (the second < 0 on an outer face); face F of the macro: 0 is i + j + k = n,
 // 1 i = 0, 2 j = 0, 3 k = 0.
@@ -213,11 +230,6 @@ struct FaceBlock {
 struct FacePoint {
   int16_t i, j, k, pad;
 };
-constexpr int ROW_LG = 7;       // log2 of the lanes that share a node (the same in the whole warp)
-constexpr int ROW_VDIR = 8;     // velocity-Dirichlet node (Stokes lists)
-constexpr int ROW_FIRST = 32;   // the node's first incidence (counts in norms)
-constexpr int ROW_ROUNDS_SHIFT = 8;  // rounds of 32 lanes of the warp (the same in the whole warp)
-
 // device view of one level
 struct LevelDev {
   int n;
@@ -250,15 +262,14 @@ struct LevelDev {
   const int8_t* skel_dir;    // Dirichlet flag per skeleton node
   const uint8_t* mask;       // [entries] 1 = owned copy of a free node (dot products)
   int32_t nface_nodes, nev;  // free nodes in the interior of macro faces; on macro edges and vertices
-  // skeleton rows (hhg_rows.cuh).  Nodes on macro edges and vertices: lanes in units of 32, the first
-  // unit of every warp; _stk: with the velocity-Dirichlet nodes (their pressure rows are free)
-  int32_t nrow_skel, nrow_stk;
-  const RowLane* row_lanes;
-  const int32_t* row_warps;
-  const RowLane* row_lanes_stk;
-  const int32_t* row_warps_stk;
+  // skeleton rows (hhg_rows.cuh); [1] of each: the Stokes lists, with the velocity-Dirichlet nodes
+  // (their pressure rows are free).  Macro vertices and edges:
+  int32_t nev_blocks[2], nedge_blocks[2];
+  const EvWarp* ev_warps[2];  // four a block
+  const EdgeBlock* edge_blocks[2];
+  const EdgeSide* edge_sides[2];
   // nodes in the interior of macro faces: points of block b from its side q at
-  // face_points[64 b + 32 q ..]; [1]: the Stokes lists
+  // face_points[64 b + 32 q ..]
   int32_t nface_blocks[2];
   const FaceBlock* face_blocks[2];
   const FacePoint* face_points[2];

@@ -108,6 +108,7 @@ int launch_copy_entries(int64_t count, const int64_t* idx, int comps, int64_t E,
 // constant-memory direction tables of the skeleton kernel (once per device)
 int upload_direction_tables();
 // its parts, one for every translation unit with skeleton rows
+int upload_tables_rows_f64();
 int upload_tables_f32();
 int upload_tables_f64();
 int upload_tables_stokes_f32();

@@ -32,19 +32,6 @@ namespace hhg {
 
 namespace {
 
-// (j, i) of the t-th interior point of a slice with M = n-1-k: rows j = 1..M-1 hold
-// M-j points; C(j) = (j-1)(2M-j)/2 points precede row j.
-__device__ __forceinline__ void slice_decode(int M, int t, int& j, int& i) {
-  const float b = (float)(2 * M - 1);
-  int u = (int)floorf(0.5f * (b - sqrtf(fmaxf(b * b - 8.0f * (float)t, 0.0f))));
-  u = max(0, min(u, M - 2));
-  // exact correction: C(u+1) <= t < C(u+2)
-  if (((u + 1) * (2 * M - u - 2)) / 2 <= t) ++u;
-  if ((u * (2 * M - u - 1)) / 2 > t) --u;
-  j = u + 1;
-  i = t - (u * (2 * M - u - 1)) / 2 + 1;
-}
-
 // The scaled-stencil row of one macro-interior node (Lemma 2.1, eq. correctionterm3D) from
 // the coefficients kk[d] = k_{i+d}, k0 = k_i and the neighbour differences
 // dx/dy/dz[d] = x_{i+d} - x_i of its 14 stencil directions: (A x)_i = (ax, ay, az) and, with

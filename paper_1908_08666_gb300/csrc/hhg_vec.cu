@@ -13,6 +13,7 @@
 
 #include "hhg_internal.h"
 #include "hhg_launch.h"
+#include "hhg_row.cuh"
 
 namespace hhg {
 
@@ -54,10 +55,10 @@ __global__ void k_dot(const uint8_t* __restrict__ mask, int64_t E, int comps, co
   block_store(v, partials + blockIdx.x);
 }
 
-// fine point (i, j, k) of macro `m` of the fine level; adds P e_c
-template <typename T>
-__global__ void k_prolong_add(const LevelDev Lf, const LevelDev Lc, const T* __restrict__ ec, T* __restrict__ ef,
-                              int comps) {
+// fine point (i, j, k) of macro `m` of the fine level; adds P e_c.  Bound by memory (the fine field read
+// and written); all components' loads are in flight together.
+template <typename T, int COMPS>
+__global__ void k_prolong_add(const LevelDev Lf, const LevelDev Lc, const T* __restrict__ ec, T* __restrict__ ef) {
   const int m = blockIdx.y;
   const int32_t tile = Lf.tiles_all[blockIdx.x];
   const int k = tile >> 20;
@@ -65,64 +66,83 @@ __global__ void k_prolong_add(const LevelDev Lf, const LevelDev Lc, const T* __r
   const int i = (tile & 1023) + threadIdx.x;
   const int n = Lf.n, nc = Lc.n;
   if (i + j + k > n) return;
-  const int X = i + j + k, Y = j + k, Z = k;
-  const int pX = X & 1, pY = Y & 1, pZ = Z & 1;
-  const int64_t ef0 = (int64_t)m * Lf.nt + lattice_index(n, i, j, k);
-  const int64_t cb = (int64_t)m * Lc.nt;
-  if (!(pX | pY | pZ)) {
-    const int64_t c = cb + lattice_index(nc, i >> 1, j >> 1, k >> 1);
-    for (int q = 0; q < comps; ++q) ef[ef0 + q * Lf.entries] += ec[c + q * Lc.entries];
-  } else {
-    const int di = pX - pY, dj = pY - pZ, dk = pZ;
-    const int64_t ca = cb + lattice_index(nc, (i - di) >> 1, (j - dj) >> 1, (k - dk) >> 1);
-    const int64_t cc = cb + lattice_index(nc, (i + di) >> 1, (j + dj) >> 1, (k + dk) >> 1);
-    for (int q = 0; q < comps; ++q)
-      ef[ef0 + q * Lf.entries] += (T)0.5 * (ec[ca + q * Lc.entries] + ec[cc + q * Lc.entries]);
+  const int pX = (i + j + k) & 1, pY = (j + k) & 1, pZ = k & 1;
+  const int64_t Ef = Lf.entries, Ec = Lc.entries;
+  T* f = ef + (int64_t)m * Lf.nt + lattice_index32(n, i, j, k);
+  const T* __restrict__ c = ec + (int64_t)m * Lc.nt;
+  // the coarse edge's end points, (i, j, k) -+ the parities' direction (both the point itself on a
+  // coarse point)
+  const int di = pX - pY, dj = pY - pZ, dk = pZ;
+  const int ca = lattice_index32(nc, (i - di) >> 1, (j - dj) >> 1, (k - dk) >> 1);
+  const int cb = lattice_index32(nc, (i + di) >> 1, (j + dj) >> 1, (k + dk) >> 1);
+  T v[COMPS], a[COMPS], b[COMPS];
+#pragma unroll
+  for (int q = 0; q < COMPS; ++q) {
+    v[q] = f[q * Ef];
+    a[q] = __ldg(c + ca + q * Ec);
+    b[q] = __ldg(c + cb + q * Ec);
   }
+#pragma unroll
+  for (int q = 0; q < COMPS; ++q) f[q * Ef] = v[q] + ((pX | pY | pZ) ? (T)0.5 * (a[q] + b[q]) : a[q]);
 }
 
 // coarse macro-interior points: rc(p) = rf(2p) + 1/2 sum_d rf(2p + d)
-template <typename T>
-__global__ void k_restrict_interior(const LevelDev Lf, const LevelDev Lc, const T* __restrict__ rf,
-                                    T* __restrict__ rc, int comps) {
+template <typename T, int COMPS>
+__global__ void __launch_bounds__(INTERIOR_BLOCK)
+    k_restrict_interior(const LevelDev Lf, const LevelDev Lc, const T* __restrict__ rf, T* __restrict__ rc) {
   const int m = blockIdx.y;
-  const int32_t tile = Lc.tiles_int[blockIdx.x];
-  const int k = tile >> 20;
-  const int j = ((tile >> 10) & 1023) + threadIdx.y;
-  const int i = (tile & 1023) + threadIdx.x;
-  const int n = Lf.n, nc = Lc.n;
-  if (i + j + k > nc - 1) return;
-  const int64_t fb = (int64_t)m * Lf.nt;
-  const int64_t c = (int64_t)m * Lc.nt + lattice_index(nc, i, j, k);
-  const int64_t f0 = fb + lattice_index(n, 2 * i, 2 * j, 2 * k);
-  for (int q = 0; q < comps; ++q) {
-    const T* r = rf + q * Lf.entries;
-    T s = 0;
+  const int32_t tile = Lc.tiles_lin[blockIdx.x];
+  const int nc = Lc.n;
+  const int k = tile >> 20, M = nc - 1 - k;
+  const int t = (tile & 0xFFFFF) + threadIdx.x;
+  if (t >= (M - 1) * M / 2) return;
+  int j, i;
+  slice_decode(M, t, j, i);
+  int nb[NDIR];
+  lattice_neighbours(Lf.n, 2 * i, 2 * j, 2 * k, nb);
+  const T* __restrict__ r = rf + (int64_t)m * Lf.nt;
+  T s[COMPS], o[COMPS];
 #pragma unroll
-    for (int d = 0; d < NDIR; ++d) s += r[fb + lattice_index(n, 2 * i + dir_di(d), 2 * j + dir_dj(d), 2 * k + dir_dk(d))];
-    rc[c + q * Lc.entries] = r[f0] + (T)0.5 * s;
+  for (int q = 0; q < COMPS; ++q) {
+    o[q] = r[nb[0] - 1 + q * Lf.entries];
+    s[q] = 0;
+#pragma unroll
+    for (int d = 0; d < NDIR; ++d) s[q] += r[nb[d] + q * Lf.entries];
   }
+  T* c = rc + (int64_t)m * Lc.nt + lattice_index32(nc, i, j, k);
+#pragma unroll
+  for (int q = 0; q < COMPS; ++q) c[q * Lc.entries] = o[q] + (T)0.5 * s[q];
 }
 
-// coarse skeleton points: precomputed list of unique fine points and weights
-template <typename T>
-__global__ void k_restrict_skeleton(const LevelDev Lc, const int32_t* __restrict__ rptr,
-                                    const int64_t* __restrict__ rent, const T* __restrict__ rw, int64_t Ef,
-                                    const T* __restrict__ rf, T* __restrict__ rc, int comps, int use_dir) {
-  const int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= Lc.nskel) return;
-  T acc[3] = {0, 0, 0};
-  if (!(use_dir && Lc.skel_dir[s])) {
-    for (int q = rptr[s]; q < rptr[s + 1]; ++q) {
+// coarse skeleton points: precomputed list of unique fine points and weights (about 15 per point of a
+// face), 16 lanes to a point: a lane per list walked it one load after the other, 19-26 us a level
+template <typename T, int COMPS>
+__global__ void __launch_bounds__(128)
+    k_restrict_skeleton(const LevelDev Lc, const int32_t* __restrict__ rptr, const int64_t* __restrict__ rent,
+                        const T* __restrict__ rw, int64_t Ef, const T* __restrict__ rf, T* __restrict__ rc,
+                        int use_dir) {
+  const int s = (blockIdx.x * 128 + threadIdx.x) >> 4, lane = threadIdx.x & 15;
+  T acc[COMPS];
+#pragma unroll
+  for (int c = 0; c < COMPS; ++c) acc[c] = 0;
+  if (s < Lc.nskel && !(use_dir && Lc.skel_dir[s])) {
+    for (int q = rptr[s] + lane; q < rptr[s + 1]; q += 16) {
       const int64_t e = rent[q];
       const T w = rw[q];
-      for (int c = 0; c < comps; ++c) acc[c] += w * rf[e + c * Ef];
+#pragma unroll
+      for (int c = 0; c < COMPS; ++c) acc[c] += w * rf[e + c * Ef];
     }
   }
-  for (int q = Lc.skel_ptr[s]; q < Lc.skel_ptr[s + 1]; ++q) {
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+    for (int c = 0; c < COMPS; ++c) acc[c] += __shfl_xor_sync(0xffffffffu, acc[c], o);
+  if (s >= Lc.nskel) return;
+  for (int q = Lc.skel_ptr[s] + lane; q < Lc.skel_ptr[s + 1]; q += 16) {
     const SkelInc I = Lc.skel_inc[q];
-    const int64_t e = (int64_t)I.macro * Lc.nt + lattice_index(Lc.n, I.i, I.j, I.k);
-    for (int c = 0; c < comps; ++c) rc[e + c * Lc.entries] = acc[c];
+    const int64_t e = (int64_t)I.macro * Lc.nt + lattice_index32(Lc.n, I.i, I.j, I.k);
+#pragma unroll
+    for (int c = 0; c < COMPS; ++c) rc[e + c * Lc.entries] = acc[c];
   }
 }
 
@@ -241,14 +261,20 @@ __global__ void k_hash_unique(int64_t U, int comps, const int8_t* __restrict__ u
   }
 }
 
+// a warp per row: a thread per row read its row alone, one cache line per value (0.25 ms for 1029
+// unknowns in FP64)
 template <typename T>
-__global__ void k_dense_matvec(int N, const T* __restrict__ A, const int64_t* __restrict__ idx,
-                               const T* __restrict__ src, T* __restrict__ dst) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+__global__ void __launch_bounds__(128)
+    k_dense_matvec(int N, const T* __restrict__ A, const int64_t* __restrict__ idx, const T* __restrict__ src,
+                   T* __restrict__ dst) {
+  const int i = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (i >= N) return;
   T acc = 0;
-  for (int j = 0; j < N; ++j) acc += A[(int64_t)i * N + j] * src[idx[j]];
-  dst[idx[i]] = acc;
+#pragma unroll 4
+  for (int j = lane; j < N; j += 32) acc += A[(int64_t)i * N + j] * src[idx[j]];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if (lane == 0) dst[idx[i]] = acc;
 }
 
 template <typename T>
@@ -623,8 +649,13 @@ int launch_add_const(int64_t n, T v, T* dst, void* stream) {
 
 template <typename T>
 int launch_prolong_add(const LevelDev& Lf, const LevelDev& Lc, const T* ec, T* ef, void* stream, int comps) {
-  dim3 grid(Lf.ntiles_all, Lf.nmacro);
-  k_prolong_add<T><<<grid, dim3(TILE_I, TILE_J), 0, (cudaStream_t)stream>>>(Lf, Lc, ec, ef, comps);
+  const dim3 grid(Lf.ntiles_all, Lf.nmacro), block(TILE_I, TILE_J);
+  cudaStream_t s = (cudaStream_t)stream;
+  if (comps == 3)
+    k_prolong_add<T, 3><<<grid, block, 0, s>>>(Lf, Lc, ec, ef);
+  else
+    for (int c = 0; c < comps; ++c)
+      k_prolong_add<T, 1><<<grid, block, 0, s>>>(Lf, Lc, ec + c * Lc.entries, ef + c * Lf.entries);
   return (int)cudaGetLastError();
 }
 
@@ -632,13 +663,20 @@ template <typename T>
 int launch_restrict(const LevelDev& Lf, const LevelDev& Lc, const int32_t* rptr, const int64_t* rent, const T* rw,
                     const T* rf, T* rc, void* stream, int comps, int use_dir) {
   cudaStream_t s = (cudaStream_t)stream;
-  if (Lc.ntiles_int > 0) {
-    dim3 grid(Lc.ntiles_int, Lc.nmacro);
-    k_restrict_interior<T><<<grid, dim3(TILE_I, TILE_J), 0, s>>>(Lf, Lc, rf, rc, comps);
+  const dim3 grid(Lc.ntiles_lin, Lc.nmacro);
+  const unsigned nb = (unsigned)(((int64_t)Lc.nskel * 16 + 127) / 128);
+  if (comps == 3) {
+    if (Lc.ntiles_lin > 0) k_restrict_interior<T, 3><<<grid, INTERIOR_BLOCK, 0, s>>>(Lf, Lc, rf, rc);
+    if (Lc.nskel > 0)
+      k_restrict_skeleton<T, 3><<<nb, 128, 0, s>>>(Lc, rptr, rent, rw, Lf.entries, rf, rc, use_dir);
+  } else {
+    for (int c = 0; c < comps; ++c) {
+      const T* f = rf + c * Lf.entries;
+      T* o = rc + c * Lc.entries;
+      if (Lc.ntiles_lin > 0) k_restrict_interior<T, 1><<<grid, INTERIOR_BLOCK, 0, s>>>(Lf, Lc, f, o);
+      if (Lc.nskel > 0) k_restrict_skeleton<T, 1><<<nb, 128, 0, s>>>(Lc, rptr, rent, rw, Lf.entries, f, o, use_dir);
+    }
   }
-  if (Lc.nskel > 0)
-    k_restrict_skeleton<T><<<(Lc.nskel + 127) / 128, 128, 0, s>>>(Lc, rptr, rent, rw, Lf.entries, rf, rc, comps,
-                                                                  use_dir);
   return (int)cudaGetLastError();
 }
 
@@ -728,7 +766,7 @@ int launch_hash_unique(int64_t U, int comps, const int8_t* udir, T* u, void* str
 
 template <typename T>
 int launch_dense_matvec(int N, const T* A, const int64_t* idx, const T* src_u, T* dst_u, void* stream) {
-  k_dense_matvec<T><<<(N + 127) / 128, 128, 0, (cudaStream_t)stream>>>(N, A, idx, src_u, dst_u);
+  k_dense_matvec<T><<<(N + 3) / 4, 128, 0, (cudaStream_t)stream>>>(N, A, idx, src_u, dst_u);
   return (int)cudaGetLastError();
 }
 
