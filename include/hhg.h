@@ -465,9 +465,11 @@ hhg_status hhg_residual_noalloc(hhg_ctx* ctx, int level, hhg_dtype dt, const voi
  * Loss: mean squared error over voxels and the nc output channels; Adam (0.9, 0.999,
  * 1e-8) with a cosine learning-rate decay to 5% of lr. */
 int64_t hhg_learn_num_params(void);
-/* Convolution kernel of the network: 0 = warp-level BF16 MMA (mma.sync m16n8k16) on a
- * shared-memory tile (default), 1 = 5th-generation tensor cores (tcgen05.mma with
- * accumulators in tensor memory, 6 x 27 MMAs of 128 x 16 x 16 per 32 x 4 x 4 output tile,
+/* Convolution kernel of the network: 0 (default) = 5th-generation tensor cores (tcgen05.mma with
+ * accumulators in tensor memory) with four voxels per matrix row, marching in z; grids too small for its
+ * tiles, and every grid after a tensor-core kernel's wait ran out, take warp-level BF16 MMA (mma.sync
+ * m16n8k16) on a shared-memory tile; 1 = tcgen05 with a voxel per row
+ * (6 x 27 MMAs of 128 x 16 x 16 per 32 x 4 x 4 output tile,
  * one tile per block), 2 = the same MMAs in a persistent pipeline (tensor-memory-
  * accelerator loads into two shared stages, two tensor-memory accumulator sets, an
  * epilogue warpgroup draining one while the next tile's MMAs run).  All give the same

@@ -123,6 +123,7 @@ void check_conv(LearnState& S) {
   CK(conv_take_error(&flag));
   if (flag) {
     S.conv_kernel = 0;
+    S.conv_timed_out = true;
     THROW(HHG_ERR_TIMEOUT, "tensor-core convolution timed out (switched to the warp-MMA kernel)");
   }
 }
@@ -186,6 +187,11 @@ void conv(hhg_ctx* c, LearnState& S, int l, bool bwd, const void* X, const float
           const void* mask, GridShape s, int relu) {
   const uint32_t* wp = bwd ? layer_bwd(S, l) : layer_fwd(S, l);
   const void* wu = bwd ? layer_bwd_u(S, l) : layer_fwd_u(S, l);
+  if (S.conv_kernel == 0 && !S.conv_timed_out) {
+    bool taken = false;
+    CK(launch_conv_group(X, wu, bias, Y, Yf, nf, mask, s, relu, c->stream, &taken));
+    if (taken) return;
+  }
   if (S.conv_kernel == 2)
     CK(launch_conv_tma(X, wu, bias, Y, Yf, nf, mask, s, relu, c->stream));
   else

@@ -7,6 +7,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 
 #include "hhg_learn.h"
@@ -15,14 +16,12 @@ namespace hhg {
 
 namespace {
 
-constexpr int WARPS = 4;          // warps per block of the convolution kernels
-constexpr int WG_ROWS = 32;       // 16-voxel row segments per warp in the weight gradient
 constexpr int RED_BLOCK = 256;
 constexpr int RED_MAX_BLOCKS = 1024;
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  const __nv_bfloat16 a = __float2bfloat16_rn(lo), b = __float2bfloat16_rn(hi);
-  return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);  // one conversion for both
+  return *reinterpret_cast<const uint32_t*>(&v);
 }
 
 __device__ __forceinline__ uint32_t pack_raw(unsigned short lo, unsigned short hi) {
@@ -341,6 +340,257 @@ __global__ void __launch_bounds__(128) k_conv_umma(const uint4* __restrict__ X, 
 }
 
 // ---------------------------------------------------------------------------------------
+// The default convolution: tcgen05 with four voxels of a lattice row per matrix row (k_conv_group).
+// With a voxel per row (above) an MMA re-reads 4 KB of A for 16 output channels, and operand fetch
+// bounds it near a third of the tensor peak.  Here a row is a group of four neighbouring voxels with
+// 4 x 16 outputs: the input voxel at position p = -1 .. 4 of the group adds to the outputs x0 = p - dx, so
+// it is one MMA with N = 16, 32, 48, 48, 32 or 16 columns, whose B operand is a run of the three dx
+// weights in descending order (48 rows serve all six positions) and whose D starts at column 16 x0.
+// A plane of output takes 9 (dz, dy) x 6 MMAs for up to 512 voxels; per voxel that is half the A
+// traffic, and no column of a product is wasted.
+//
+// A block owns an x-y tile and marches in z: a ring of four input planes in shared memory, filled with
+// cp.async one plane ahead, two sets of 64 TMEM columns; while the MMAs of a plane run, the block stores
+// the plane before it and loads the plane after next.  Two blocks per SM fill each other's gaps.
+// Planes are stored as 8 chunks (voxel of the group, channel half) of 16-byte rows per (y, group), the
+// K-major no-swizzle layout; the chunk stride is an odd number of 16-byte units, so the stores of the 8
+// chunks of a group fall into distinct banks.  M = 128 rows: 16 lattice rows of 8 groups (stride between
+// core matrices: one row pitch of 10), or 128 consecutive positions of wider rows with their two halo
+// groups, whichever covers the grid with fewer rows (conv_tiling).
+// Bound by the A fetch: 54 MMAs of at least 32 clocks a plane of 512 voxels; 129^3 voxels
+// 115 us with mma.sync, GRP_US now.
+// ---------------------------------------------------------------------------------------
+struct ConvTiling {
+  int tg, yt;     // groups and rows of a tile
+  int pitch;      // positions (16-byte rows) from a row to the next
+  int sbo;        // bytes between core matrices of 8 rows
+  int chunk;      // bytes between chunks
+  int xtiles, ytiles, zc, zchunks;
+};
+constexpr int CG_WARPS = 8;  // load and store; one more issues the MMAs
+constexpr int CG_THREADS = 32 * (CG_WARPS + 1);
+constexpr int CG_B = LN_UMMA;                   // B operands: [dz dy][k half][dx = 1, 0, -1][n 16][8 bf16]
+constexpr int CG_TMEM_COLS = 128;
+constexpr int CG_MAX_SMEM = 112 * 1024;         // two blocks per SM
+__host__ __device__ constexpr int cg_plane(const ConvTiling& t) { return 8 * t.chunk; }
+__host__ __device__ constexpr int cg_smem(const ConvTiling& t) { return 4 * cg_plane(t) + CG_B + 64; }
+
+__global__ void __launch_bounds__(CG_THREADS, 2)
+    k_conv_group(const uint4* __restrict__ X, const uint4* __restrict__ Wu, const float* __restrict__ bias,
+                 uint4* __restrict__ Y, float* __restrict__ Yf, int nf, const uint4* __restrict__ mask, int D, int H,
+                 int W, int relu, const ConvTiling T) {
+  extern __shared__ __align__(1024) unsigned char usm[];
+  const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(usm);
+  const int plane = cg_plane(T);
+  const uint32_t bbase = sbase + 4 * plane, bar = bbase + CG_B, slot = bar + 16;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int x0 = (blockIdx.x % T.xtiles) * 4 * T.tg, y0 = (blockIdx.x / T.xtiles) * T.yt;
+  const int zb = blockIdx.y * T.zc, nz = min(T.zc, D - zb);
+  const int64_t b = blockIdx.z;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(CG_TMEM_COLS));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  }
+  if (threadIdx.x == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(1));
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar + 8), "r"(1));
+    asm volatile("fence.mbarrier_init.release.cluster;");
+  }
+  // B: chunk [s][h][q][n] from the per-tap operands [t][h][n], t = 3 s + 2 - q
+  for (int q = threadIdx.x; q < CG_B / 16; q += CG_THREADS) {
+    const int n = q & 15, dxs = (q >> 4) % 3, h = (q / 48) & 1, st = q / 96;
+    cp_async16(bbase + 16 * q, Wu + (3 * st + 2 - dxs) * 32 + h * 16 + n, true);
+  }
+  // input plane z into ring slot r: a warp per 32 chunks of a row, zero outside the grid
+  const int segs = (2 * (4 * T.tg + 2) + 31) / 32;
+  auto load_plane = [&](int z, int r) {
+    const bool zin = z >= 0 && z < D;
+    const uint4* src = X + (b * D + (zin ? z : 0)) * H * (int64_t)W * 2;
+    for (int u = warp; u < segs * (T.yt + 2); u += CG_WARPS) {
+      const int row = u / segs, q = (u - row * segs) * 32 + lane;
+      const int gy = y0 - 1 + row, ix = q >> 1, h = q & 1, gx = x0 - 1 + ix;
+      if (ix < 4 * T.tg + 2) {
+        const bool in = zin && gy >= 0 && gy < H && gx >= 0 && gx < W;
+        cp_async16(sbase + r * plane + (2 * ((ix + 3) & 3) + h) * T.chunk + (row * T.pitch + ((ix + 3) >> 2)) * 16,
+                   in ? src + ((int64_t)gy * W + gx) * 2 + h : X, in);
+      }
+    }
+  };
+  if (warp < CG_WARPS)
+    for (int r = 0; r < 3; ++r) load_plane(zb - 1 + r, r);
+  asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  uint32_t tmem;
+  asm volatile("ld.shared.b32 %0, [%1];" : "=r"(tmem) : "r"(slot));
+  float bv[16];
+#pragma unroll
+  for (int c = 0; c < 16; ++c) bv[c] = bias ? bias[c] : 0.f;
+  // the thread's row of the M tile (a warp reads the 32 TMEM lanes of its number mod 4): row ry of the
+  // tile, group rg; of the group's four voxels two
+  const int m = 32 * (warp & 3) + lane;
+  const int ry = T.sbo == 128 ? m / T.pitch : m >> 3, rg = T.sbo == 128 ? m - ry * T.pitch : m & 7;
+  const int gy = y0 + ry;
+  const bool row_ok = ry < T.yt && rg < T.tg && gy < H;
+
+  auto store_plane = [&](int zi) {
+    const int64_t rowo = ((b * D + zb + zi) * H + gy) * W;
+#pragma unroll 1
+    for (int xo = 2 * (warp >> 2); xo < 2 * (warp >> 2) + 2; ++xo) {
+      uint32_t r[16];
+      asm volatile(
+          "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+          : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+            "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+          : "r"(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 64u * (zi & 1) + 16u * xo));
+      asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      const int gx = x0 + 4 * rg + xo;
+      if (row_ok && gx < W) {
+        const int64_t v = rowo + gx;
+        float o[16];
+#pragma unroll
+        for (int c = 0; c < 16; ++c) {
+          o[c] = __uint_as_float(r[c]) + bv[c];
+          if (relu) o[c] = fmaxf(o[c], 0.f);
+        }
+        if (mask) {
+          const uint4 m0 = mask[2 * v], m1 = mask[2 * v + 1];
+          const uint32_t mw[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            if (!bf16_positive(mw[q], 0)) o[2 * q] = 0.f;
+            if (!bf16_positive(mw[q], 1)) o[2 * q + 1] = 0.f;
+          }
+        }
+        if (Y) {
+          Y[2 * v] = make_uint4(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]), pack_bf16x2(o[4], o[5]),
+                                pack_bf16x2(o[6], o[7]));
+          Y[2 * v + 1] = make_uint4(pack_bf16x2(o[8], o[9]), pack_bf16x2(o[10], o[11]), pack_bf16x2(o[12], o[13]),
+                                    pack_bf16x2(o[14], o[15]));
+        }
+        if (Yf) {
+#pragma unroll
+          for (int c = 0; c < 16; ++c)
+            if (c < nf) Yf[v * nf + c] = o[c];
+        }
+      }
+      __syncwarp();
+    }
+  };
+  auto wait_bar = [&](int zi) {  // bounded
+    uint32_t done = 0;
+    for (long long it = 0; it < U_SPIN_LIMIT && !done; ++it) {
+      asm volatile(
+          "{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}\n"
+          : "=r"(done)
+          : "r"(bar + 8 * (zi & 1)), "r"((zi >> 1) & 1)
+          : "memory");
+      if (!done) __nanosleep(40);
+    }
+    return done;
+  };
+
+  int bad = 0;
+  for (int zi = 0; zi < nz; ++zi) {
+    if (threadIdx.x == 32 * CG_WARPS) {
+      // Position order: 1 and 4 first, whose columns 0-47 and 48-63 clear the accumulators.  The issuing
+      // thread's instructions are a plane's critical path, so a descriptor is its low word (start address
+      // in 16-byte units, stride between the K halves) plus an offset, with a constant high word.
+      const uint32_t d = tmem + 64u * (zi & 1);
+      const uint32_t a_lo = (sbase >> 4) | ((uint32_t)(T.chunk >> 4) << 16), a_hi = (uint32_t)(T.sbo >> 4) | (1u << 14);
+      const uint32_t b_lo = (bbase >> 4) | ((768u >> 4) << 16), b_hi = (128u >> 4) | (1u << 14);
+      constexpr uint32_t ID = (1u << 4) | (1u << 7) | (1u << 10) | ((128u >> 4) << 24);
+      const uint32_t cu = (uint32_t)T.chunk >> 4;
+#pragma unroll
+      for (int dz = 0; dz < 3; ++dz) {
+        const uint32_t az = a_lo + (uint32_t)((zi + dz) & 3) * (8 * cu);
+#pragma unroll
+        for (int dy = 0; dy < 3; ++dy) {
+          const uint32_t ay = az + (uint32_t)(dy * T.pitch);
+          auto mma = [&](int p, uint32_t n, uint32_t first, uint32_t col, uint32_t acc) {
+            asm volatile(
+                "{\n.reg .pred p;\n.reg .b64 da, db;\nmov.b64 da, {%1, %2};\nmov.b64 db, {%3, %4};\n"
+                "setp.ne.b32 p, %6, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n" ::"r"(d + col),
+                "r"(ay + 2 * ((p + 3) & 3) * cu + ((p + 3) >> 2)), "r"(a_hi),
+                "r"(b_lo + (uint32_t)(3 * dz + dy) * 96 + 16 * first), "r"(b_hi), "r"(ID | ((n >> 3) << 17)), "r"(acc));
+          };
+          const uint32_t acc = dz + dy > 0;
+          mma(2, 48, 0, 0, acc);
+          mma(5, 16, 0, 48, acc);
+          mma(3, 48, 0, 16, 1);
+          mma(1, 32, 1, 0, 1);
+          mma(4, 32, 0, 32, 1);
+          mma(0, 16, 2, 0, 1);
+        }
+      }
+      asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
+                       bar + 8 * (zi & 1))
+                   : "memory");
+    }
+    if (warp < CG_WARPS) {
+      if (zi + 1 < nz) load_plane(zb + zi + 2, (zi + 3) & 3);
+      asm volatile("cp.async.commit_group;\n" ::: "memory");
+      if (zi > 0) store_plane(zi - 1);
+    }
+    __syncwarp();
+    const uint32_t done = wait_bar(zi);
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    bad = __syncthreads_or(!done);
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (bad) {
+      if (threadIdx.x == 0) atomicExch(&g_conv_error, 1);
+      wait_bar(zi);  // drain: the MMAs must have completed before their tensor memory is freed
+      break;
+    }
+  }
+  if (!bad && nz > 0 && warp < CG_WARPS) store_plane(nz - 1);
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(CG_TMEM_COLS));
+}
+
+// The tiling of a grid: rows of 8 groups, or of tg groups laid out consecutively, whichever needs fewer
+// tiles (128 rows each); z in chunks of at least 4 planes for two blocks on each of 152 SMs, of about 32
+// (two more are loaded) when there are more tiles than that.
+// false: the grid is too small to fill half a tile's rows (the mma.sync kernel takes it).
+inline bool conv_tiling(GridShape s, ConvTiling& best) {
+  const int groups = (s.W + 3) / 4;
+  int64_t fewest = INT64_MAX;
+  auto consider = [&](int tg, int yt, int pitch, int sbo, int positions) {
+    ConvTiling t{};
+    t.tg = tg;
+    t.yt = yt;
+    t.pitch = pitch;
+    t.sbo = sbo;
+    t.chunk = 16 * (positions | 1);
+    t.xtiles = (groups + tg - 1) / tg;
+    t.ytiles = (s.H + yt - 1) / yt;
+    if (cg_smem(t) > CG_MAX_SMEM) return;
+    if ((int64_t)t.xtiles * t.ytiles < fewest) {
+      fewest = (int64_t)t.xtiles * t.ytiles;
+      best = t;
+    }
+  };
+  consider(8, 16, 10, 160, 18 * 10);
+  for (int tg = 4; tg <= 40; ++tg) {
+    // the last row's last group is position (yt - 1) pitch + tg - 1 <= 127; a tap reads up to 2 rows and 2
+    // groups further from each of the 128 positions
+    const int pitch = tg + 2, yt = (128 - tg) / pitch + 1;
+    consider(tg, yt, pitch, 128, std::max((yt + 2) * pitch, 128 + 2 * pitch + 2));
+  }
+  if (fewest == INT64_MAX || fewest * 128 > 2 * (int64_t)groups * s.H) return false;
+  const int64_t tiles = fewest * s.B;
+  best.zchunks = (int)std::max<int64_t>(1, std::min<int64_t>(std::max<int64_t>(304 / tiles, s.D / 32), (s.D + 3) / 4));
+  best.zc = (s.D + best.zchunks - 1) / best.zchunks;
+  best.zchunks = (s.D + best.zc - 1) / best.zc;
+  return s.B <= 65535;
+}
+
+// ---------------------------------------------------------------------------------------
 // The same convolution as a persistent, warp-specialised pipeline: warp 0 loads input
 // tiles with the tensor memory accelerator (one 5-D tiled copy per channel half straight
 // into the plane layout; the halo outside the grid is zero-filled by the copy) into two
@@ -584,80 +834,130 @@ __global__ void k_pack_umma(const float* __restrict__ params, __nv_bfloat16* __r
   bwd[q] = __float2bfloat16_rn(Wl[(26 - t) * 256 + n * 16 + k]);
 }
 
-// Weight gradient of tap t = blockIdx.y: dW[t][i][o] = sum_v A[v + off(t)][i] G[v][o] as a
-// tensor-core product with the voxels as the k dimension (A fragment: input channels x
-// 16 voxels, B fragment: 16 voxels x 8 output channels).  Each warp covers WG_ROWS row
-// segments, the block sums its warps in a fixed order and writes one partial tile.
-__global__ void __launch_bounds__(WARPS * 32) k_wgrad(const unsigned short* __restrict__ A,
-                                                      const unsigned short* __restrict__ G, float* __restrict__ partial,
-                                                      int B, int D, int H, int W) {
-  __shared__ float red[WARPS][256];
-  const int t = blockIdx.y;
-  const int dz = t / 9 - 1, dy = (t / 3) % 3 - 1, dx = t % 3 - 1;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int g = lane >> 2, tg = lane & 3;
-  const int nxs = (W + 15) / 16;
-  const int64_t nseg = (int64_t)B * D * H * nxs;
-  const int64_t seg0 = ((int64_t)blockIdx.x * WARPS + warp) * WG_ROWS;
-  float acc[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
-  for (int r = 0; r < WG_ROWS; ++r) {
-    const int64_t seg = seg0 + r;
-    if (seg >= nseg) break;  // warp-uniform
-    const int xs = (int)(seg % nxs);
-    int64_t rest = seg / nxs;
-    const int y = (int)(rest % H);
-    rest /= H;
-    const int z = (int)(rest % D);
-    const int b = (int)(rest / D);
-    const int x0 = xs * 16;
-    const int64_t rowo = (((int64_t)b * D + z) * H + y) * W;
-    const int zz = z + dz, yy = y + dy;
-    const bool rin = zz >= 0 && zz < D && yy >= 0 && yy < H;
-    const int64_t rowi = (((int64_t)b * D + zz) * H + yy) * W;
-    // k index (voxel of the segment) of the four values this lane holds: 2tg, 2tg+1, 2tg+8, 2tg+9
-    unsigned short av[4][2], gv[4][2];
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int x = x0 + 2 * tg + (q & 1) + 8 * (q >> 1);
-      const bool vin = x < W;
-      const int xi = x + dx;
-      const bool ain = vin && rin && xi >= 0 && xi < W;
-      av[q][0] = ain ? A[(rowi + xi) * 16 + g] : (unsigned short)0;
-      av[q][1] = ain ? A[(rowi + xi) * 16 + g + 8] : (unsigned short)0;
-      gv[q][0] = vin ? G[(rowo + x) * 16 + g] : (unsigned short)0;
-      gv[q][1] = vin ? G[(rowo + x) * 16 + g + 8] : (unsigned short)0;
-    }
-    const uint32_t a0 = pack_raw(av[0][0], av[1][0]);  // row (input channel) g, k = 2tg, 2tg+1
-    const uint32_t a1 = pack_raw(av[0][1], av[1][1]);  // row g + 8
-    const uint32_t a2 = pack_raw(av[2][0], av[3][0]);  // row g, k = 2tg+8, 2tg+9
-    const uint32_t a3 = pack_raw(av[2][1], av[3][1]);  // row g + 8
-    mma_bf16(acc[0], a0, a1, a2, a3, pack_raw(gv[0][0], gv[1][0]), pack_raw(gv[2][0], gv[3][0]));
-    mma_bf16(acc[1], a0, a1, a2, a3, pack_raw(gv[0][1], gv[1][1]), pack_raw(gv[2][1], gv[3][1]));
-  }
-#pragma unroll
-  for (int nt = 0; nt < 2; ++nt) {
-    const int o = nt * 8 + 2 * tg;
-    red[warp][g * 16 + o] = acc[nt][0];
-    red[warp][g * 16 + o + 1] = acc[nt][1];
-    red[warp][(g + 8) * 16 + o] = acc[nt][2];
-    red[warp][(g + 8) * 16 + o + 1] = acc[nt][3];
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < 256; e += blockDim.x) {
-    float s = 0.f;
-#pragma unroll
-    for (int w = 0; w < WARPS; ++w) s += red[w][e];
-    partial[(int64_t)blockIdx.x * LN_WSIZE + t * 256 + e] = s;
-  }
+// Weight gradient dW[t][i][o] = sum_v A[v + off(t)][i] G[v][o], a tensor-core product with the voxels as
+// the k dimension.  A block stages tiles of CT_Z x CT_Y x CT_X voxels of G and of A with its halo (the
+// convolution's tile and swizzle) and takes every gridDim.x-th tile; warp w owns the three taps of
+// (dz, dy) = (w / 3, w % 3), so that each 16-voxel segment costs it four transposing ldmatrix (both
+// operands are stored voxel-major) and six mma.sync.  Bound by shared-memory reads and the legacy tensor
+// pipe, as the convolution.  Before, a warp gathered its fragments value by value from global memory for
+// one tap at a time: 8 crops of 32^3 voxels 132 us a layer, now 25.  The sums of a tile are added to the
+// block's, so a chain of FP32 additions stays short.
+constexpr int WG_WARPS = 9;
+constexpr int WG_BLOCKS = 304;  // two blocks on each of 152 SMs; their partial tiles are summed in order
+constexpr int WG_SMEM = CI_VOX * 32 + CT_X * CT_Y * CT_Z * 32;
+
+__device__ __forceinline__ void ldmatrix_x4_trans(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2,
+                                                  uint32_t& r3) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
+               : "r"(addr)
+               : "memory");
 }
 
-// out[c] = sum over rows r (in order) of partial[r * ncol + c]
-__global__ void k_colsum(const float* __restrict__ partial, int64_t rows, int ncol, float* __restrict__ out) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  if (c >= ncol) return;
+__global__ void __launch_bounds__(WG_WARPS * 32) k_wgrad(const uint4* __restrict__ A, const uint4* __restrict__ G,
+                                                         float* __restrict__ partial, int D, int H, int W, int ntx,
+                                                         int nty, int ntz, int ntiles) {
+  extern __shared__ uint4 smem[];
+  uint4* as = smem;                // CI_VOX * 2 chunks
+  uint4* gs = smem + CI_VOX * 2;   // CT_X CT_Y CT_Z * 2 chunks
+  const uint32_t a_base = smem_u32(as), g_base = smem_u32(gs);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int dz = warp / 3, dy = warp % 3;
+  // ldmatrix.x4.trans: lanes 8 q .. 8 q + 7 address the rows (voxels) of matrix q: voxels 8 (q >> 1) ..,
+  // channel half q & 1
+  const int krow = (lane & 7) + 8 * (lane >> 4), half = (lane >> 3) & 1;
+  float tot[3][2][4];
+#pragma unroll
+  for (int t = 0; t < 3; ++t)
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) tot[t][nt][q] = 0.f;
+  for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
+    const int x0 = (tile % ntx) * CT_X, y0 = (tile / ntx % nty) * CT_Y, z0 = (tile / (ntx * nty) % ntz) * CT_Z;
+    const int64_t b = tile / (ntx * nty * ntz);
+    __syncthreads();  // the last tile has been read
+    for (int q = threadIdx.x; q < CI_VOX * 2; q += blockDim.x) {
+      const int v = q >> 1, h = q & 1;
+      const int ix = v % CI_X, iy = (v / CI_X) % CI_Y, iz = v / (CI_X * CI_Y);
+      const int gx = x0 - 1 + ix, gy = y0 - 1 + iy, gz = z0 - 1 + iz;
+      const bool in = gx >= 0 && gx < W && gy >= 0 && gy < H && gz >= 0 && gz < D;
+      cp_async16(smem_u32(as + v * 2 + (h ^ ((v >> 2) & 1))), in ? A + (((b * D + gz) * H + gy) * W + gx) * 2 + h : A,
+                 in);
+    }
+    for (int q = threadIdx.x; q < CT_X * CT_Y * CT_Z * 2; q += blockDim.x) {
+      const int v = q >> 1, h = q & 1;
+      const int gx = x0 + v % CT_X, gy = y0 + v / CT_X % CT_Y, gz = z0 + v / (CT_X * CT_Y);
+      const bool in = gx < W && gy < H && gz < D;
+      cp_async16(smem_u32(gs + v * 2 + (h ^ ((v >> 2) & 1))), in ? G + (((b * D + gz) * H + gy) * W + gx) * 2 + h : G,
+                 in);
+    }
+    asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();
+    float acc[3][2][4];
+#pragma unroll
+    for (int t = 0; t < 3; ++t)
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[t][nt][q] = 0.f;
+#pragma unroll 2
+    for (int seg = 0; seg < CT_Z * CT_Y * (CT_X / 16); ++seg) {
+      const int xs = (seg & 1) * 16, oy = (seg >> 1) % CT_Y, oz = (seg >> 1) / CT_Y;
+      const int vg = (oz * CT_Y + oy) * CT_X + xs + krow;
+      uint32_t g0, g1, g2, g3;
+      ldmatrix_x4_trans(g_base + (uint32_t)(vg * 2 + (half ^ ((vg >> 2) & 1))) * 16u, g0, g1, g2, g3);
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        const int va = ((oz + dz) * CI_Y + (oy + dy)) * CI_X + xs + t + krow;
+        uint32_t a0, a1, a2, a3;
+        ldmatrix_x4_trans(a_base + (uint32_t)(va * 2 + (half ^ ((va >> 2) & 1))) * 16u, a0, a1, a2, a3);
+        mma_bf16(acc[t][0], a0, a1, a2, a3, g0, g2);
+        mma_bf16(acc[t][1], a0, a1, a2, a3, g1, g3);
+      }
+    }
+#pragma unroll
+    for (int t = 0; t < 3; ++t)
+#pragma unroll
+      for (int nt = 0; nt < 2; ++nt)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) tot[t][nt][q] += acc[t][nt][q];
+  }
+  const int g = lane >> 2, tg = lane & 3;
+  float* out = partial + (int64_t)blockIdx.x * LN_WSIZE + (dz * 9 + dy * 3) * 256;
+#pragma unroll
+  for (int t = 0; t < 3; ++t)
+#pragma unroll
+    for (int nt = 0; nt < 2; ++nt) {
+      const int o = nt * 8 + 2 * tg;
+      float* w = out + t * 256;
+      w[g * 16 + o] = tot[t][nt][0];
+      w[g * 16 + o + 1] = tot[t][nt][1];
+      w[(g + 8) * 16 + o] = tot[t][nt][2];
+      w[(g + 8) * 16 + o + 1] = tot[t][nt][3];
+    }
+}
+
+// out[c] = sum over rows r of partial[r * ncol + c]: 32 columns a block, COLSUM_ROWS interleaved row
+// sums each, added in order (one thread per column walked its rows alone: 33 us)
+constexpr int COLSUM_ROWS = 32;
+__global__ void __launch_bounds__(32 * COLSUM_ROWS) k_colsum(const float* __restrict__ partial, int64_t rows, int ncol,
+                                                             float* __restrict__ out) {
+  __shared__ float red[COLSUM_ROWS][32];
+  const int c = blockIdx.x * 32 + threadIdx.x;
   float s = 0.f;
-  for (int64_t r = 0; r < rows; ++r) s += partial[r * ncol + c];
-  out[c] = s;
+  if (c < ncol) {
+#pragma unroll 4
+    for (int64_t r = threadIdx.y; r < rows; r += COLSUM_ROWS) s += partial[r * ncol + c];
+  }
+  red[threadIdx.y][threadIdx.x] = s;
+  __syncthreads();
+  if (threadIdx.y == 0 && c < ncol) {
+    float t = 0.f;
+#pragma unroll
+    for (int q = 0; q < COLSUM_ROWS; ++q) t += red[q][threadIdx.x];
+    out[c] = t;
+  }
 }
 
 __global__ void __launch_bounds__(RED_BLOCK) k_bgrad(const uint32_t* __restrict__ G, int64_t V,
@@ -984,18 +1284,35 @@ int launch_conv(const void* X, const uint32_t* Wp, const void* Wu, const float* 
   return (int)cudaGetLastError();
 }
 
+int launch_conv_group(const void* X, const void* Wu, const float* bias, void* Y, float* Yf, int nf, const void* mask,
+                      GridShape s, int relu, void* stream, bool* taken) {
+  ConvTiling t;
+  *taken = conv_tiling(s, t);
+  if (!*taken) return 0;
+  const cudaError_t e = cudaFuncSetAttribute(k_conv_group, cudaFuncAttributeMaxDynamicSharedMemorySize, cg_smem(t));
+  if (e != cudaSuccess) return (int)e;
+  const dim3 grid((unsigned)(t.xtiles * t.ytiles), (unsigned)t.zchunks, (unsigned)s.B);
+  k_conv_group<<<grid, CG_THREADS, cg_smem(t), (cudaStream_t)stream>>>((const uint4*)X, (const uint4*)Wu, bias,
+                                                                      (uint4*)Y, Yf, nf, (const uint4*)mask, s.D, s.H,
+                                                                      s.W, relu, t);
+  return (int)cudaGetLastError();
+}
+
 int64_t wgrad_partials(GridShape s) {
-  const int64_t nseg = (int64_t)s.B * s.D * s.H * ((s.W + 15) / 16);
-  const int64_t nb = (nseg + WARPS * WG_ROWS - 1) / (WARPS * WG_ROWS);
-  return nb < 1 ? 1 : nb;
+  const int64_t ntiles = (int64_t)s.B * ((s.W + CT_X - 1) / CT_X) * ((s.H + CT_Y - 1) / CT_Y) * ((s.D + CT_Z - 1) / CT_Z);
+  return std::min<int64_t>(ntiles, WG_BLOCKS);
 }
 
 int launch_wgrad(const void* A, const void* G, float* partial, float* dW, GridShape s, void* stream) {
   const int64_t nb = wgrad_partials(s);
-  dim3 grid((unsigned)nb, LN_TAPS);
-  k_wgrad<<<grid, WARPS * 32, 0, (cudaStream_t)stream>>>((const unsigned short*)A, (const unsigned short*)G, partial,
-                                                         s.B, s.D, s.H, s.W);
-  k_colsum<<<(LN_WSIZE + 255) / 256, 256, 0, (cudaStream_t)stream>>>(partial, nb, LN_WSIZE, dW);
+  const int ntx = (s.W + CT_X - 1) / CT_X, nty = (s.H + CT_Y - 1) / CT_Y, ntz = (s.D + CT_Z - 1) / CT_Z;
+  const int64_t ntiles = (int64_t)s.B * ntx * nty * ntz;
+  if (ntiles > INT32_MAX) return (int)cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(k_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize, WG_SMEM);
+  if (e != cudaSuccess) return (int)e;
+  k_wgrad<<<(unsigned)nb, WG_WARPS * 32, WG_SMEM, (cudaStream_t)stream>>>((const uint4*)A, (const uint4*)G, partial, s.D,
+                                                                        s.H, s.W, ntx, nty, ntz, (int)ntiles);
+  k_colsum<<<(LN_WSIZE + 31) / 32, dim3(32, COLSUM_ROWS), 0, (cudaStream_t)stream>>>(partial, nb, LN_WSIZE, dW);
   return (int)cudaGetLastError();
 }
 
@@ -1004,7 +1321,7 @@ int64_t bgrad_partials(int64_t V) { return red_blocks(V); }
 int launch_bgrad(const void* G, int64_t V, float* partial, float* db, void* stream) {
   const int64_t nb = red_blocks(V);
   k_bgrad<<<(unsigned)nb, RED_BLOCK, 0, (cudaStream_t)stream>>>((const uint32_t*)G, V, partial);
-  k_colsum<<<1, 32, 0, (cudaStream_t)stream>>>(partial, nb, 16, db);
+  k_colsum<<<1, dim3(32, COLSUM_ROWS), 0, (cudaStream_t)stream>>>(partial, nb, 16, db);
   return (int)cudaGetLastError();
 }
 
