@@ -231,9 +231,9 @@ __global__ void __launch_bounds__(GSM_BLOCK) k_gs_macro(const LevelDev L, const 
 
 constexpr int GS_MAX_MACROS = 65535;  // grid.y
 
-// Which form: measured with 48 macros in FP64, one smoothing step (8 colours): 8 intervals per macro
-// edge (210 points per colour) 14 us in one launch against 52 in eight, 16 (2730) 36 against 60, 32
-// (27,000) 310 against 235.
+// Which form, by points of a colour over all macros.  48 macros in FP64, a whole smoothing step (skeleton
+// rows and 8 colours): 8 intervals per macro edge (210 points) 68-72 us in one launch against 197 in
+// eight, 16 (2730) 113-119 against 205, 32 (27,000) 581 against 322.
 constexpr int64_t GS_MACRO_MAX_POINTS = 12000;
 
 }  // namespace

@@ -793,7 +793,7 @@ hhg_status hhg_learn_init(hhg_ctx* c, uint64_t seed) {
 
 hhg_status hhg_learn_set_conv_kernel(hhg_ctx* c, int kernel) {
   return guard(c, [&] {
-    if (kernel < 0 || kernel > 2) THROW(HHG_ERR_ARG, "conv kernel 0 (warp MMA), 1 (tcgen05) or 2 (TMA + tcgen05)");
+    if (kernel < 0 || kernel > 2) THROW(HHG_ERR_ARG, "conv kernel 0 (default), 1 (tcgen05) or 2 (TMA + tcgen05)");
     state(c).conv_kernel = kernel;
   });
 }

@@ -18,8 +18,8 @@
 //
 // What bounds them: latency, and on meshes of many macros instructions.  There are few such nodes (2 % of
 // 129^3), but most of a face's or edge's neighbours lie in different rows.  FP32 apply on 384 macros at
-// level 5, rows alone: one unrolled kernel per node 93 + 62 us, the general form with run-time rings 73,
-// this one 64 (half a warp per incidence of an edge's nodes: 90).
+// level 5, whole sweep: 209 us with an unrolled kernel per node kind (rows 93 + 62), 112 with this layout
+// (160 with half a warp per incidence for the nodes of edges too).
 #pragma once
 #include <cuda_runtime.h>
 
