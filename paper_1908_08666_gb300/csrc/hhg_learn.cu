@@ -435,6 +435,13 @@ __global__ void __launch_bounds__(CG_THREADS, 2)
   const int gy = y0 + ry;
   const bool row_ok = ry < T.yt && rg < T.tg && gy < H;
 
+  auto clear = [&](uint32_t col) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], {%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1,%1};" ::"r"(
+            tmem + ((uint32_t)(32 * (warp & 3)) << 16) + col),
+        "r"(0));
+  };
+  // writes a plane and clears its accumulators for the plane after next
   auto store_plane = [&](int zi) {
     const int64_t rowo = ((b * D + zb + zi) * H + gy) * W;
 #pragma unroll 1
@@ -446,6 +453,7 @@ __global__ void __launch_bounds__(CG_THREADS, 2)
             "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
           : "r"(tmem + ((uint32_t)(32 * (warp & 3)) << 16) + 64u * (zi & 1) + 16u * xo));
       asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      clear(64u * (zi & 1) + 16u * xo);
       const int gx = x0 + 4 * rg + xo;
       if (row_ok && gx < W) {
         const int64_t v = rowo + gx;
@@ -478,6 +486,7 @@ __global__ void __launch_bounds__(CG_THREADS, 2)
       }
       __syncwarp();
     }
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
   };
   auto wait_bar = [&](int zi) {  // bounded
     uint32_t done = 0;
@@ -492,11 +501,19 @@ __global__ void __launch_bounds__(CG_THREADS, 2)
     return done;
   };
 
+  if (warp < CG_WARPS) {
+    for (int q = 0; q < 4; ++q) clear(64u * (q & 1) + 16u * (2 * (warp >> 2) + (q >> 1)));
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+
   int bad = 0;
   for (int zi = 0; zi < nz; ++zi) {
     if (threadIdx.x == 32 * CG_WARPS) {
-      // Position order: 1 and 4 first, whose columns 0-47 and 48-63 clear the accumulators.  The issuing
-      // thread's instructions are a plane's critical path, so a descriptor is its low word (start address
+      // Positions in ascending order, so that every output sums its 27 taps in the order of the kernels
+      // above; the accumulators start from the zeros of clear().  The issuing thread's instructions are a plane's critical path, so a descriptor is its low word (start address
       // in 16-byte units, stride between the K halves) plus an offset, with a constant high word.
       const uint32_t d = tmem + 64u * (zi & 1);
       const uint32_t a_lo = (sbase >> 4) | ((uint32_t)(T.chunk >> 4) << 16), a_hi = (uint32_t)(T.sbo >> 4) | (1u << 14);
@@ -509,20 +526,19 @@ __global__ void __launch_bounds__(CG_THREADS, 2)
 #pragma unroll
         for (int dy = 0; dy < 3; ++dy) {
           const uint32_t ay = az + (uint32_t)(dy * T.pitch);
-          auto mma = [&](int p, uint32_t n, uint32_t first, uint32_t col, uint32_t acc) {
+          auto mma = [&](int p, uint32_t n, uint32_t first, uint32_t col) {
             asm volatile(
                 "{\n.reg .pred p;\n.reg .b64 da, db;\nmov.b64 da, {%1, %2};\nmov.b64 db, {%3, %4};\n"
-                "setp.ne.b32 p, %6, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n" ::"r"(d + col),
+                "setp.eq.b32 p, 0, 0;\ntcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %5, p;\n}\n" ::"r"(d + col),
                 "r"(ay + 2 * ((p + 3) & 3) * cu + ((p + 3) >> 2)), "r"(a_hi),
-                "r"(b_lo + (uint32_t)(3 * dz + dy) * 96 + 16 * first), "r"(b_hi), "r"(ID | ((n >> 3) << 17)), "r"(acc));
+                "r"(b_lo + (uint32_t)(3 * dz + dy) * 96 + 16 * first), "r"(b_hi), "r"(ID | ((n >> 3) << 17)));
           };
-          const uint32_t acc = dz + dy > 0;
-          mma(2, 48, 0, 0, acc);
-          mma(5, 16, 0, 48, acc);
-          mma(3, 48, 0, 16, 1);
-          mma(1, 32, 1, 0, 1);
-          mma(4, 32, 0, 32, 1);
-          mma(0, 16, 2, 0, 1);
+          mma(0, 16, 2, 0);
+          mma(1, 32, 1, 0);
+          mma(2, 48, 0, 0);
+          mma(3, 48, 0, 16);
+          mma(4, 32, 0, 32);
+          mma(5, 16, 0, 48);
         }
       }
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(

@@ -45,3 +45,23 @@ def test_gradients_at_tile_edges(ctx, shape):  # noqa: F811
     for l in range(4):
         assert np.linalg.norm(gW[l] - dWs[l]) <= 2e-2 * np.linalg.norm(dWs[l]), l
         assert np.linalg.norm(gb[l] - dbs[l]) <= 2e-2 * np.linalg.norm(dbs[l]) + 1e-12, l
+
+
+@pytest.mark.parametrize("shape", [(1, 5, 16, 32), (2, 6, 33, 66), (1, 33, 20, 129)])
+def test_every_kernel_sums_in_the_same_order(ctx, shape):  # noqa: F811
+    """A hidden activation is rounded to BF16, so another order of the sums shows in the outputs: the three
+    kernels agree to the last bit."""
+    t = ctx.torch
+    Ws, bs = _params(6)
+    B.hhg_learn_set_params(ctx.h, _flat(Ws, bs))
+    x = ctx.dev(np.random.default_rng(sum(shape)).normal(size=shape + (LN.CIN,)), t.float32)
+    outs = []
+    try:
+        for kernel in (0, 1, 2):
+            B.hhg_learn_set_conv_kernel(ctx.h, kernel)
+            outs.append(t.empty(shape + (LN.COUT,), dtype=t.float32, device="cuda"))
+            B.hhg_learn_forward(ctx.h, x, LN.CIN, *shape, outs[-1], LN.COUT)
+        t.cuda.synchronize()
+    finally:
+        B.hhg_learn_set_conv_kernel(ctx.h, 0)
+    assert t.equal(outs[0], outs[1]) and t.equal(outs[0], outs[2])
