@@ -129,7 +129,7 @@ struct CarreauParams {
   double eta0, eta_inf, kappa, r;
 };
 struct SlopeOp {
-  double Q[NDIR][3];
+  double Q[7][3];
 };
 struct PatchLists {
   int32_t nnodes;

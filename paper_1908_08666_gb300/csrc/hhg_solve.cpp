@@ -934,15 +934,20 @@ void carreau_setup(hhg_ctx* c, int l) {
   };
   L.slope.resize(M);
   for (int m = 0; m < M; ++m) {
-    double dx[NDIR][3], G[3][3] = {{0}};
-    double o[3];
-    phys(m, 0, 0, 0, o);
-    for (int d = 0; d < NDIR; ++d) {
-      double q[3];
-      phys(m, dir_di(d), dir_dj(d), dir_dk(d), q);
-      for (int a = 0; a < 3; ++a) dx[d][a] = q[a] - o[a];
+    // direction d and its opposite: dx and -dx, so a pair adds 2 dx dx^T to G
+    const Vec3d& v0 = c->xyz[c->tets[m][0]];
+    double dx[7][3], G[3][3] = {{0}};
+    for (int d = 0; d < 7; ++d) {
+      for (int a = 0; a < 3; ++a) dx[d][a] = 0.0;
+      const int o[3] = {dir_di(d), dir_dj(d), dir_dk(d)};
+      for (int b = 0; b < 3; ++b) {
+        const Vec3d& v = c->xyz[c->tets[m][1 + b]];
+        dx[d][0] += o[b] * (v.x - v0.x) / n;
+        dx[d][1] += o[b] * (v.y - v0.y) / n;
+        dx[d][2] += o[b] * (v.z - v0.z) / n;
+      }
       for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) G[a][b] += dx[d][a] * dx[d][b];
+        for (int b = 0; b < 3; ++b) G[a][b] += 2.0 * dx[d][a] * dx[d][b];
     }
     // G^{-1} by cofactors
     const double det = G[0][0] * (G[1][1] * G[2][2] - G[1][2] * G[2][1]) -
@@ -958,7 +963,7 @@ void carreau_setup(hhg_ctx* c, int l) {
     Gi[2][0] = (G[1][0] * G[2][1] - G[1][1] * G[2][0]) / det;
     Gi[2][1] = (G[0][1] * G[2][0] - G[0][0] * G[2][1]) / det;
     Gi[2][2] = (G[0][0] * G[1][1] - G[0][1] * G[1][0]) / det;
-    for (int d = 0; d < NDIR; ++d)
+    for (int d = 0; d < 7; ++d)
       for (int a = 0; a < 3; ++a)
         L.slope[m].Q[d][a] = Gi[a][0] * dx[d][0] + Gi[a][1] * dx[d][1] + Gi[a][2] * dx[d][2];
   }
