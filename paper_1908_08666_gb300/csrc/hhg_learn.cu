@@ -20,7 +20,13 @@ constexpr int RED_BLOCK = 256;
 constexpr int RED_MAX_BLOCKS = 1024;
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
-  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);  // one conversion for both
+  const __nv_bfloat16 a = __float2bfloat16_rn(lo), b = __float2bfloat16_rn(hi);
+  return (uint32_t)__bfloat16_as_ushort(a) | ((uint32_t)__bfloat16_as_ushort(b) << 16);
+}
+
+// the same values with one conversion for both
+__device__ __forceinline__ uint32_t pack_pair(float lo, float hi) {
+  const __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
@@ -473,10 +479,10 @@ __global__ void __launch_bounds__(CG_THREADS, 2)
           }
         }
         if (Y) {
-          Y[2 * v] = make_uint4(pack_bf16x2(o[0], o[1]), pack_bf16x2(o[2], o[3]), pack_bf16x2(o[4], o[5]),
-                                pack_bf16x2(o[6], o[7]));
-          Y[2 * v + 1] = make_uint4(pack_bf16x2(o[8], o[9]), pack_bf16x2(o[10], o[11]), pack_bf16x2(o[12], o[13]),
-                                    pack_bf16x2(o[14], o[15]));
+          Y[2 * v] = make_uint4(pack_pair(o[0], o[1]), pack_pair(o[2], o[3]), pack_pair(o[4], o[5]),
+                                pack_pair(o[6], o[7]));
+          Y[2 * v + 1] = make_uint4(pack_pair(o[8], o[9]), pack_pair(o[10], o[11]), pack_pair(o[12], o[13]),
+                                    pack_pair(o[14], o[15]));
         }
         if (Yf) {
 #pragma unroll
@@ -572,8 +578,16 @@ __global__ void __launch_bounds__(CG_THREADS, 2)
 // The tiling of a grid: rows of 8 groups, or of tg groups laid out consecutively, whichever needs fewer
 // tiles (128 rows each); z in chunks of at least 4 planes for two blocks on each of 152 SMs, of about 32
 // (two more are loaded) when there are more tiles than that.
-// false: the grid is too small to fill half a tile's rows (the mma.sync kernel takes it).
+// false (the mma.sync kernel takes the grid): less than half of the tiles' rows would be filled, or k_conv
+// needs at most three of its blocks per SM.  On such grids the marches do not fill the chip and their time
+// stays at 81-90 us for four layers, where k_conv's grows with its blocks: forward pass, us, k_conv / this
+// kernel: 17^3 voxels (25 blocks) 57 / 81, 33^3 (162) 66 / 82, 129 x 33 x 32 (297) 73 / 90, 49^3 (338)
+// 82 / 83, 300 x 21^2 (450) 82 / 83; 5 x 160 x 165 (480) 92 / 81, 65^2 x 33 (578) 98 / 84, 65^3 (867)
+// 124 / 107.
+constexpr int64_t CG_MIN_BLOCKS = 3 * 152;
 inline bool conv_tiling(GridShape s, ConvTiling& best) {
+  const int64_t conv_blocks = (int64_t)((s.W + CT_X - 1) / CT_X) * ((s.H + CT_Y - 1) / CT_Y) * ((s.D + CT_Z - 1) / CT_Z) * s.B;
+  if (conv_blocks <= CG_MIN_BLOCKS) return false;
   const int groups = (s.W + 3) / 4;
   int64_t fewest = INT64_MAX;
   auto consider = [&](int tg, int yt, int pitch, int sbo, int positions) {

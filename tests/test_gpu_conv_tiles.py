@@ -13,7 +13,13 @@ from test_gpu_learned import _flat, _params, _unflat, ctx  # noqa: F401  (module
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("shape", [(1, 5, 16, 32), (1, 3, 17, 33), (2, 6, 33, 66), (1, 33, 20, 129), (1, 1, 11, 36)])
+# grids under and over the size (456 tiles of 4 x 4 x 32 voxels) from which the default is the grouped
+# tcgen05 kernel
+SMALL = [(1, 5, 16, 32), (1, 3, 17, 33), (2, 6, 33, 66), (1, 33, 20, 129), (1, 1, 11, 36)]
+LARGE = [(1, 29, 65, 127), (1, 33, 65, 66), (2, 16, 129, 65), (1, 5, 160, 165), (8, 31, 31, 32), (1, 2, 256, 257)]
+
+
+@pytest.mark.parametrize("shape", SMALL + LARGE)
 def test_forward_at_tile_edges(ctx, shape):  # noqa: F811
     t = ctx.torch
     B.hhg_learn_set_conv_kernel(ctx.h, 0)
@@ -29,7 +35,7 @@ def test_forward_at_tile_edges(ctx, shape):  # noqa: F811
     assert np.linalg.norm(got - want) <= 3e-3 * np.linalg.norm(want)
 
 
-@pytest.mark.parametrize("shape", [(1, 5, 16, 32), (1, 3, 17, 33), (2, 6, 33, 66)])
+@pytest.mark.parametrize("shape", SMALL[:3] + [(1, 29, 65, 127)])
 def test_gradients_at_tile_edges(ctx, shape):  # noqa: F811
     t = ctx.torch
     B.hhg_learn_set_conv_kernel(ctx.h, 0)
@@ -47,7 +53,7 @@ def test_gradients_at_tile_edges(ctx, shape):  # noqa: F811
         assert np.linalg.norm(gb[l] - dbs[l]) <= 2e-2 * np.linalg.norm(dbs[l]) + 1e-12, l
 
 
-@pytest.mark.parametrize("shape", [(1, 5, 16, 32), (2, 6, 33, 66), (1, 33, 20, 129)])
+@pytest.mark.parametrize("shape", SMALL + LARGE)
 def test_every_kernel_sums_in_the_same_order(ctx, shape):  # noqa: F811
     """A hidden activation is rounded to BF16, so another order of the sums shows in the outputs: the three
     kernels agree to the last bit."""
