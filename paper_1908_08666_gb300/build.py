@@ -13,11 +13,14 @@ CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT, "libhhgs.so")
 
-SOURCES = ["hhg_host.cpp", "hhg_solve.cpp", "hhg_learn.cpp", "hhg_sweep.cu", "hhg_sweep_f32.cu", "hhg_sweep_f64.cu", "hhg_stokes_f32.cu", "hhg_stokes_f64.cu",
-           "hhg_rows_f32.cu", "hhg_rows_f64.cu", "hhg_gs.cu", "hhg_vec.cu", "hhg_learn.cu",
-           "hhg_twod.cu"]
+# many instantiations of unrolled kernels: ptxas in parallel.  Not for the other files: parallel ptxas made
+# the mma.sync convolution slower (forward pass on 33^3 voxels 65 -> 71 us).
+SPLIT = ["hhg_sweep_f32.cu", "hhg_sweep_f64.cu", "hhg_stokes_f32.cu", "hhg_stokes_f64.cu", "hhg_rows_f32.cu",
+         "hhg_rows_f64.cu"]
+SOURCES = ["hhg_host.cpp", "hhg_solve.cpp", "hhg_learn.cpp", "hhg_sweep.cu", "hhg_gs.cu", "hhg_vec.cu", "hhg_learn.cu",
+           "hhg_twod.cu", *SPLIT]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
-FLAGS = ["-O3", "--split-compile", "0", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC,-O2",
+FLAGS = ["-O3", "-lineinfo", "-std=c++17", "--expt-relaxed-constexpr", "-Xcompiler", "-fPIC,-O2",
          "-I" + os.path.join(os.path.dirname(HERE), "include")]
 
 
@@ -30,7 +33,8 @@ def nvcc():
 
 def _compile(src, extra):
     obj = os.path.join(OUT, src + ".o")
-    cmd = [nvcc(), *ARCH, *FLAGS, *extra, "-c", os.path.join(CSRC, src), "-o", obj]
+    split = ["--split-compile", "0"] if src in SPLIT else []
+    cmd = [nvcc(), *ARCH, *FLAGS, *split, *extra, "-c", os.path.join(CSRC, src), "-o", obj]
     r = subprocess.run(cmd, capture_output=True, text=True)
     if r.returncode != 0:
         raise RuntimeError("nvcc failed for %s:\n%s\n%s" % (src, " ".join(cmd), r.stderr))
