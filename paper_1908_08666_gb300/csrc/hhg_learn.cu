@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(128) k_conv_umma(const uint4* __restrict__ X, 
 // core matrices: one row pitch of 10), or 128 consecutive positions of wider rows with their two halo
 // groups, whichever covers the grid with fewer rows (conv_tiling).
 // Bound by the A fetch: 54 MMAs of at least 32 clocks a plane of 512 voxels; 129^3 voxels
-// 115 us with mma.sync, 65 with this kernel.
+// 115 us with mma.sync, 63 with this kernel (ncu, cold).
 // ---------------------------------------------------------------------------------------
 struct ConvTiling {
   int tg, yt;     // groups and rows of a tile
