@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 
 #include "hhg_learn.h"
@@ -1319,8 +1320,18 @@ int launch_conv_group(const void* X, const void* Wu, const float* bias, void* Y,
   ConvTiling t;
   *taken = conv_tiling(s, t);
   if (!*taken) return 0;
-  const cudaError_t e = cudaFuncSetAttribute(k_conv_group, cudaFuncAttributeMaxDynamicSharedMemorySize, cg_smem(t));
+  // The limit belongs to the function on this device and not to the launch: set to the bound of every
+  // tiling, once, so that no thread lowers it between another one's setting and its launch.
+  static std::atomic<bool> gattr[64] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return (int)e;
+  if (dev < 0 || dev >= 64) return (int)cudaErrorInvalidDevice;
+  if (!gattr[dev].load(std::memory_order_acquire)) {
+    e = cudaFuncSetAttribute(k_conv_group, cudaFuncAttributeMaxDynamicSharedMemorySize, CG_MAX_SMEM);
+    if (e != cudaSuccess) return (int)e;
+    gattr[dev].store(true, std::memory_order_release);
+  }
   const dim3 grid((unsigned)(t.xtiles * t.ytiles), (unsigned)t.zchunks, (unsigned)s.B);
   k_conv_group<<<grid, CG_THREADS, cg_smem(t), (cudaStream_t)stream>>>((const uint4*)X, (const uint4*)Wu, bias,
                                                                       (uint4*)Y, Yf, nf, (const uint4*)mask, s.D, s.H,

@@ -1,0 +1,79 @@
+"""Network convolutions of two contexts from two host threads: what belongs to a device as a whole must not
+pass from one context's calls to the other's."""
+
+import threading
+
+import numpy as np
+import pytest
+
+import hhg_inputs as hi
+from paper_1908_08666_gb300 import binding as B
+
+from hhg_gpu import torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+
+class Net:
+    """A context with a network on a stream of its own, and an input."""
+
+    def __init__(self, seed, shape):
+        self.torch = t = torch_cuda()
+        self.stream = t.cuda.Stream()
+        self.shape = shape
+        self.h = B.hhg_create(0, self.stream.cuda_stream)
+        xyz, tets = hi.unit_tet()
+        B.hhg_set_macro_mesh(self.h, xyz, tets)
+        B.hhg_refine(self.h, 2)
+        B.hhg_set_problem(self.h)
+        B.hhg_learn_init(self.h, seed)
+        self.x = t.as_tensor(np.random.default_rng(seed).normal(size=shape + (7,)), dtype=t.float32, device="cuda")
+        self.out = t.empty(shape + (3,), dtype=t.float32, device="cuda")
+        t.cuda.synchronize()
+
+    def forward(self):
+        B.hhg_learn_forward(self.h, self.x, 7, *self.shape, self.out)
+
+    def close(self):
+        B.hhg_destroy(self.h)
+
+
+def _together(*loops):
+    """Runs the functions in a thread each, starting together; returns what they raised."""
+    errors, gate = [], threading.Barrier(len(loops))
+
+    def body(f):
+        gate.wait()
+        try:
+            f()
+        except BaseException as e:  # noqa: BLE001  (reported by the caller)
+            errors.append(e)
+
+    threads = [threading.Thread(target=body, args=(f,)) for f in loops]
+    for th in threads:
+        th.start()
+    for th in threads:
+        th.join()
+    return errors
+
+
+def test_grids_of_different_tilings_from_two_threads():
+    """Grids whose tiles take 104 and 85 KB of shared memory: the limit that one launch needs is not lowered
+    by the other context's."""
+    nets = [Net(1, (8, 31, 31, 32)), Net(2, (24, 16, 20, 16))]
+    try:
+        want = []
+        for net in nets:
+            net.forward()
+            want.append(net.out.clone())
+
+        def loop(net):
+            for _ in range(400):
+                net.forward()
+
+        assert _together(*(lambda net=net: loop(net) for net in nets)) == []
+        for net, w in zip(nets, want):
+            assert net.torch.equal(net.out, w)
+    finally:
+        for net in nets:
+            net.close()
