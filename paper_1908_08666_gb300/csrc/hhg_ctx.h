@@ -193,6 +193,12 @@ struct LearnGrid {
 
 // Learned preconditioner: network parameters, optimiser state, training pairs, buffers.
 struct LearnState {
+  LearnState() = default;
+  LearnState(const LearnState&) = delete;
+  LearnState& operator=(const LearnState&) = delete;
+  ~LearnState() {
+    if (conv_error) cudaFreeHost(conv_error);
+  }
   bool have_params = false;
   int adam_step = 0;
   DevMem params, grad, m, v, fwd, bwd;  // LN_NPARAM floats; packed fragments LN_LAYERS * LN_PACK words
@@ -201,6 +207,7 @@ struct LearnState {
   // per tile, 2 TMA + tcgen05 pipeline
   int conv_kernel = 0;
   bool conv_timed_out = false;
+  int* conv_error = nullptr;             // pinned: set by this context's convolutions when a wait runs out
   int64_t conv_wait_polls = -1;          // bound of kernel 1's wait for its MMAs (-1: the default)
   std::map<int, std::unique_ptr<LearnGrid>> grids;
   // training pairs of one level: inputs (ln_pair_in(pair_nc) BF16 per voxel) and targets

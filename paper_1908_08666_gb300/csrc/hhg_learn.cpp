@@ -49,7 +49,12 @@ using namespace hhg::host;
 enum { LW_Z0 = 0, LW_AZ0, LW_R1, LW_C, LW_AC, LW_R, LW_Z, LW_AZ, LW_P, LW_Q, LW_X, LW_XS, LW_E, LW_CR, LW_CZ, LW_CE };
 
 LearnState& state(hhg_ctx* c) {
-  if (!c->learn) c->learn.reset(new LearnState());
+  if (!c->learn) {
+    std::unique_ptr<LearnState> S(new LearnState());
+    CK(cudaMallocHost((void**)&S->conv_error, sizeof(int)));
+    *S->conv_error = 0;
+    c->learn = std::move(S);
+  }
   return *c->learn;
 }
 
@@ -119,9 +124,9 @@ void repack(hhg_ctx* c, LearnState& S) {
 // after a wait on the stream: a tensor-core convolution whose bounded wait ran out disables
 // that kernel for the context (the warp-MMA convolution takes over) and fails the call
 void check_conv(LearnState& S) {
-  int flag = 0;
-  CK(conv_take_error(&flag));
-  if (flag) {
+  volatile int* error = S.conv_error;
+  if (*error) {
+    *error = 0;
     S.conv_kernel = 0;
     S.conv_timed_out = true;
     THROW(HHG_ERR_TIMEOUT, "tensor-core convolution timed out (switched to the warp-MMA kernel)");
@@ -189,14 +194,14 @@ void conv(hhg_ctx* c, LearnState& S, int l, bool bwd, const void* X, const float
   const void* wu = bwd ? layer_bwd_u(S, l) : layer_fwd_u(S, l);
   if (S.conv_kernel == 0 && !S.conv_timed_out) {
     bool taken = false;
-    CK(launch_conv_group(X, wu, bias, Y, Yf, nf, mask, s, relu, c->stream, &taken));
+    CK(launch_conv_group(X, wu, bias, Y, Yf, nf, mask, s, relu, c->stream, S.conv_error, &taken));
     if (taken) return;
   }
   if (S.conv_kernel == 2)
-    CK(launch_conv_tma(X, wu, bias, Y, Yf, nf, mask, s, relu, c->stream));
+    CK(launch_conv_tma(X, wu, bias, Y, Yf, nf, mask, s, relu, c->stream, S.conv_error));
   else
     CK(launch_conv(X, wp, S.conv_kernel == 1 ? wu : nullptr, bias, Y, Yf, nf, mask, s, relu, c->stream,
-                   S.conv_wait_polls));
+                   S.conv_error, S.conv_wait_polls));
 }
 
 // forward pass from act[0]: act[1..3] = hidden activations, out = the first nout FP32

@@ -211,7 +211,11 @@ constexpr long long U_SPIN_LIMIT = 1ll << 24;           // bound of the mbarrier
 static_assert(U_P0 + 128 * U_MT - 1 + U_P0 < U_PLANE_VOX, "plane too small for the shifted rows");
 static_assert((UZ * UPY + UY) * UPX + UX <= U_P0 + 128 * U_MT - 1, "M tiles do not cover the tile");
 
-__device__ int g_conv_error = 0;  // set when a tensor-core convolution's wait ran out
+// A tensor-core convolution whose wait ran out sets *error, a word of the context's pinned host memory.
+__device__ __forceinline__ void report_timeout(int* error) {
+  *(volatile int*)error = 1;
+  __threadfence_system();
+}
 
 // shared-memory matrix descriptor: start address, leading (K) and stride (M/N) byte
 // offsets of the core matrices, descriptor version 1, no swizzle
@@ -223,7 +227,7 @@ __device__ __forceinline__ uint64_t umma_desc(uint32_t addr, uint32_t lbo, uint3
 __global__ void __launch_bounds__(128) k_conv_umma(const uint4* __restrict__ X, const uint4* __restrict__ Wu,
                                                    const float* __restrict__ bias, uint4* __restrict__ Y,
                                                    float* __restrict__ Yf, int nf, const uint4* __restrict__ mask,
-                                                   int D, int H, int W, int ntz, int relu, long long wait_polls) {
+                                                   int D, int H, int W, int ntz, int relu, long long wait_polls, int* error) {
   extern __shared__ __align__(1024) unsigned char usm[];
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(usm);
   const uint32_t bar = sbase + U_BAR;
@@ -284,7 +288,7 @@ __global__ void __launch_bounds__(128) k_conv_umma(const uint4* __restrict__ X, 
   }
   done = __all_sync(0xffffffffu, done);
   if (!done) {
-    if (lane == 0) atomicExch(&g_conv_error, 1);
+    if (lane == 0) report_timeout(error);
     // drain: the MMAs this CTA issued must have completed before their tensor memory is
     // freed below; this wait keeps the full bound whatever wait_polls was
     uint32_t drained = 0;
@@ -385,7 +389,7 @@ __host__ __device__ constexpr int cg_smem(const ConvTiling& t) { return 4 * cg_p
 __global__ void __launch_bounds__(CG_THREADS, 2)
     k_conv_group(const uint4* __restrict__ X, const uint4* __restrict__ Wu, const float* __restrict__ bias,
                  uint4* __restrict__ Y, float* __restrict__ Yf, int nf, const uint4* __restrict__ mask, int D, int H,
-                 int W, int relu, const ConvTiling T) {
+                 int W, int relu, const ConvTiling T, int* error) {
   extern __shared__ __align__(1024) unsigned char usm[];
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(usm);
   const int plane = cg_plane(T);
@@ -565,7 +569,7 @@ __global__ void __launch_bounds__(CG_THREADS, 2)
     bad = __syncthreads_or(!done);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (bad) {
-      if (threadIdx.x == 0) atomicExch(&g_conv_error, 1);
+      if (threadIdx.x == 0) report_timeout(error);
       wait_bar(zi);  // drain: the MMAs must have completed before their tensor memory is freed
       break;
     }
@@ -640,7 +644,7 @@ constexpr int P_SMEM = P_BAR + 128;
 constexpr int P_TMEM_COLS = 256;
 constexpr uint32_t P_TX = 2u * U_VOX * 16u;  // bytes of one stage (two halves of 8 channels)
 
-__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile int* abort) {
+__device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile int* abort, int* error) {
   for (long long it = 0; it < U_SPIN_LIMIT; ++it) {
     uint32_t ok;
     asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}\n"
@@ -652,12 +656,12 @@ __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, volatile
     __nanosleep(64);
   }
   *abort = 1;
-  atomicExch(&g_conv_error, 1);
+  report_timeout(error);
   return false;
 }
 
 // bounded wait that ignores the abort flag: used to drain a block's own copies and MMAs
-__device__ __forceinline__ void bar_drain(uint32_t bar, uint32_t parity) {
+__device__ __forceinline__ void bar_drain(uint32_t bar, uint32_t parity, int* error) {
   for (long long it = 0; it < U_SPIN_LIMIT; ++it) {
     uint32_t ok;
     asm volatile("{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}\n"
@@ -667,7 +671,7 @@ __device__ __forceinline__ void bar_drain(uint32_t bar, uint32_t parity) {
     if (ok) return;
     __nanosleep(64);
   }
-  atomicExch(&g_conv_error, 1);
+  report_timeout(error);
 }
 
 __device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count) {
@@ -688,7 +692,7 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_conv_tma(const __grid_constant
                                                            const float* __restrict__ bias, uint4* __restrict__ Y,
                                                            float* __restrict__ Yf, int nf,
                                                            const uint4* __restrict__ mask, int D, int H, int W,
-                                                           int ntx, int nty, int ntz, int ntiles, int relu) {
+                                                           int ntx, int nty, int ntz, int ntiles, int relu, int* error) {
   extern __shared__ __align__(1024) unsigned char psm[];
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(psm);
   volatile int* abort = (volatile int*)(psm + P_ABORT);
@@ -725,7 +729,7 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_conv_tma(const __grid_constant
       int last[P_STAGES] = {-1, -1};
       for (int k = 0; k < ntile_mine; ++k) {
         const int st = k & 1;
-        if (k >= 2 && !bar_wait(sbase + P_EMPTY + 8 * st, ((k >> 1) - 1) & 1, abort)) break;
+        if (k >= 2 && !bar_wait(sbase + P_EMPTY + 8 * st, ((k >> 1) - 1) & 1, abort, error)) break;
         last[st] = k;
         const int tile = (int)blockIdx.x + k * (int)gridDim.x;
         const int tx = tile % ntx, ty = (tile / ntx) % nty, tzb = tile / (ntx * nty);
@@ -743,15 +747,15 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_conv_tma(const __grid_constant
       // no tensor copy of this block may still be writing shared memory when it exits
       if (*abort)
         for (int st = 0; st < P_STAGES; ++st)
-          if (last[st] >= 0) bar_drain(sbase + P_FULL + 8 * st, (last[st] >> 1) & 1);
+          if (last[st] >= 0) bar_drain(sbase + P_FULL + 8 * st, (last[st] >> 1) & 1, error);
     }
   } else if (warp == 1) {
-    if (lane == 0 && bar_wait(sbase + P_WBAR, 0, abort)) {
+    if (lane == 0 && bar_wait(sbase + P_WBAR, 0, abort, error)) {
       int last[P_STAGES] = {-1, -1};
       for (int k = 0; k < ntile_mine; ++k) {
         const int st = k & 1;
-        if (!bar_wait(sbase + P_FULL + 8 * st, (k >> 1) & 1, abort)) break;
-        if (k >= 2 && !bar_wait(sbase + P_TEMPTY + 8 * st, ((k >> 1) - 1) & 1, abort)) break;
+        if (!bar_wait(sbase + P_FULL + 8 * st, (k >> 1) & 1, abort, error)) break;
+        if (k >= 2 && !bar_wait(sbase + P_TEMPTY + 8 * st, ((k >> 1) - 1) & 1, abort, error)) break;
         last[st] = k;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
         // descriptors as base + offset in 16-byte units (the start-address field): an M tile
@@ -782,7 +786,7 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_conv_tma(const __grid_constant
       // no MMA of this block may still be running when its tensor memory is freed
       if (*abort)
         for (int st = 0; st < P_STAGES; ++st)
-          if (last[st] >= 0) bar_drain(sbase + P_EMPTY + 8 * st, (last[st] >> 1) & 1);
+          if (last[st] >= 0) bar_drain(sbase + P_EMPTY + 8 * st, (last[st] >> 1) & 1, error);
     }
     __syncwarp();
   } else {
@@ -792,7 +796,7 @@ __global__ void __launch_bounds__(P_THREADS, 1) k_conv_tma(const __grid_constant
     for (int c = 0; c < 16; ++c) bv[c] = bias ? bias[c] : 0.f;
     for (int k = 0; k < ntile_mine; ++k) {
       const int st = k & 1;
-      const bool ok = __all_sync(0xffffffffu, bar_wait(sbase + P_TFULL + 8 * st, (k >> 1) & 1, abort));
+      const bool ok = __all_sync(0xffffffffu, bar_wait(sbase + P_TFULL + 8 * st, (k >> 1) & 1, abort, error));
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       const int tile = (int)blockIdx.x + k * (int)gridDim.x;
@@ -1277,7 +1281,7 @@ inline int64_t red_blocks(int64_t V) { return blocks_for(V, RED_BLOCK, RED_MAX_B
 }  // namespace
 
 int launch_conv(const void* X, const uint32_t* Wp, const void* Wu, const float* bias, void* Y, float* Yf, int nf,
-                const void* mask, GridShape s, int relu, void* stream, int64_t wait_polls) {
+                const void* mask, GridShape s, int relu, void* stream, int* error, int64_t wait_polls) {
   if (s.voxels() == 0) return 0;
   if (Wu) {
     static bool uattr[64] = {};
@@ -1294,7 +1298,7 @@ int launch_conv(const void* X, const uint32_t* Wp, const void* Wu, const float* 
     dim3 grid((unsigned)((s.W + UX - 1) / UX), (unsigned)((s.H + UY - 1) / UY), (unsigned)(ntz * s.B));
     k_conv_umma<<<grid, 128, U_SMEM, (cudaStream_t)stream>>>((const uint4*)X, (const uint4*)Wu, bias, (uint4*)Y, Yf,
                                                              nf, (const uint4*)mask, s.D, s.H, s.W, ntz, relu,
-                                                             wait_polls < 0 ? U_SPIN_LIMIT : (long long)wait_polls);
+                                                             wait_polls < 0 ? U_SPIN_LIMIT : (long long)wait_polls, error);
     return (int)cudaGetLastError();
   }
   static bool attr[64] = {};  // per device: dynamic shared memory above 48 KB
@@ -1316,7 +1320,7 @@ int launch_conv(const void* X, const uint32_t* Wp, const void* Wu, const float* 
 }
 
 int launch_conv_group(const void* X, const void* Wu, const float* bias, void* Y, float* Yf, int nf, const void* mask,
-                      GridShape s, int relu, void* stream, bool* taken) {
+                      GridShape s, int relu, void* stream, int* error, bool* taken) {
   ConvTiling t;
   *taken = conv_tiling(s, t);
   if (!*taken) return 0;
@@ -1335,7 +1339,7 @@ int launch_conv_group(const void* X, const void* Wu, const float* bias, void* Y,
   const dim3 grid((unsigned)(t.xtiles * t.ytiles), (unsigned)t.zchunks, (unsigned)s.B);
   k_conv_group<<<grid, CG_THREADS, cg_smem(t), (cudaStream_t)stream>>>((const uint4*)X, (const uint4*)Wu, bias,
                                                                       (uint4*)Y, Yf, nf, (const uint4*)mask, s.D, s.H,
-                                                                      s.W, relu, t);
+                                                                      s.W, relu, t, error);
   return (int)cudaGetLastError();
 }
 
@@ -1411,7 +1415,7 @@ static int encode_act_map(CUtensorMap* map, const void* X, GridShape s) {
 }
 
 int launch_conv_tma(const void* X, const void* Wu, const float* bias, void* Y, float* Yf, int nf, const void* mask,
-                    GridShape s, int relu, void* stream) {
+                    GridShape s, int relu, void* stream, int* error) {
   if (s.voxels() == 0) return 0;
   static bool pattr[64] = {};
   int dev = 0;
@@ -1431,7 +1435,7 @@ int launch_conv_tma(const void* X, const void* Wu, const float* bias, void* Y, f
   const int grid = ntiles < 2 * 152 ? ntiles : 2 * 152;
   k_conv_tma<<<grid, P_THREADS, P_SMEM, (cudaStream_t)stream>>>(map, (const uint4*)Wu, bias, (uint4*)Y, Yf, nf,
                                                                  (const uint4*)mask, s.D, s.H, s.W, ntx, nty, ntz,
-                                                                 ntiles, relu);
+                                                                 ntiles, relu, error);
   return (int)cudaGetLastError();
 }
 
@@ -1439,20 +1443,6 @@ int launch_pack_umma(const float* params, void* fwd, void* bwd, void* stream) {
   const int n = LN_LAYERS * LN_TAPS * 256;
   k_pack_umma<<<(n + 255) / 256, 256, 0, (cudaStream_t)stream>>>(params, (__nv_bfloat16*)fwd, (__nv_bfloat16*)bwd);
   return (int)cudaGetLastError();
-}
-
-int conv_take_error(int* flag) {
-  int v = 0;
-  cudaError_t e = cudaMemcpyFromSymbol(&v, g_conv_error, sizeof(int));
-  if (e != cudaSuccess) return (int)e;
-  if (v) {
-    const int zero = 0;
-    e = cudaMemcpyToSymbol(g_conv_error, &zero, sizeof(int));
-    // landed before a kernel on a (non-blocking) library stream can read the flag
-    if (e == cudaSuccess) e = cudaStreamSynchronize(cudaStreamLegacy);
-  }
-  *flag = v;
-  return (int)e;
 }
 
 int launch_pack(const float* params, uint32_t* fwd, uint32_t* bwd, void* stream) {

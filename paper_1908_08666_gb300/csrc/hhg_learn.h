@@ -45,21 +45,20 @@ struct GridShape {
 // Wu (nullable): the layer's tcgen05 operands (launch_pack_umma); when given, the
 // tensor-memory kernel runs instead of the warp-MMA one, its wait for the MMAs bounded by
 // wait_polls polls (negative: the default bound).
+// error (of every tensor-core convolution): a word of pinned host memory, set to 1 when a wait runs out.
 int launch_conv(const void* X, const uint32_t* Wp, const void* Wu, const float* bias, void* Y, float* Yf, int nf,
-                const void* mask, GridShape s, int relu, void* stream,
+                const void* mask, GridShape s, int relu, void* stream, int* error,
                 int64_t wait_polls = -1);
 // The same convolution as a persistent TMA + tcgen05 pipeline (Wu required)
 int launch_conv_tma(const void* X, const void* Wu, const float* bias, void* Y, float* Yf, int nf, const void* mask,
-                    GridShape s, int relu, void* stream);
+                    GridShape s, int relu, void* stream, int* error);
 // The same convolution with four voxels per matrix row on tcgen05 (Wu required); *taken = false, and
 // nothing is launched, for grids too small for its tiles
 int launch_conv_group(const void* X, const void* Wu, const float* bias, void* Y, float* Yf, int nf, const void* mask,
-                      GridShape s, int relu, void* stream, bool* taken);
+                      GridShape s, int relu, void* stream, int* error, bool* taken);
 // tcgen05 operands of every layer (LN_UMMA bytes each, forward and input-gradient weights)
 constexpr int LN_UMMA = LN_TAPS * 256 * 2;
 int launch_pack_umma(const float* params, void* fwd, void* bwd, void* stream);
-// *flag = whether a tensor-core convolution's bounded wait ran out since the last call (resets it)
-int conv_take_error(int* flag);
 
 // dW[t][i][o] = sum_v A[v + off(t)][i] G[v][o] for all taps: per-block partial sums into
 // partial (wgrad_partials() blocks x LN_WSIZE floats), then their ordered sum into dW.

@@ -77,3 +77,30 @@ def test_grids_of_different_tilings_from_two_threads():
     finally:
         for net in nets:
             net.close()
+
+
+def test_a_timeout_is_reported_to_its_own_context():
+    """One context's wait for its MMAs runs out in every call (bound of zero polls); the other one's calls,
+    whose kernel has no such wait, succeed meanwhile."""
+    nets = [Net(3, (1, 3, 4, 16)), Net(4, (1, 3, 4, 16))]
+    try:
+        nets[1].forward()
+        want = nets[1].out.clone()
+        B.hhg_learn_set_conv_wait(nets[0].h, 0)
+
+        def times_out():
+            for _ in range(300):
+                B.hhg_learn_set_conv_kernel(nets[0].h, 1)
+                with pytest.raises(B.HhgError) as e:
+                    nets[0].forward()
+                assert e.value.status == 7
+
+        def succeeds():
+            for _ in range(300):
+                nets[1].forward()
+
+        assert _together(times_out, succeeds) == []
+        assert nets[1].torch.equal(nets[1].out, want)
+    finally:
+        for net in nets:
+            net.close()
