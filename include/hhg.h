@@ -467,20 +467,20 @@ hhg_status hhg_residual_noalloc(hhg_ctx* ctx, int level, hhg_dtype dt, const voi
 int64_t hhg_learn_num_params(void);
 /* Convolution kernel of the network: 0 (default) = 5th-generation tensor cores (tcgen05.mma with
  * accumulators in tensor memory) with four voxels per matrix row, marching in z; grids too small for its
- * tiles, and every grid after a tensor-core kernel's wait ran out, take warp-level BF16 MMA (mma.sync
- * m16n8k16) on a shared-memory tile; 1 = tcgen05 with a voxel per row
+ * tiles, and every grid after a tensor-core kernel's wait ran out (until the next call of this function),
+ * take warp-level BF16 MMA (mma.sync m16n8k16) on a shared-memory tile; 1 = tcgen05 with a voxel per row
  * (6 x 27 MMAs of 128 x 16 x 16 per 32 x 4 x 4 output tile,
  * one tile per block), 2 = the same MMAs in a persistent pipeline (tensor-memory-
  * accelerator loads into two shared stages, two tensor-memory accumulator sets, an
  * epilogue warpgroup draining one while the next tile's MMAs run).  All give the same
  * results up to FP32 summation order. */
 hhg_status hhg_learn_set_conv_kernel(hhg_ctx* ctx, int kernel);
-/* Bound of the tensor-core convolution's (kernel 1) wait for its MMAs, in polls about 100 ns
- * apart; negative restores the default (2^24 polls).  Fault handling, not the paper: when the
+/* Bound of the waits of the tensor-core convolutions 0 and 1 for their MMAs, in polls 40 (kernel 0) or
+ * 100 ns apart; negative restores the default (2^24 polls).  Fault handling, not the paper: when a
  * wait runs out the kernel records an error, still waits (with the default bound) for the MMAs
  * it issued before freeing their tensor memory, skips its epilogue and returns; the call then
- * fails with HHG_ERR_TIMEOUT and the context falls back to convolution kernel 0.  A short
- * bound lets a test make the wait run out without a fault; the context stays usable. */
+ * fails with HHG_ERR_TIMEOUT and the context falls back to the warp-level MMA kernel (kernel 0 on small
+ * grids).  A short bound lets a test make the wait run out without a fault; the context stays usable. */
 hhg_status hhg_learn_set_conv_wait(hhg_ctx* ctx, int64_t polls);
 /* Coarse-grid mode (elasticity; levels = 0 default, 1..3): the network runs on the node
  * grid `levels` levels below the solve's.  Its inputs there are r1 restricted (P^T, as in

@@ -206,9 +206,9 @@ struct LearnState {
   // 0 tcgen05 with four voxels per row (warp MMA on small grids and after a timed-out wait), 1 tcgen05
   // per tile, 2 TMA + tcgen05 pipeline
   int conv_kernel = 0;
-  bool conv_timed_out = false;
+  bool conv_timed_out = false;           // until the kernel is chosen again
   int* conv_error = nullptr;             // pinned: set by this context's convolutions when a wait runs out
-  int64_t conv_wait_polls = -1;          // bound of kernel 1's wait for its MMAs (-1: the default)
+  int64_t conv_wait_polls = -1;          // bound of the waits of kernels 0 and 1 for their MMAs (-1: the default)
   std::map<int, std::unique_ptr<LearnGrid>> grids;
   // training pairs of one level: inputs (ln_pair_in(pair_nc) BF16 per voxel) and targets
   // (pair_nc FP32), pair_nc = components of the problem they came from

@@ -121,8 +121,8 @@ void repack(hhg_ctx* c, LearnState& S) {
   CK(launch_pack_umma(S.params.as<float>(), S.fwd_u.p, S.bwd_u.p, c->stream));
 }
 
-// after a wait on the stream: a tensor-core convolution whose bounded wait ran out disables
-// that kernel for the context (the warp-MMA convolution takes over) and fails the call
+// after a wait on the stream: a tensor-core convolution whose bounded wait ran out fails the call, and
+// the warp-MMA convolution takes over in the context until hhg_learn_set_conv_kernel
 void check_conv(LearnState& S) {
   volatile int* error = S.conv_error;
   if (*error) {
@@ -194,7 +194,8 @@ void conv(hhg_ctx* c, LearnState& S, int l, bool bwd, const void* X, const float
   const void* wu = bwd ? layer_bwd_u(S, l) : layer_fwd_u(S, l);
   if (S.conv_kernel == 0 && !S.conv_timed_out) {
     bool taken = false;
-    CK(launch_conv_group(X, wu, bias, Y, Yf, nf, mask, s, relu, c->stream, S.conv_error, &taken));
+    CK(launch_conv_group(X, wu, bias, Y, Yf, nf, mask, s, relu, c->stream, S.conv_error, S.conv_wait_polls,
+                         &taken));
     if (taken) return;
   }
   if (S.conv_kernel == 2)
@@ -529,6 +530,7 @@ double precondition(hhg_ctx* c, int l, const float* r, float* z, float* az, bool
       b = 0.0;
     }
   }
+  check_conv(S);  // the inner products waited for the network
   const double w = b / a;
   S.applications++;
   if (b == 0.0) S.fallbacks++;
@@ -767,7 +769,6 @@ void learned_ir(hhg_ctx* c, const hhg_solve_opts* o, const double* f, double* x,
   if (st) project_pressure64(c, l, x);
   R.rel_residual = r0 > 0.0 ? std::sqrt(rr / r0) : 0.0;
   R.converged = R.rel_residual <= o->rtol;
-  if (use_net) check_conv(state(c));
 }
 
 }  // namespace host
@@ -800,6 +801,7 @@ hhg_status hhg_learn_set_conv_kernel(hhg_ctx* c, int kernel) {
   return guard(c, [&] {
     if (kernel < 0 || kernel > 2) THROW(HHG_ERR_ARG, "conv kernel 0 (default), 1 (tcgen05) or 2 (TMA + tcgen05)");
     state(c).conv_kernel = kernel;
+    state(c).conv_timed_out = false;
   });
 }
 
@@ -1088,7 +1090,6 @@ hhg_status hhg_learn_precondition(hhg_ctx* c, int level, int use_net, const void
     float* az = lwork(c, G, level, LW_AZ);
     const double a = precondition(c, level, (const float*)r, (float*)z, az, use_net != 0);
     wait_stream(c);
-    check_conv(state(c));
     if (alpha) *alpha = a;
   });
 }

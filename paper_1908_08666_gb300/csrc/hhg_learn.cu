@@ -206,7 +206,7 @@ constexpr int U_BAR = 2 * U_PLANE + U_WBYTES;           // mbarrier and TMEM-add
 constexpr int U_SMEM = U_BAR + 64;
 constexpr int U_TMEM_COLS = 128;                        // 6 accumulators x 16 columns, rounded up
 constexpr uint32_t U_IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((16u >> 3) << 17) | ((128u >> 4) << 24);
-constexpr long long U_SPIN_LIMIT = 1ll << 24;           // bound of the mbarrier wait (polls, 100 ns apart)
+constexpr long long U_SPIN_LIMIT = 1ll << 24;           // bound of the mbarrier waits (polls, 40 to 100 ns apart)
 
 static_assert(U_P0 + 128 * U_MT - 1 + U_P0 < U_PLANE_VOX, "plane too small for the shifted rows");
 static_assert((UZ * UPY + UY) * UPX + UX <= U_P0 + 128 * U_MT - 1, "M tiles do not cover the tile");
@@ -389,7 +389,7 @@ __host__ __device__ constexpr int cg_smem(const ConvTiling& t) { return 4 * cg_p
 __global__ void __launch_bounds__(CG_THREADS, 2)
     k_conv_group(const uint4* __restrict__ X, const uint4* __restrict__ Wu, const float* __restrict__ bias,
                  uint4* __restrict__ Y, float* __restrict__ Yf, int nf, const uint4* __restrict__ mask, int D, int H,
-                 int W, int relu, const ConvTiling T, int* error) {
+                 int W, int relu, const ConvTiling T, long long wait_polls, int* error) {
   extern __shared__ __align__(1024) unsigned char usm[];
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(usm);
   const int plane = cg_plane(T);
@@ -499,9 +499,9 @@ __global__ void __launch_bounds__(CG_THREADS, 2)
     }
     asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
   };
-  auto wait_bar = [&](int zi) {  // bounded
+  auto wait_bar = [&](int zi, long long polls) {  // bounded
     uint32_t done = 0;
-    for (long long it = 0; it < U_SPIN_LIMIT && !done; ++it) {
+    for (long long it = 0; it < polls && !done; ++it) {
       asm volatile(
           "{\n.reg .pred q;\nmbarrier.try_wait.parity.shared::cta.b64 q, [%1], %2;\nselp.u32 %0, 1, 0, q;\n}\n"
           : "=r"(done)
@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(CG_THREADS, 2)
       if (zi > 0) store_plane(zi - 1);
     }
     __syncwarp();
-    const uint32_t done = wait_bar(zi);
+    const uint32_t done = wait_bar(zi, wait_polls);
     asm volatile("cp.async.wait_group 0;\n" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -570,7 +570,9 @@ __global__ void __launch_bounds__(CG_THREADS, 2)
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     if (bad) {
       if (threadIdx.x == 0) report_timeout(error);
-      wait_bar(zi);  // drain: the MMAs must have completed before their tensor memory is freed
+      // drain: the MMAs must have completed before their tensor memory is freed; the full bound whatever
+      // wait_polls was
+      wait_bar(zi, U_SPIN_LIMIT);
       break;
     }
   }
@@ -1320,7 +1322,7 @@ int launch_conv(const void* X, const uint32_t* Wp, const void* Wu, const float* 
 }
 
 int launch_conv_group(const void* X, const void* Wu, const float* bias, void* Y, float* Yf, int nf, const void* mask,
-                      GridShape s, int relu, void* stream, int* error, bool* taken) {
+                      GridShape s, int relu, void* stream, int* error, int64_t wait_polls, bool* taken) {
   ConvTiling t;
   *taken = conv_tiling(s, t);
   if (!*taken) return 0;
@@ -1339,7 +1341,9 @@ int launch_conv_group(const void* X, const void* Wu, const float* bias, void* Y,
   const dim3 grid((unsigned)(t.xtiles * t.ytiles), (unsigned)t.zchunks, (unsigned)s.B);
   k_conv_group<<<grid, CG_THREADS, cg_smem(t), (cudaStream_t)stream>>>((const uint4*)X, (const uint4*)Wu, bias,
                                                                       (uint4*)Y, Yf, nf, (const uint4*)mask, s.D, s.H,
-                                                                      s.W, relu, t, error);
+                                                                      s.W, relu, t,
+                                                                      wait_polls < 0 ? U_SPIN_LIMIT : (long long)wait_polls,
+                                                                      error);
   return (int)cudaGetLastError();
 }
 

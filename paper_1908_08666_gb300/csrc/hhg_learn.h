@@ -52,10 +52,10 @@ int launch_conv(const void* X, const uint32_t* Wp, const void* Wu, const float* 
 // The same convolution as a persistent TMA + tcgen05 pipeline (Wu required)
 int launch_conv_tma(const void* X, const void* Wu, const float* bias, void* Y, float* Yf, int nf, const void* mask,
                     GridShape s, int relu, void* stream, int* error);
-// The same convolution with four voxels per matrix row on tcgen05 (Wu required); *taken = false, and
-// nothing is launched, for grids too small for its tiles
+// The same convolution with four voxels per matrix row on tcgen05 (Wu required; wait_polls as above);
+// *taken = false, and nothing is launched, for grids too small for its tiles
 int launch_conv_group(const void* X, const void* Wu, const float* bias, void* Y, float* Yf, int nf, const void* mask,
-                      GridShape s, int relu, void* stream, int* error, bool* taken);
+                      GridShape s, int relu, void* stream, int* error, int64_t wait_polls, bool* taken);
 // tcgen05 operands of every layer (LN_UMMA bytes each, forward and input-gradient weights)
 constexpr int LN_UMMA = LN_TAPS * 256 * 2;
 int launch_pack_umma(const float* params, void* fwd, void* bwd, void* stream);

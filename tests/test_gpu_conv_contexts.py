@@ -104,3 +104,39 @@ def test_a_timeout_is_reported_to_its_own_context():
     finally:
         for net in nets:
             net.close()
+
+
+# grids up to 456 tiles of 4 x 4 x 32 voxels take the warp-level kernel, which has no wait; larger ones the
+# grouped tcgen05 kernel, in both of its tile forms, batched and with a ragged march in z
+@pytest.mark.parametrize("shape,grouped", [((1, 33, 20, 129), False), ((1, 29, 65, 127), True), ((1, 33, 65, 66), True),
+                                           ((24, 16, 20, 16), True), ((1, 5, 160, 165), True)])
+def test_default_kernel_timeout_falls_back(shape, grouped):
+    """With a bound of zero polls the grouped kernel's wait runs out in every block: the call reports it, the
+    next ones run on the warp-level kernel, and choosing the kernel again brings the grouped one back.  All
+    results agree to the last bit, as the kernels do."""
+    net = Net(5, shape)
+    try:
+        t = net.torch
+        net.forward()
+        want = net.out.clone()
+
+        def same():
+            net.out.fill_(7.0)
+            t.cuda.synchronize()
+            net.forward()
+            return t.equal(net.out, want)
+
+        B.hhg_learn_set_conv_wait(net.h, 0)
+        if not grouped:
+            assert same()
+            return
+        for _ in range(2):
+            with pytest.raises(B.HhgError) as e:
+                net.forward()
+            assert e.value.status == 7 and "timed out" in str(e.value)
+            assert same()  # the warp-level kernel: the bound is still zero
+            B.hhg_learn_set_conv_kernel(net.h, 0)
+        B.hhg_learn_set_conv_wait(net.h, -1)
+        assert same()
+    finally:
+        net.close()
