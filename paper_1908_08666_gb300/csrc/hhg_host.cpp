@@ -386,7 +386,9 @@ MacroConsts<T> cast_consts(const MacroConsts<double>& c) {
 
 // Blocks of the skeleton rows (LevelDev).  Macro vertices take 1, 2 or 4 warps of a block by their number
 // of incidences (two per warp and round, two rounds), the widest first (they run longest); nodes inside a
-// macro edge lie in the same macros and are numbered along it; nodes inside faces are ordered by macros and face types, those next to the face's edges apart.
+// macro edge lie in the same macros and are numbered along it; nodes inside faces are ordered by macros and
+// face types, those next to the face's edges apart.  A face block has two sides, so the nodes of a face in
+// more than two macros (the mesh need not be a manifold) go to the vertices' list.
 void build_rows(LevelHost& L) {
   const int n = L.n;
   const int64_t nskel = (int64_t)L.skel_dir.size();
@@ -421,7 +423,7 @@ void build_rows(LevelHost& L) {
       const SkelInc& I = L.skel_inc[b0];
       if (L.skel_support[s] == 3)
         for (const int w : {n - I.i - I.j - I.k, (int)I.i, (int)I.j, (int)I.k}) q.near |= w == 1;
-      (L.skel_support[s] == 3 ? faces : keys).push_back(q);
+      (L.skel_support[s] == 3 && ni <= 2 ? faces : keys).push_back(q);
     }
     for (auto& ed : edges) {
       std::sort(ed.second.begin(), ed.second.end());
