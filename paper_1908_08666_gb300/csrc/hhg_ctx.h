@@ -326,6 +326,15 @@ struct hhg_ctx {
 namespace hhg {
 namespace host {
 
+// Element matrices of one macro's 6 Kuhn element types: the stiffness, and for the Stokes blocks
+// bd[type][a][b][l] = -int phi_a d_l phi_b (pressure test vertex a, velocity trial vertex b) and
+// lc[type][a][b] = -(h^2/12) int grad phi_a . grad phi_b.
+struct ElementMatrices {
+  NodalConsts<double> ke;
+  double bd[6][4][4][3];
+  double lc[6][4][4];
+};
+
 // Slots of the partial-sum scratch: the largest sweep's blocks, and at least the partials of two
 // dot-product launches in a row (1024 blocks each: the Stokes inner product over the velocity and
 // the pressure components writes both before reducing them together).

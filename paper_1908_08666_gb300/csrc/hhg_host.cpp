@@ -19,6 +19,10 @@
 
 namespace {
 
+void check_element(double det) {
+  if (std::fabs(det) < 1e-300) THROW(HHG_ERR_ARG, "degenerate element");
+}
+
 // element stiffness K[a][b][m][l] = |t| (c_eps eps(phi_b e_l):eps(phi_a e_m) + c_div div(phi_b e_l) div(phi_a e_m))
 void element_stiffness(const Vec3d v[4], double c_eps, double c_div, double K[4][4][9]) {
   double J[3][3];
@@ -29,7 +33,7 @@ void element_stiffness(const Vec3d v[4], double c_eps, double c_div, double K[4]
   }
   const double det = J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) - J[0][1] * (J[1][0] * J[2][2] - J[1][2] * J[2][0]) +
                      J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
-  if (std::fabs(det) < 1e-300) THROW(HHG_ERR_ARG, "degenerate element");
+  check_element(det);
   // inverse of J; gradient of barycentric a (a=1..3) = column a-1 of J^{-1}
   double inv[3][3];
   inv[0][0] = (J[1][1] * J[2][2] - J[1][2] * J[2][1]) / det;
@@ -97,12 +101,8 @@ int dir_from_kuhn(const int v[3]) {
   return -1;
 }
 
-// Per-macro constants at intervals n: element stiffness of the 6 Kuhn element
-// types and the interior stencil (Shat and the correction axial vectors).
 // P1 gradients and volume of one element
 void element_gradients(const Vec3d v[4], double g[4][3], double& vol) {
-  double K[4][4][9];
-  element_stiffness(v, 1.0, 0.0, K);  // validates the element
   double J[3][3];
   const Vec3d* w[3] = {&v[1], &v[2], &v[3]};
   for (int r = 0; r < 3; ++r) {
@@ -112,6 +112,7 @@ void element_gradients(const Vec3d v[4], double g[4][3], double& vol) {
   }
   const double det = J[0][0] * (J[1][1] * J[2][2] - J[1][2] * J[2][1]) - J[0][1] * (J[1][0] * J[2][2] - J[1][2] * J[2][0]) +
                      J[0][2] * (J[1][0] * J[2][1] - J[1][1] * J[2][0]);
+  check_element(det);
   // columns of J^{-1} = gradients of barycentrics 1..3 (cofactor formula)
   const double c00 = (J[1][1] * J[2][2] - J[1][2] * J[2][1]), c01 = (J[0][2] * J[2][1] - J[0][1] * J[2][2]),
                c02 = (J[0][1] * J[1][2] - J[0][2] * J[1][1]);
@@ -127,9 +128,77 @@ void element_gradients(const Vec3d v[4], double g[4][3], double& vol) {
   vol = std::fabs(det) / 6.0;
 }
 
-void macro_constants(const MacroGeom& G, int n, double c_eps, double c_div, MacroConsts<double>& out) {
-  double KE[6][4][4][9];
-  double BD[6][4][4][3], LC[6][4][4];
+// The patch of the edge (0, d): its elements (Kuhn type p; point 0 and point d are the vertices a and b),
+// the neighbours that are their vertices (direction, NDIR for point 0) and those vertices' reflections
+// through the edge's midpoint, and the element's place in the cyclic order of the edge's ring.  The same in
+// every macro, so built once: searched per macro, hhg_set_problem took 48 ms for 384 macros on levels 2 and
+// 3, now 11.
+struct Patch {
+  struct Element {
+    int p, a, b, at, vertex[4], mirror[4];
+  };
+  int count = 0;
+  Element e[6];
+};
+
+int node_of(const int off[3]) { return off[0] == 0 && off[1] == 0 && off[2] == 0 ? NDIR : dir_from_kuhn(off); }
+
+std::array<Patch, NDIR> build_patches() {
+  std::array<Patch, NDIR> out;
+  for (int d = 0; d < NDIR; ++d) {
+    Patch& T = out[d];
+    int dk[3];
+    dir_kuhn(d, dk);
+    const int nring = dir_red(d) ? 6 : 4;
+    double wk[NDIR + 1] = {0};
+    for (int p = 0; p < 6; ++p) {
+      int P[4][3];
+      kuhn_vertices(p, P);
+      for (int a = 0; a < 4; ++a)
+        for (int b = 0; b < 4; ++b) {
+          if (a == b || P[b][0] - P[a][0] != dk[0] || P[b][1] - P[a][1] != dk[1] || P[b][2] - P[a][2] != dk[2]) continue;
+          if (T.count == nring) THROW(HHG_ERR_STATE, "patch of direction %d has more than %d elements", d, nring);
+          Patch::Element& e = T.e[T.count++];
+          e.p = p;
+          e.a = a;
+          e.b = b;
+          e.at = -1;
+          int other[2], no = 0;
+          for (int v = 0; v < 4; ++v) {
+            const int off[3] = {P[v][0] - P[a][0], P[v][1] - P[a][1], P[v][2] - P[a][2]};
+            const int ref[3] = {dk[0] - off[0], dk[1] - off[1], dk[2] - off[2]};
+            e.vertex[v] = node_of(off);
+            e.mirror[v] = node_of(ref);
+            if (e.vertex[v] < 0 || e.mirror[v] < 0) THROW(HHG_ERR_STATE, "patch vertex is not a stencil neighbour");
+            wk[e.vertex[v]] += 0.25 / nring;
+            if (v != a && v != b) other[no++] = e.vertex[v];
+          }
+          for (int q = 0; q < nring; ++q)
+            if ((ring_cyc(d, q) == other[0] && ring_cyc(d, q + 1) == other[1]) ||
+                (ring_cyc(d, q) == other[1] && ring_cyc(d, q + 1) == other[0]))
+              e.at = q;
+          if (e.at < 0) THROW(HHG_ERR_STATE, "element outside the ring of direction %d", d);
+        }
+    }
+    if (T.count != nring) THROW(HHG_ERR_STATE, "patch of direction %d has %d elements", d, T.count);
+    // the weights of khat that the kernels use
+    for (int q = 0; q <= NDIR; ++q) {
+      bool ring = false;
+      for (int c = 0; c < ring_count(d); ++c) ring |= (q == ring_a(d, c) || q == ring_b(d, c));
+      const double want = (q == NDIR || q == d) ? 0.25 : (ring ? (dir_red(d) ? 1.0 / 12.0 : 0.125) : 0.0);
+      if (std::fabs(wk[q] - want) > 1e-14) THROW(HHG_ERR_STATE, "patch-mean weight mismatch (dir %d)", d);
+    }
+  }
+  return out;
+}
+
+// Per-macro constants at intervals n: the element matrices of the 6 Kuhn element types, and from them the
+// interior stencil (Shat and the correction axial vectors) and the rows' constants.
+void macro_constants(const MacroGeom& G, int n, double c_eps, double c_div, ElementMatrices& em, MacroConsts<double>& out) {
+  static const std::array<Patch, NDIR> patches = build_patches();
+  auto &KE = em.ke.ke;
+  auto &BD = em.bd;
+  auto &LC = em.lc;
   // stabilisation length of the macro's refined mesh: h = (6 |T|)^{1/3} / n (the lattice
   // spacing 1/n on the Kuhn cube)
   double hT;
@@ -145,134 +214,65 @@ void macro_constants(const MacroGeom& G, int n, double c_eps, double c_div, Macr
     Vec3d v[4];
     for (int a = 0; a < 4; ++a) v[a] = G.kuhn_to_x(P[a][0], P[a][1], P[a][2], n);
     element_stiffness(v, c_eps, c_div, KE[p]);
-    for (int a = 0; a < 4; ++a)
-      for (int b = 0; b < 4; ++b)
-        for (int q = 0; q < 9; ++q) out.ke[p][a][b][q] = KE[p][a][b][q];
     double g[4][3], vol;
     element_gradients(v, g, vol);
     for (int a = 0; a < 4; ++a)
       for (int b = 0; b < 4; ++b) {
         for (int l = 0; l < 3; ++l) BD[p][a][b][l] = -0.25 * vol * g[b][l];
         LC[p][a][b] = -(hT * hT / 12.0) * vol * (g[a][0] * g[b][0] + g[a][1] * g[b][1] + g[a][2] * g[b][2]);
-        for (int l = 0; l < 3; ++l) out.bd[p][a][b][l] = BD[p][a][b][l];
-        out.lc[p][a][b] = LC[p][a][b];
       }
   }
-  // patches of the 14 directions
   for (int d = 0; d < NDIR; ++d) {
-    int dk[3];
-    dir_kuhn(d, dk);
+    const Patch& patch = patches[d];
     double Sh[9] = {0};
     // coefficient matrix of k at each neighbour offset (index = direction, 14 = centre)
     double C[NDIR + 1][9];
-    double wk[NDIR + 1];
     std::memset(C, 0, sizeof(C));
-    std::memset(wk, 0, sizeof(wk));
-    int count = 0;
-    struct PatchEl {
-      int p, a, b;
-      int c[3];
-    };
-    std::vector<PatchEl> patch;
-    for (int p = 0; p < 6; ++p) {
-      int P[4][3];
-      kuhn_vertices(p, P);
-      for (int a = 0; a < 4; ++a)
-        for (int b = 0; b < 4; ++b) {
-          if (a == b) continue;
-          if (P[b][0] - P[a][0] == dk[0] && P[b][1] - P[a][1] == dk[1] && P[b][2] - P[a][2] == dk[2]) {
-            PatchEl e;
-            e.p = p;
-            e.a = a;
-            e.b = b;
-            for (int c = 0; c < 3; ++c) e.c[c] = -P[a][c];
-            patch.push_back(e);
-          }
-        }
-    }
-    count = (int)patch.size();
-    if (count != (dir_red(d) ? 6 : 4)) THROW(HHG_ERR_STATE, "patch of direction %d has %d elements", d, count);
-    auto node_of = [&](const int off[3]) -> int {
-      if (off[0] == 0 && off[1] == 0 && off[2] == 0) return NDIR;
-      return dir_from_kuhn(off);
-    };
     for (int l = 0; l < 3; ++l) {
       out.st.B[d][l] = 0;
       out.st.G[d][l] = 0;
     }
     out.st.C[d] = 0;
-    for (const PatchEl& e : patch) {
+    for (int q = 0; q < 6 * 16; ++q) out.el[d][q / 16][q % 16] = 0;
+    for (int q = 0; q < patch.count; ++q) {
+      const Patch::Element& e = patch.e[q];
+      const double* K = KE[e.p][e.a][e.b];
       for (int l = 0; l < 3; ++l) {
         out.st.B[d][l] += BD[e.p][e.a][e.b][l];
         out.st.G[d][l] += BD[e.p][e.b][e.a][l];
       }
       out.st.C[d] += LC[e.p][e.a][e.b];
-    }
-    for (const PatchEl& e : patch) {
-      const double* K = KE[e.p][e.a][e.b];
       for (int m = 0; m < 3; ++m)
         for (int l = 0; l < 3; ++l) Sh[m * 3 + l] += 0.5 * (K[m * 3 + l] + K[l * 3 + m]);
-      int P[4][3];
-      kuhn_vertices(e.p, P);
-      // vertices of t and of its reflection t^m (d - v)
-      for (int v = 0; v < 4; ++v) {
-        int off[3] = {e.c[0] + P[v][0], e.c[1] + P[v][1], e.c[2] + P[v][2]};
-        int ref[3] = {dk[0] - off[0], dk[1] - off[1], dk[2] - off[2]};
-        const int iv = node_of(off), ir = node_of(ref);
-        if (iv < 0 || ir < 0) THROW(HHG_ERR_STATE, "patch vertex is not a stencil neighbour");
-        wk[iv] += 0.25 / count;
+      for (int v = 0; v < 4; ++v)
         for (int m = 0; m < 3; ++m)
           for (int l = 0; l < 3; ++l) {
             const double an = 0.5 * (K[m * 3 + l] - K[l * 3 + m]);
-            C[iv][m * 3 + l] += 0.5 * 0.25 * an;
-            C[ir][m * 3 + l] -= 0.5 * 0.25 * an;
+            C[e.vertex[v]][m * 3 + l] += 0.5 * 0.25 * an;
+            C[e.mirror[v]][m * 3 + l] -= 0.5 * 0.25 * an;
           }
+      double* el = out.el[d][e.at];
+      for (int r = 0; r < 9; ++r) el[r] = K[r];
+      for (int l = 0; l < 3; ++l) {
+        el[9 + l] = BD[e.p][e.a][e.b][l];
+        el[12 + l] = BD[e.p][e.b][e.a][l];
       }
+      el[15] = LC[e.p][e.a][e.b];
     }
-    // the elements of the edge in cyclic order of its ring
-    {
-      for (int e = 0; e < 6; ++e)
-        for (int q = 0; q < 16; ++q) out.el[d][e][q] = 0;
-      for (const PatchEl& e : patch) {
-        int P[4][3], other[2], no = 0;
-        kuhn_vertices(e.p, P);
-        for (int v = 0; v < 4; ++v) {
-          if (v == e.a || v == e.b) continue;
-          const int off[3] = {e.c[0] + P[v][0], e.c[1] + P[v][1], e.c[2] + P[v][2]};
-          other[no++] = node_of(off);
-        }
-        int at = -1;
-        for (int q = 0; q < count; ++q)
-          if ((ring_cyc(d, q) == other[0] && ring_cyc(d, q + 1) == other[1]) ||
-              (ring_cyc(d, q) == other[1] && ring_cyc(d, q + 1) == other[0]))
-            at = q;
-        if (at < 0) THROW(HHG_ERR_STATE, "element outside the ring of direction %d", d);
-        double* el = out.el[d][at];
-        for (int q = 0; q < 9; ++q) el[q] = KE[e.p][e.a][e.b][q];
-        for (int l = 0; l < 3; ++l) {
-          el[9 + l] = BD[e.p][e.a][e.b][l];
-          el[12 + l] = BD[e.p][e.b][e.a][l];
-        }
-        el[15] = LC[e.p][e.a][e.b];
-      }
-    }
-    // checks: Shat symmetric, khat weights, ring structure, pair antisymmetry
+    // checks: Shat symmetric, ring structure, pair antisymmetry
     for (int m = 0; m < 3; ++m)
       for (int l = 0; l < 3; ++l) {
         double full = 0;
-        for (const PatchEl& e : patch) full += KE[e.p][e.a][e.b][m * 3 + l];
+        for (int q = 0; q < patch.count; ++q) full += KE[patch.e[q].p][patch.e[q].a][patch.e[q].b][m * 3 + l];
         if (std::fabs(full - Sh[m * 3 + l]) > 1e-12 * (1 + std::fabs(full)))
           THROW(HHG_ERR_STATE, "reference stencil of direction %d is not symmetric", d);
       }
-    const double wr = dir_red(d) ? 1.0 / 12.0 : 0.125;
     double cmax = 0;
     for (int q = 0; q <= NDIR; ++q)
       for (int r = 0; r < 9; ++r) cmax = std::max(cmax, std::fabs(C[q][r]));
     for (int q = 0; q <= NDIR; ++q) {
       bool ring = false;
       for (int c = 0; c < ring_count(d); ++c) ring |= (q == ring_a(d, c) || q == ring_b(d, c));
-      const double want = (q == NDIR || q == d) ? 0.25 : (ring ? wr : 0.0);
-      if (std::fabs(wk[q] - want) > 1e-14) THROW(HHG_ERR_STATE, "patch-mean weight mismatch (dir %d)", d);
       if (!ring) {
         for (int r = 0; r < 9; ++r)
           if (std::fabs(C[q][r]) > 1e-12 * cmax) THROW(HHG_ERR_STATE, "correction outside the ring (dir %d)", d);
@@ -346,16 +346,15 @@ void macro_constants(const MacroGeom& G, int n, double c_eps, double c_div, Macr
     out.sb[d][6] = out.st.C[d];
     out.sb[d][7] = 0;
   }
-  out.pad[0] = out.pad[1] = 0;
 }
 
 // the centre terms of B, B^T and C at a macro-interior node, from the 24 elements around it
-void check_stokes_row_sums(const MacroConsts<double>& mc) {
+void check_stokes_row_sums(const MacroConsts<double>& mc, const ElementMatrices& em) {
   double b0[3] = {0, 0, 0}, c0 = 0, scale = 0;
   for (int p = 0; p < 6; ++p)
     for (int a = 0; a < 4; ++a) {
-      for (int l = 0; l < 3; ++l) b0[l] += mc.bd[p][a][a][l];
-      c0 += mc.lc[p][a][a];
+      for (int l = 0; l < 3; ++l) b0[l] += em.bd[p][a][a][l];
+      c0 += em.lc[p][a][a];
     }
   double sb[3] = {b0[0], b0[1], b0[2]}, sg[3] = {b0[0], b0[1], b0[2]}, sc = c0;
   for (int d = 0; d < NDIR; ++d) {
@@ -372,14 +371,13 @@ void check_stokes_row_sums(const MacroConsts<double>& mc) {
   if (std::fabs(sc) > 1e-12 * (std::fabs(c0) + 1e-300)) THROW(HHG_ERR_STATE, "stabilisation row sum");
 }
 
-template <typename T>
-MacroConsts<T> cast_consts(const MacroConsts<double>& c) {
-  MacroConsts<T> o;
+// rounded to FP32, value by value (both precisions have the same layout)
+template <template <typename> class S>
+void cast_values(const S<double>& c, S<float>& o) {
+  static_assert(sizeof(S<double>) == 2 * sizeof(S<float>), "layout");
   const double* s = (const double*)&c;
-  T* d = (T*)&o;
-  static_assert(sizeof(MacroConsts<double>) / sizeof(double) == sizeof(MacroConsts<T>) / sizeof(T), "layout");
-  for (size_t q = 0; q < sizeof(MacroConsts<double>) / sizeof(double); ++q) d[q] = (T)s[q];
-  return o;
+  float* d = (float*)&o;
+  for (size_t q = 0; q < sizeof(S<double>) / sizeof(double); ++q) d[q] = (float)s[q];
 }
 
 
@@ -1110,6 +1108,7 @@ hhg_status hhg_set_problem(hhg_ctx* c, const hhg_problem* p) {
       const int M = (int)c->tets.size();
       std::vector<MacroConsts<double>> mc64(M);
       std::vector<MacroConsts<float>> mc32(M);
+      std::vector<ElementMatrices> em(M);
       L.st64.resize(M);
       L.st32.resize(M);
       L.nc64.resize(M);
@@ -1117,13 +1116,13 @@ hhg_status hhg_set_problem(hhg_ctx* c, const hhg_problem* p) {
       for (int m = 0; m < M; ++m) {
         MacroGeom G;
         for (int q = 0; q < 4; ++q) G.v[q] = c->xyz[c->tets[m][q]];
-        macro_constants(G, L.n, ce, cd, mc64[m]);
-        check_stokes_row_sums(mc64[m]);
-        mc32[m] = cast_consts<float>(mc64[m]);
+        macro_constants(G, L.n, ce, cd, em[m], mc64[m]);
+        check_stokes_row_sums(mc64[m], em[m]);
+        cast_values(mc64[m], mc32[m]);
         L.st64[m] = mc64[m].st;
         L.st32[m] = mc32[m].st;
-        std::memcpy(L.nc64[m].ke, mc64[m].ke, sizeof(L.nc64[m].ke));
-        std::memcpy(L.nc32[m].ke, mc32[m].ke, sizeof(L.nc32[m].ke));
+        L.nc64[m] = em[m].ke;
+        cast_values(em[m].ke, L.nc32[m]);
       }
       upload(L.d_mc64, mc64);
       upload(L.d_mc32, mc32);
@@ -1146,7 +1145,7 @@ hhg_status hhg_set_problem(hhg_ctx* c, const hhg_problem* p) {
         std::vector<double> dint(M, 0.0);
         for (int m = 0; m < M; ++m)
           for (int pp = 0; pp < 6; ++pp)
-            for (int av = 0; av < 4; ++av) dint[m] -= mc64[m].lc[pp][av][av];
+            for (int av = 0; av < 4; ++av) dint[m] -= em[m].lc[pp][av][av];
         for (int m = 0; m < M; ++m)
           for (int64_t q = 0; q < L.nt; ++q) {
             const int64_t u = L.entry_to_unique[(int64_t)m * L.nt + q];
@@ -1157,7 +1156,7 @@ hhg_status hhg_set_problem(hhg_ctx* c, const hhg_problem* p) {
             const SkelInc& I = L.skel_inc[q];
             for (int pp = 0; pp < 6; ++pp)
               for (int av = 0; av < 4; ++av)
-                if (inside(I.i, I.j, I.k, pp, av)) du[nint + sk] -= mc64[I.macro].lc[pp][av][av];
+                if (inside(I.i, I.j, I.k, pp, av)) du[nint + sk] -= em[I.macro].lc[pp][av][av];
           }
         std::vector<double> d64(L.entries);
         for (int64_t e = 0; e < L.entries; ++e) d64[e] = du[L.entry_to_unique[e]];

@@ -153,12 +153,6 @@ struct MacroStencil {
   T C[NDIR];
 };
 
-// Constants of one macro for the skeleton kernel (global memory): the interior
-// stencil plus the 6 element stiffness matrices K[type][a][b][m][l] (test
-// vertex a, trial vertex b) of the Kuhn element types.
-// Element matrices for the Stokes blocks: bd[type][a][b][l] = -int phi_a d_l phi_b
-// (pressure test vertex a, velocity trial vertex b), lc[type][a][b] = -(h^2/12) int
-// grad phi_a . grad phi_b.
 // Element stiffness of one macro's 6 Kuhn element types for the nodal-integration
 // interior kernel (kernel parameter, 864 values): ke[type][a][b][3 m + l].
 template <typename T>
@@ -166,6 +160,7 @@ struct NodalConsts {
   T ke[6][4][4][9];
 };
 
+// Constants of one macro in global memory, for the sweeps.
 // el[d][e]: element e of the edge (0, d), the one whose other two vertices are the ring nodes e and
 // e + 1 of the edge in cyclic order (ring_cyc), as seen by the row of point 0: the 3x3 block
 // (test vertex 0, trial vertex d), then bd(0, d), bd(d, 0) and lc(0, d).
@@ -180,9 +175,6 @@ struct alignas(16) MacroConsts {
   // (ring_cyc 0 and 2; 0 and 1 of a four-element edge), B, G, C
   T mar[7][20];
   MacroStencil<T> st;
-  T ke[6][4][4][9];
-  T bd[6][4][4][3];
-  T lc[6][4][4];
   T pad[2];  // a whole number of 16-byte words in FP32 as in FP64
 };
 static_assert(sizeof(MacroConsts<float>) % 16 == 0 && sizeof(MacroConsts<double>) == 2 * sizeof(MacroConsts<float>),
