@@ -231,9 +231,18 @@ __global__ void __launch_bounds__(GSM_BLOCK) k_gs_macro(const LevelDev L, const 
 
 constexpr int GS_MAX_MACROS = 65535;  // grid.y
 
-// Which form, by points of a colour over all macros.  48 macros in FP64, a whole smoothing step (skeleton
-// rows and 8 colours): 8 intervals per macro edge (210 points) 68-72 us in one launch against 197 in
-// eight, 16 (2730) 113-119 against 205, 32 (27,000) 581 against 322.
+// Which form.  k_gs_macro takes parts * GSM_BLOCK / 8 points of a macro at a time, in rounds that follow one
+// another, so it takes the levels whose colours fit a few rounds, and of those the ones that do not fill
+// the chip (95 against 70 FP64 instructions per four points).  A smoothing step (skeleton rows and 8 colours)
+// in FP64 / FP32, us, in one launch and in eight:
+//   rounds  macros x intervals per edge        one launch    eight launches
+//   1       48 x 8 (10 points a colour)        74 / 27       204 / 62
+//   2       48 x 16 (84)                       124 / 39      216 / 64
+//   3       6 x 32 (680)                       207 / 59      199 / 62
+//   3       96 x 16 (84)                       193 / 45      251 / 66
+//   6       24 x 32 (680)                      345 / 86      236 / 63
+//   22      1 x 64 (5456)                      1125 / 251    175 / 60
+constexpr int GS_MACRO_MAX_ROUNDS = 3;
 constexpr int64_t GS_MACRO_MAX_POINTS = 12000;
 
 }  // namespace
@@ -276,11 +285,11 @@ int launch_gs(const LevelDev& L, const MacroConsts<T>* mc, const OpFlags& fl, co
   for (int c = 0; c < 8; ++c) most = std::max(most, L.gs_ptr[c + 1] - L.gs_ptr[c]);
   for (int m0 = 0; m0 < L.nmacro; m0 += GS_MAX_MACROS) {
     const int nm = std::min(GS_MAX_MACROS, L.nmacro - m0);
-    if ((int64_t)most * L.nmacro <= GS_MACRO_MAX_POINTS) {
-      // blocks per macro: enough for the largest colour, no more than share the SMs, a power of two up
-      // to 8 (three blocks per macro were slower than two: 118 against 73 us on 48 macros)
-      int parts = 1;
-      while (parts < 8 && parts * (GSM_BLOCK / 8) < most && 2 * parts * L.nmacro <= 152) parts *= 2;
+    // blocks per macro: enough for the largest colour, no more than share the SMs, a power of two up
+    // to 8 (three blocks per macro were slower than two: 118 against 73 us on 48 macros)
+    int parts = 1;
+    while (parts < 8 && parts * (GSM_BLOCK / 8) < most && 2 * parts * L.nmacro <= 152) parts *= 2;
+    if (most <= GS_MACRO_MAX_ROUNDS * parts * (GSM_BLOCK / 8) && (int64_t)most * L.nmacro <= GS_MACRO_MAX_POINTS) {
       cudaLaunchConfig_t cfg = {};
       cfg.gridDim = dim3(parts, nm);
       cfg.blockDim = dim3(GSM_BLOCK);
