@@ -101,8 +101,8 @@ struct KeyHash {
 struct LevelHost {
   int level = 0, n = 0;
   int64_t nt = 0, entries = 0;
-  std::vector<int32_t> tiles_int, tiles_all, tiles_lin, tiles_pair, tiles3, gs_points, columns;
-  int32_t column_len = 1;
+  std::vector<int32_t> tiles_int, tiles_all, tiles_lin, tiles_pair, tiles3, gs_points, columns[2];
+  int32_t column_len[2] = {1, 1};  // FP32, FP64
   int32_t gs_ptr[9] = {0};
   std::vector<int64_t> skel_entries;
   std::vector<int32_t> skel_ptr;
@@ -128,7 +128,7 @@ struct LevelHost {
   std::vector<int64_t> rent;
   std::vector<double> rw;
   // device
-  DevMem d_columns, d_tiles_pair, d_tiles3, d_gs_points, d_skel_entries;
+  DevMem d_columns[2], d_tiles_pair, d_tiles3, d_gs_points, d_skel_entries;
   DevMem d_tiles_int, d_tiles_all, d_tiles_lin, d_skel_ptr, d_skel_inc, d_skel_dir, d_mask, d_first, d_e2u;
   DevMem d_ev_warps[2], d_edge_blocks[2], d_edge_sides[2], d_face_blocks[2], d_face_points[2], d_dir_entries;
   DevMem d_mask_own, d_invm64, d_invm32;  // owned-node mask; inverse lumped mass
@@ -342,7 +342,8 @@ inline int64_t max_partials(hhg_ctx* c) {
   int64_t mx = 2 * 1024;
   for (int l = c->level_min; l <= c->level_max; ++l) {
     const LevelHost& L = *c->levels[l];
-    mx = std::max<int64_t>(mx, (int64_t)std::max({L.tiles_lin.size(), L.tiles3.size(), (L.columns.size() + 127) / 128}) * (int64_t)c->tets.size() +
+    const size_t columns = std::max(L.columns[0].size(), L.columns[1].size());
+    mx = std::max<int64_t>(mx, (int64_t)std::max({L.tiles_lin.size(), L.tiles3.size(), (columns + 127) / 128}) * (int64_t)c->tets.size() +
                                    (int64_t)std::max(L.ev_warps[0].size() / 4 + L.edge_blocks[0].size() + L.face_blocks[0].size(),
                                                      L.ev_warps[1].size() / 4 + L.edge_blocks[1].size() + L.face_blocks[1].size()) + 8);
   }

@@ -510,16 +510,22 @@ void build_level(hhg_ctx* c, int level) {
   {
     const int64_t points = (int64_t)M * (n >= 4 ? tetnum(n - 3) : 0);
     // length: the longer, the less the loads before a column's first point weigh (44 of 28 per
-    // point), but the fewer columns there are; about 3.5 columns per thread that fits the GPU (152
-    // SMs x 512) leave no large last wave.  FP32 apply on 129^3 / 257^3 nodes: length 4 61 / 432
-    // us, 8 61 / 405, 16 67 / 391; FP64 residual on 129^3: 4 1.76 ms, 8 1.83; V-cycle: at least 2
-    // on its coarse levels (1.01 ms; 1: 1.02, 4: 1.03)
+    // point), but the fewer columns there are.
+    // FP32: about 3.5 columns per thread that fits the GPU (152 SMs x 512) leave no large last wave.
+    // FP32 apply on 129^3 / 257^3 nodes: length 4 57 / 433 us, 8 57 / 397, 16 62 / 387; V-cycle: at least
+    // 2 on its coarse levels (1.01 ms; 1: 1.02, 4: 1.03).
+    // FP64: a point's chain of FP64 instructions is 16 us, and the edge before a column's first point a
+    // quarter of it, so short columns.  FP64 apply, length 1 / 2 / 4, us: one macro of 33^3 / 6 nodes 21 /
+    // 37 / 68, six of them 44 / 66 / 125, cube of 65^3 nodes 234 / 244 / 270, of 129^3 1742 / 1705 / 1708,
+    // of 257^3 13768 / 13355 / 13128.
     int len = 2;
     while (len < 16 && 2 * points > 7 * (2 * len) * (int64_t)152 * 512) len *= 2;
-    L->column_len = len;
-    for (int cc = 2; cc <= n - 2; ++cc)
-      for (int k0 = 1; k0 <= cc - 1; k0 += len)
-        for (int i = 1; i <= n - 1 - cc; ++i) L->columns.push_back((cc << 20) | (k0 << 10) | i);
+    L->column_len[0] = len;
+    L->column_len[1] = points <= 300000 ? 1 : points <= 4000000 ? 2 : 4;
+    for (int q = 0; q < 2; ++q)
+      for (int cc = 2; cc <= n - 2; ++cc)
+        for (int k0 = 1; k0 <= cc - 1; k0 += L->column_len[q])
+          for (int i = 1; i <= n - 1 - cc; ++i) L->columns[q].push_back((cc << 20) | (k0 << 10) | i);
   }
   // boxes of TILE3_I x TILE3_J x TILE3_K lattice points (i, j, k) with at least one
   // macro-interior point, for the shared-memory tile kernel
@@ -721,7 +727,7 @@ void upload_level(hhg_ctx* c, LevelHost& L) {
   upload(L.d_tiles_int, L.tiles_int);
   upload(L.d_tiles_all, L.tiles_all);
   upload(L.d_tiles_lin, L.tiles_lin);
-  upload(L.d_columns, L.columns);
+  for (int q = 0; q < 2; ++q) upload(L.d_columns[q], L.columns[q]);
   upload(L.d_tiles_pair, L.tiles_pair);
   upload(L.d_tiles3, L.tiles3);
   upload(L.d_gs_points, L.gs_points);
@@ -774,9 +780,11 @@ void upload_level(hhg_ctx* c, LevelHost& L) {
   D.tiles_all = L.d_tiles_all.as<int32_t>();
   D.ntiles_lin = (int32_t)L.tiles_lin.size();
   D.tiles_lin = L.d_tiles_lin.as<int32_t>();
-  D.ncolumns = (int32_t)L.columns.size();
-  D.column_len = L.column_len;
-  D.columns = L.d_columns.as<int32_t>();
+  for (int q = 0; q < 2; ++q) {
+    D.ncolumns[q] = (int32_t)L.columns[q].size();
+    D.column_len[q] = L.column_len[q];
+    D.columns[q] = L.d_columns[q].as<int32_t>();
+  }
   D.ntiles_pair = (int32_t)L.tiles_pair.size();
   D.tiles_pair = L.d_tiles_pair.as<int32_t>();
   D.ntiles3 = (int32_t)L.tiles3.size();

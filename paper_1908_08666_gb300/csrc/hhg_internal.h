@@ -234,10 +234,10 @@ struct LevelDev {
   const int32_t* tiles_lin;
   int32_t ntiles_pair;  // 128-pair chunks of the point pairs of each slice (FP32 sweeps): (k << 20) | start
   const int32_t* tiles_pair;
-  // columns of the marching kernel: (c << 20) | (k0 << 10) | i, the points (i, c - k, k), k = k0 ..
-  // min(k0 + column_len, c) - 1
-  int32_t ncolumns, column_len;
-  const int32_t* columns;
+  // columns of the marching kernel in FP32 [0] and FP64 [1]: (c << 20) | (k0 << 10) | i, the points
+  // (i, c - k, k), k = k0 .. min(k0 + column_len, c) - 1
+  int32_t ncolumns[2], column_len[2];
+  const int32_t* columns[2];
   int32_t ntiles3;      // boxes of the shared-memory tile kernel: (k0 << 20) | (j0 << 10) | i0
   const int32_t* tiles3;
   // hybrid Gauss-Seidel: the macro-interior points (k << 20) | (j << 10) | i of each colour

@@ -269,7 +269,7 @@ struct March {
   T pprev;  // (Stokes) pressure of the column's previous point
 };
 
-// A block of columns of one macro (LevelDev::columns); cst: 7 MARCH_C values.
+// A block of columns of one macro (LevelDev::columns, FP64); cst: 7 MARCH_C values.
 template <typename T, int OP, int GEN, int STK>
 __device__ __forceinline__ void march_block(const LevelDev& L, const MacroConsts<T>* __restrict__ mc, const int macro,
                                             const int block, const OpFlags& fl, const SweepArgs<T>& a, T* cst,
@@ -281,12 +281,12 @@ __device__ __forceinline__ void march_block(const LevelDev& L, const MacroConsts
   __syncthreads();
   const int t = block * MARCH_BLOCK + threadIdx.x;
   double r2 = 0.0;
-  if (t < L.ncolumns) {
-    const int32_t col = L.columns[t];
+  if (t < L.ncolumns[1]) {
+    const int32_t col = L.columns[1][t];
     const int n = L.n;
     const int c = col >> 20, i = col & 0x3FF;
     int k = (col >> 10) & 0x3FF;
-    const int kend = min(k + L.column_len, c);
+    const int kend = min(k + L.column_len[1], c);
     March<T, OP, GEN, STK> M;
     const int64_t base = (int64_t)macro * L.nt;
     M.E = L.entries;
@@ -553,12 +553,12 @@ __device__ __forceinline__ void march2_block(const LevelDev& L, const MacroConst
   __syncthreads();
   const int t = block * MARCH_BLOCK + threadIdx.x;
   double r2 = 0.0;
-  if (t < L.ncolumns) {
-    const int32_t col = L.columns[t];
+  if (t < L.ncolumns[0]) {
+    const int32_t col = L.columns[0][t];
     const int n = L.n;
     const int c = col >> 20, i = col & 0x3FF;
     int k = (col >> 10) & 0x3FF;
-    const int kend = min(k + L.column_len, c);
+    const int kend = min(k + L.column_len[0], c);
     March2<OP, GEN, STK, KB> M;
     constexpr int NF = STK ? 5 : 4;
     const int64_t base = (int64_t)macro * L.nt;
@@ -652,8 +652,9 @@ int launch(const LevelDev& L, const MacroConsts<T>* mc, const OpFlags& fl, const
            int64_t* partial_count) {
   const bool gen = !(fl.physical == 1 && fl.khat_edge == 0);
   const RowBlocks<T, STK> R(L);
-  const int per = std::max(1, (L.ncolumns + MARCH_BLOCK - 1) / MARCH_BLOCK);
-  const int64_t inner = L.ncolumns > 0 ? (int64_t)per * L.nmacro : 0;
+  const int columns = L.ncolumns[sizeof(T) == 8];
+  const int per = std::max(1, (columns + MARCH_BLOCK - 1) / MARCH_BLOCK);
+  const int64_t inner = columns > 0 ? (int64_t)per * L.nmacro : 0;
   if (partial_count) *partial_count = inner + R.partials();
   if (inner + R.total == 0) return 0;
   if (inner + R.total > INT32_MAX) return (int)cudaErrorInvalidValue;

@@ -1,0 +1,113 @@
+"""The one-launch sweep where its layout changes with the level: columns of one, two and more points in FP64 and
+of more than two in FP32.  Against the interior kernels of hhg_set_interior_kernel (which share the skeleton
+rows).
+
+Tolerances.  FP64: two sums of the same terms, 1e-11 of the largest value as in test_gpu_rows.py.  FP32: the
+rounding bound of test_gpu_parity.py is 64 2^-24 sum_j |A_ij| |x_j - x_i|; for random x the 42 terms of a row
+sum to at most sqrt(42) < 10 times their root mean square, and the largest |A x| of many rows is at least
+that; twice the bound, since both sides round."""
+
+import pytest
+
+import hhg_inputs as hi
+from paper_1908_08666_gb300 import binding as B
+
+from hhg_gpu import Ctx
+from test_gpu_parity import FP32_C, _kfun
+
+pytestmark = pytest.mark.gpu
+
+F64, F32 = 1e-11, 2 * 10 * FP32_C
+
+
+def _close(got, want, comps, tol):
+    for g, w in zip(got.double().reshape(comps, -1), want.double().reshape(comps, -1)):
+        assert (g - w).abs().max().item() <= tol * w.abs().max().item()
+
+
+def _sweeps(ctx, comps, dt, tdt, tol, kernels):
+    """apply, residual and its norm of kernel 0 against the others'"""
+    t, l = ctx.torch, ctx.level
+    x = ctx.to_lib(hi.node_noise(ctx.coords_u, seed=3, comps=comps), tdt, comps)
+    f = ctx.to_lib(hi.node_noise(ctx.coords_u, seed=4, comps=comps), tdt, comps)
+    ap, re = (B.hhg_apply, B.hhg_residual) if comps == 3 else (B.hhg_stokes_apply, B.hhg_stokes_residual)
+    out = []
+    for kernel in kernels:
+        B.hhg_set_interior_kernel(ctx.h, kernel)
+        y, r = t.full_like(x, 7.0), t.full_like(x, 7.0)
+        ap(ctx.h, l, dt, x, y)
+        out.append((y, r, re(ctx.h, l, dt, f, x, r, want_norm=True)))
+    B.hhg_set_interior_kernel(ctx.h, 0)
+    for y, r, norm2 in out[1:]:
+        _close(out[0][0], y, comps, tol)
+        _close(out[0][1], r, comps, tol)
+        assert abs(out[0][2] - norm2) <= 2 * tol * norm2
+    return x, f
+
+
+@pytest.mark.parametrize("builder,level", [(hi.kuhn_cube, 3), (hi.unit_tet, 2), (hi.unit_tet, 4), (hi.unit_tet, 7)],
+                         ids=["cube_l3", "one_l2", "one_l4", "one_l7"])
+@pytest.mark.parametrize("problem", [{}, dict(khat=B.KHAT_EDGE), dict(kind=B.STOKES)],
+                         ids=["elasticity", "edge", "stokes"])
+def test_sweeps_equal_interior_kernels(builder, level, problem):
+    ctx = Ctx(*builder(), level, problem)
+    try:
+        ctx.set_k(_kfun(ctx.coords_u))
+        comps = 4 if "kind" in problem else 3
+        for dt, tdt, tol in ((B.F64, ctx.torch.float64, F64), (B.F32, ctx.torch.float32, F32)):
+            _sweeps(ctx, comps, dt, tdt, tol, (0, 3))
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("problem", [{}, dict(khat=B.KHAT_EDGE), dict(variant=B.UNPHYSICAL), dict(kind=B.STOKES)],
+                         ids=["elasticity", "edge", "unphysical", "stokes"])
+def test_long_columns(problem):
+    """129^3 nodes: columns of four points in FP32 and two in FP64, every epilogue."""
+    ctx = Ctx(*hi.kuhn_cube(), 7, problem)
+    try:
+        t = ctx.torch
+        ctx.set_k(_kfun(ctx.coords_u))
+        comps = 4 if "kind" in problem else 3
+        for dt, tdt, tol in ((B.F64, t.float64, F64), (B.F32, t.float32, F32)):
+            x, f = _sweeps(ctx, comps, dt, tdt, tol, (0, 3))
+            if comps == 4:
+                continue
+            B.hhg_mg_setup(ctx.h)
+            d = []
+            for kernel in (0, 3):
+                B.hhg_set_interior_kernel(ctx.h, kernel)
+                d.append(t.full_like(x, 7.0))
+                B.hhg_diagonal(ctx.h, 7, dt, d[-1])
+            _close(d[0], d[1], 3, tol)
+            for smoother in (B.SMOOTH_CHEBYSHEV, B.SMOOTH_JACOBI):
+                B.hhg_set_mg_params(ctx.h, smoother=smoother)
+                out = []
+                for kernel in (0, 3):
+                    B.hhg_set_interior_kernel(ctx.h, kernel)
+                    out.append(x.clone())
+                    B.hhg_smooth(ctx.h, 7, dt, 2, f * 1e-3, out[-1])
+                t.cuda.synchronize()
+                _close(out[0], out[1], 3, tol)
+    finally:
+        ctx.close()
+
+
+def test_long_columns_bf16_coefficient():
+    ctx = Ctx(*hi.kuhn_cube(), 7, dict(nu=0.3))
+    try:
+        t = ctx.torch
+        k = ctx.to_lib(_kfun(ctx.coords_u), t.float64, 1)
+        B.hhg_set_coefficient(ctx.h, k.to(t.bfloat16), B.BF16)
+        _sweeps(ctx, 3, B.F32, t.float32, F32, (0, 3))
+    finally:
+        ctx.close()
+
+
+def test_columns_of_four_points_in_fp64():
+    ctx = Ctx(*hi.skewed_pair(), 8, dict(nu=0.3))
+    try:
+        ctx.set_k(_kfun(ctx.coords_u))
+        _sweeps(ctx, 3, B.F64, ctx.torch.float64, F64, (0, 3))
+    finally:
+        ctx.close()
