@@ -386,9 +386,14 @@ void cast_values(const S<double>& c, S<float>& o) {
 // of incidences (two per warp and round, two rounds), the widest first (they run longest); nodes inside a
 // macro edge lie in the same macros and are numbered along it; nodes inside faces are ordered by macros and
 // face types, those next to the face's edges apart.  A face block has two sides, so the nodes of a face in
-// more than two macros (the mesh need not be a manifold) go to the vertices' list.
+// more than two macros (the mesh need not be a manifold) go to the vertices' list, and so do faces and edges of
+// up to VERTEX_LIKE nodes: three lanes of a block's 32 were busy there.  Apply on 3072 macros of 4 intervals per
+// edge, FP32 / FP64, us: elasticity 71 / 831 with blocks, 57 / 410 so, Stokes 123 / 1276 and 82 / 592; with
+// the edges of 8 intervals (7 nodes) too, elasticity on 3072 of those 98 / 1261 and 136 / 1367.
+constexpr int VERTEX_LIKE = 3;
 void build_rows(LevelHost& L) {
   const int n = L.n;
+  const bool edge_blocks = n - 1 > VERTEX_LIKE, face_blocks = (n - 1) * (n - 2) / 2 > VERTEX_LIKE;
   const int64_t nskel = (int64_t)L.skel_dir.size();
   auto primitive = [&](const SkelInc& I) {
     return (I.i + I.j + I.k == n ? 1 : 0) | (I.i == 0 ? 2 : 0) | (I.j == 0 ? 4 : 0) | (I.k == 0 ? 8 : 0);
@@ -406,7 +411,7 @@ void build_rows(LevelHost& L) {
     std::map<std::array<int64_t, 2>, std::vector<std::pair<int64_t, int64_t>>> edges;  // vertices -> (weight, node)
     for (int64_t s = 0; s < nskel; ++s) {
       if (L.skel_dir[s] && !stk) continue;
-      if (L.skel_support[s] == 2) {
+      if (L.skel_support[s] == 2 && edge_blocks) {
         const std::array<int64_t, 3>& key = L.skel_key[s];
         edges[{key[0] / 4096, key[1] / 4096}].push_back({key[0] % 4096, s});
         continue;
@@ -421,7 +426,7 @@ void build_rows(LevelHost& L) {
       const SkelInc& I = L.skel_inc[b0];
       if (L.skel_support[s] == 3)
         for (const int w : {n - I.i - I.j - I.k, (int)I.i, (int)I.j, (int)I.k}) q.near |= w == 1;
-      (L.skel_support[s] == 3 && ni <= 2 ? faces : keys).push_back(q);
+      (L.skel_support[s] == 3 && ni <= 2 && face_blocks ? faces : keys).push_back(q);
     }
     for (auto& ed : edges) {
       std::sort(ed.second.begin(), ed.second.end());

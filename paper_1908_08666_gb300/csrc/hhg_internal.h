@@ -187,10 +187,10 @@ struct SkelInc {
   int16_t pad;
 };
 
-// Rows of macro vertices: half a warp takes an incidence, `warps` warps of a block a
-// node.  EvWarp: what a warp of a block does (first < 0: nothing): `count` incidences of the node from
-// skel_inc[first] on, of which it takes 2 w, 2 w + 1, 2 (w + warps), ...; the block's warps
-// w0 .. w0 + warps - 1 share the node.
+// Rows of macro vertices (and of the other nodes that build_rows adds to them): half a warp takes an
+// incidence, `warps` warps of a block a node.  EvWarp: what a warp of a block does (first < 0: nothing):
+// `count` incidences of the node from skel_inc[first] on, of which it takes 2 w, 2 w + 1, 2 (w + warps), ...;
+// the block's warps w0 .. w0 + warps - 1 share the node.
 struct EvWarp {
   int32_t first, count;
   int16_t vdir, w, w0, warps;

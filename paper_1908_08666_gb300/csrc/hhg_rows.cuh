@@ -13,8 +13,9 @@
 //
 // Nodes inside a macro face or edge: what depends on the direction is fixed by the kind of face or edge
 // that the macro sees (prim_incidence, unrolled over the directions); a lane per node, all lanes of a warp
-// in the same macro.  Vertices, with up to dozens of macros: incidence_lane, half a warp per macro, a lane
-// per direction, the ring's coefficients by shuffles.
+// in the same macro.  Vertices, with up to dozens of macros, and the few nodes of faces and edges on the
+// coarsest level: incidence_lane, half a warp per macro, a lane per direction, the ring's coefficients by
+// shuffles.
 //
 // What bounds them: latency, and on meshes of many macros instructions.  There are few such nodes (2 % of
 // 129^3), but most of a face's or edge's neighbours lie in different rows.  FP32 apply on 384 macros at

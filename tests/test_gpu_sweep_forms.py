@@ -1,19 +1,21 @@
-"""The one-launch sweep where its layout changes with the level: columns of one, two and more points in FP64 and
-of more than two in FP32.  Against the interior kernels of hhg_set_interior_kernel (which share the skeleton
-rows).
+"""The one-launch sweep where its layout changes with the level: faces and edges of few nodes, columns
+of one, two and more points in FP64 and of more than two in FP32.  Against the interior kernels of
+hhg_set_interior_kernel (which share the skeleton rows), and on coarse levels against the oracle.
 
 Tolerances.  FP64: two sums of the same terms, 1e-11 of the largest value as in test_gpu_rows.py.  FP32: the
 rounding bound of test_gpu_parity.py is 64 2^-24 sum_j |A_ij| |x_j - x_i|; for random x the 42 terms of a row
 sum to at most sqrt(42) < 10 times their root mean square, and the largest |A x| of many rows is at least
 that; twice the bound, since both sides round."""
 
+import numpy as np
 import pytest
 
 import hhg_inputs as hi
+from oracle import mesh, operators as op
 from paper_1908_08666_gb300 import binding as B
 
 from hhg_gpu import Ctx
-from test_gpu_parity import FP32_C, _kfun
+from test_gpu_parity import FP32_C, _fp32_scale, _kfun, _oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -45,8 +47,9 @@ def _sweeps(ctx, comps, dt, tdt, tol, kernels):
     return x, f
 
 
-@pytest.mark.parametrize("builder,level", [(hi.kuhn_cube, 3), (hi.unit_tet, 2), (hi.unit_tet, 4), (hi.unit_tet, 7)],
-                         ids=["cube_l3", "one_l2", "one_l4", "one_l7"])
+@pytest.mark.parametrize("builder,level", [(hi.kuhn_cube, 2), (hi.kuhn_cube, 3), (hi.unit_tet, 2), (hi.unit_tet, 4),
+                                           (hi.unit_tet, 7)],
+                         ids=["cube_l2", "cube_l3", "one_l2", "one_l4", "one_l7"])
 @pytest.mark.parametrize("problem", [{}, dict(khat=B.KHAT_EDGE), dict(kind=B.STOKES)],
                          ids=["elasticity", "edge", "stokes"])
 def test_sweeps_equal_interior_kernels(builder, level, problem):
@@ -56,6 +59,35 @@ def test_sweeps_equal_interior_kernels(builder, level, problem):
         comps = 4 if "kind" in problem else 3
         for dt, tdt, tol in ((B.F64, ctx.torch.float64, F64), (B.F32, ctx.torch.float32, F32)):
             _sweeps(ctx, comps, dt, tdt, tol, (0, 3))
+    finally:
+        ctx.close()
+
+
+@pytest.mark.parametrize("count,level", [(2, 2), (3, 2)])
+def test_coarse_rows_match_oracle(count, level):
+    """Faces and edges of three nodes, on 48 and on 162 macros."""
+    xyz, tets = hi.kuhn_cube(count)
+    mm, lv, A = _oracle(xyz, tets, level, _kfun)
+    ctx = Ctx(xyz, tets, level, dict(nu=0.3))
+    try:
+        t = ctx.torch
+        perm = mesh.match_nodes(lv.coords, ctx.coords_u)
+        ctx.set_k(_kfun(ctx.coords_u))
+        x_or = hi.node_noise(lv.coords, seed=7)
+        x_u = np.empty_like(x_or)
+        x_u[perm] = x_or
+        y_or = op.apply(op.with_dirichlet_rows(A, lv.dirichlet), x_or)
+        scale, free = _fp32_scale(A, x_or, lv), ~lv.dirichlet
+        for dt, tdt in ((B.F64, t.float64), (B.F32, t.float32)):
+            x = ctx.to_lib(x_u, tdt, 3)
+            y = t.full_like(x, 7.0)
+            B.hhg_apply(ctx.h, level, dt, x, y)
+            yg = ctx.from_lib(y, 3)
+            assert np.array_equal(y.double().cpu().numpy().reshape(3, ctx.E).T, yg[ctx.e2u])
+            if dt == B.F64:
+                assert np.abs(yg[perm] - y_or).max() <= 1e-12 * np.abs(y_or).max()
+            else:
+                assert np.all(np.abs(yg[perm] - y_or)[free] <= FP32_C * scale[free] + 1e-30)
     finally:
         ctx.close()
 
