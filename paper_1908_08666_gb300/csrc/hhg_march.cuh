@@ -269,17 +269,20 @@ struct March {
   T pprev;  // (Stokes) pressure of the column's previous point
 };
 
-// A block of columns of one macro (LevelDev::columns, FP64); cst: 7 MARCH_C values.
+// A block of columns of one macro (LevelDev::columns, FP64), or part of a block of several macros'
+// columns: `threads` threads, a power of two.  cst: 7 MARCH_C values, of this macro's threads.
 template <typename T, int OP, int GEN, int STK>
 __device__ __forceinline__ void march_block(const LevelDev& L, const MacroConsts<T>* __restrict__ mc, const int macro,
-                                            const int block, const OpFlags& fl, const SweepArgs<T>& a, T* cst,
-                                            double* partial) {
-  for (int q = threadIdx.x; q < 7 * MARCH_C<STK>; q += MARCH_BLOCK) {
-    const int d = q / MARCH_C<STK>, r = q - d * MARCH_C<STK>;
-    cst[q] = __ldg(&mc[macro].mar[d][r]);
-  }
+                                            const int block, const int threads, const OpFlags& fl,
+                                            const SweepArgs<T>& a, T* cst, double* partial) {
+  const int own = threadIdx.x & (threads - 1);
+  if (macro < L.nmacro)
+    for (int q = own; q < 7 * MARCH_C<STK>; q += threads) {
+      const int d = q / MARCH_C<STK>, r = q - d * MARCH_C<STK>;
+      cst[q] = __ldg(&mc[macro].mar[d][r]);
+    }
   __syncthreads();
-  const int t = block * MARCH_BLOCK + threadIdx.x;
+  const int t = macro < L.nmacro ? block * threads + own : INT32_MAX;
   double r2 = 0.0;
   if (t < L.ncolumns[1]) {
     const int32_t col = L.columns[1][t];
@@ -544,14 +547,16 @@ struct March2 {
 // As march_block; cst: 7 MARCH2_C values.
 template <int OP, int GEN, int STK, int KB>
 __device__ __forceinline__ void march2_block(const LevelDev& L, const MacroConsts<float>* __restrict__ mc,
-                                             const int macro, const int block, const OpFlags& fl,
+                                             const int macro, const int block, const int threads, const OpFlags& fl,
                                              const SweepArgs<float>& a, float* cst, double* partial) {
-  for (int r = threadIdx.x; r < 7 * MARCH2_C<STK>; r += MARCH_BLOCK) {
-    const int d = r / MARCH2_C<STK>, w = r - d * MARCH2_C<STK>;
-    cst[r] = w < 8 ? (w < 6 ? __ldg(&mc[macro].mar[d][w]) : 0.0f) : __ldg(&mc[macro].mar[d][6 + (w - 8) / 2]);
-  }
+  const int own = threadIdx.x & (threads - 1);
+  if (macro < L.nmacro)
+    for (int r = own; r < 7 * MARCH2_C<STK>; r += threads) {
+      const int d = r / MARCH2_C<STK>, w = r - d * MARCH2_C<STK>;
+      cst[r] = w < 8 ? (w < 6 ? __ldg(&mc[macro].mar[d][w]) : 0.0f) : __ldg(&mc[macro].mar[d][6 + (w - 8) / 2]);
+    }
   __syncthreads();
-  const int t = block * MARCH_BLOCK + threadIdx.x;
+  const int t = macro < L.nmacro ? block * threads + own : INT32_MAX;
   double r2 = 0.0;
   if (t < L.ncolumns[0]) {
     const int32_t col = L.columns[0][t];
@@ -623,12 +628,12 @@ __device__ __forceinline__ void march2_block(const LevelDev& L, const MacroConst
 template <typename T, int OP, int GEN, int STK, int KB>
 __global__ void __launch_bounds__(MARCH_BLOCK, sizeof(T) == 4 ? 4 : 2)
     k_sweep(const LevelDev L, const MacroConsts<T>* __restrict__ mc, const OpFlags fl, const SweepArgs<T> a,
-            const int per_macro, const int rows) {
+            const int per_macro, const int threads, const int rows) {
   constexpr int NC = 7 * (sizeof(T) == 4 ? MARCH2_C<STK> : MARCH_C<STK>);
   __shared__ union U {
     RowScratch<T, false> rows;
     float4 align;
-    T cst[NC];
+    T cst[MARCH_BLOCK / 32 * NC];
     __device__ U() {}
   } sh;
   // row blocks among the first b blocks: b rows / blocks
@@ -639,12 +644,15 @@ __global__ void __launch_bounds__(MARCH_BLOCK, sizeof(T) == 4 ? 4 : 2)
     rows_block<T, OP, STK, false>(L, mc, fl, a, (int)r0, sh.rows, a.partial);
     return;
   }
-  const int q = (int)(b - r0), macro = q / per_macro, block = q - macro * per_macro;
+  // a macro's columns: per_macro blocks, or `threads` threads of one
+  const int q = (int)(b - r0), part = threadIdx.x / threads;
+  const int macro = threads < MARCH_BLOCK ? q * (MARCH_BLOCK / threads) + part : q / per_macro;
+  const int block = threads < MARCH_BLOCK ? 0 : q - macro * per_macro;
   double* partial = a.partial ? a.partial + RowBlocks<T, STK>(L).partials() + q : nullptr;
   if constexpr (sizeof(T) == 4)
-    march2_block<OP, GEN, STK, KB>(L, mc, macro, block, fl, a, sh.cst, partial);
+    march2_block<OP, GEN, STK, KB>(L, mc, macro, block, threads, fl, a, sh.cst + part * NC, partial);
   else
-    march_block<T, OP, GEN, STK>(L, mc, macro, block, fl, a, sh.cst, partial);
+    march_block<T, OP, GEN, STK>(L, mc, macro, block, threads, fl, a, sh.cst + part * NC, partial);
 }
 
 template <typename T, int OP, int STK>
@@ -653,8 +661,13 @@ int launch(const LevelDev& L, const MacroConsts<T>* mc, const OpFlags& fl, const
   const bool gen = !(fl.physical == 1 && fl.khat_edge == 0);
   const RowBlocks<T, STK> R(L);
   const int columns = L.ncolumns[sizeof(T) == 8];
-  const int per = std::max(1, (columns + MARCH_BLOCK - 1) / MARCH_BLOCK);
-  const int64_t inner = columns > 0 ? (int64_t)per * L.nmacro : 0;
+  // Macros of few columns (8 or 4 intervals per edge) share a block: a block each left one of its warps busy
+  // (FP32 apply on 3072 macros of 4 / 8 intervals 105 / 123 us, so 71 / 98).  In FP64 only with more macros
+  // than SMs: a warp's FP64 instructions fill an SM (48 macros of 8 intervals 29 us a block each, 37 so).
+  const bool share = sizeof(T) == 4 || L.nmacro > 152;
+  const int threads = share && columns <= 32 ? 32 : share && columns <= 64 ? 64 : MARCH_BLOCK;
+  const int per = std::max(1, (columns + threads - 1) / threads), macros = MARCH_BLOCK / threads;
+  const int64_t inner = columns > 0 ? (int64_t)per * ((L.nmacro + macros - 1) / macros) : 0;
   if (partial_count) *partial_count = inner + R.partials();
   if (inner + R.total == 0) return 0;
   if (inner + R.total > INT32_MAX) return (int)cudaErrorInvalidValue;
@@ -662,14 +675,14 @@ int launch(const LevelDev& L, const MacroConsts<T>* mc, const OpFlags& fl, const
   // a kernel with the variant and khat rule folded in (FP64: 1.77 against 1.94 ms for a residual on
   // 129^3 nodes), but for FP32 Stokes, where the run-time flags do not show
   if constexpr (sizeof(T) == 4 && STK) {
-    k_sweep<T, OP, 1, STK, 0><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, R.total);
+    k_sweep<T, OP, 1, STK, 0><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, threads, R.total);
   } else {
     if (gen)
-      k_sweep<T, OP, 1, STK, 0><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, R.total);
+      k_sweep<T, OP, 1, STK, 0><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, threads, R.total);
     else if (sizeof(T) == 4 && a.k16)
-      k_sweep<T, OP, 0, STK, (sizeof(T) == 4)><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, R.total);
+      k_sweep<T, OP, 0, STK, (sizeof(T) == 4)><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, threads, R.total);
     else
-      k_sweep<T, OP, 0, STK, 0><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, R.total);
+      k_sweep<T, OP, 0, STK, 0><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, threads, R.total);
   }
   return (int)cudaGetLastError();
 }

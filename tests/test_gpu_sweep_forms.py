@@ -1,6 +1,7 @@
-"""The one-launch sweep where its layout changes with the level: faces and edges of few nodes, columns
-of one, two and more points in FP64 and of more than two in FP32.  Against the interior kernels of
-hhg_set_interior_kernel (which share the skeleton rows), and on coarse levels against the oracle.
+"""The one-launch sweep where its layout changes with the level: macros of few columns that share a block, faces
+and edges of few nodes, columns of one, two and more points in FP64 and of more than two in FP32.  Against
+the interior kernels of hhg_set_interior_kernel (which share the skeleton rows), and on coarse levels
+against the oracle.
 
 Tolerances.  FP64: two sums of the same terms, 1e-11 of the largest value as in test_gpu_rows.py.  FP32: the
 rounding bound of test_gpu_parity.py is 64 2^-24 sum_j |A_ij| |x_j - x_i|; for random x the 42 terms of a row
@@ -20,6 +21,10 @@ from test_gpu_parity import FP32_C, _fp32_scale, _kfun, _oracle
 pytestmark = pytest.mark.gpu
 
 F64, F32 = 1e-11, 2 * 10 * FP32_C
+
+
+def _box162():
+    return hi.kuhn_box(3, 3, 3)
 
 
 def _close(got, want, comps, tol):
@@ -47,9 +52,9 @@ def _sweeps(ctx, comps, dt, tdt, tol, kernels):
     return x, f
 
 
-@pytest.mark.parametrize("builder,level", [(hi.kuhn_cube, 2), (hi.kuhn_cube, 3), (hi.unit_tet, 2), (hi.unit_tet, 4),
-                                           (hi.unit_tet, 7)],
-                         ids=["cube_l2", "cube_l3", "one_l2", "one_l4", "one_l7"])
+@pytest.mark.parametrize("builder,level", [(hi.kuhn_cube, 2), (hi.kuhn_cube, 3), (hi.unit_tet, 2), (_box162, 2),
+                                           (_box162, 3), (hi.unit_tet, 4), (hi.unit_tet, 7)],
+                         ids=["cube_l2", "cube_l3", "one_l2", "box_l2", "box_l3", "one_l4", "one_l7"])
 @pytest.mark.parametrize("problem", [{}, dict(khat=B.KHAT_EDGE), dict(kind=B.STOKES)],
                          ids=["elasticity", "edge", "stokes"])
 def test_sweeps_equal_interior_kernels(builder, level, problem):
