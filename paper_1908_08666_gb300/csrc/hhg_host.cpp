@@ -796,8 +796,6 @@ void upload_level(hhg_ctx* c, LevelHost& L) {
   D.tiles3 = L.d_tiles3.as<int32_t>();
   for (int q = 0; q < 9; ++q) D.gs_ptr[q] = L.gs_ptr[q];
   D.gs_points = L.d_gs_points.as<int32_t>();
-  D.nskel_entries = (int64_t)L.skel_entries.size();
-  D.skel_entries = L.d_skel_entries.as<int64_t>();
   D.nskel = (int32_t)L.skel_dir.size();
   D.skel_ptr = L.d_skel_ptr.as<int32_t>();
   D.skel_inc = L.d_skel_inc.as<SkelInc>();

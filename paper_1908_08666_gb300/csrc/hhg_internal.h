@@ -244,8 +244,6 @@ struct LevelDev {
   // 4 (i % 2) + 2 (j % 2) + (k % 2), colour c's at [gs_ptr[c], gs_ptr[c+1])
   int32_t gs_ptr[9];
   const int32_t* gs_points;
-  int64_t nskel_entries;           // entries of skeleton nodes (every copy)
-  const int64_t* skel_entries;
   const int32_t* tiles_int;  // packed (k << 20) | (j0 << 10) | i0
   const int32_t* tiles_all;
   int32_t nskel;

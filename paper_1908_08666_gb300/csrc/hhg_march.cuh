@@ -269,20 +269,17 @@ struct March {
   T pprev;  // (Stokes) pressure of the column's previous point
 };
 
-// A block of columns of one macro (LevelDev::columns, FP64), or part of a block of several macros'
-// columns: `threads` threads, a power of two.  cst: 7 MARCH_C values, of this macro's threads.
+// A block of columns of one macro (LevelDev::columns, FP64); cst: 7 MARCH_C values.
 template <typename T, int OP, int GEN, int STK>
 __device__ __forceinline__ void march_block(const LevelDev& L, const MacroConsts<T>* __restrict__ mc, const int macro,
-                                            const int block, const int threads, const OpFlags& fl,
-                                            const SweepArgs<T>& a, T* cst, double* partial) {
-  const int own = threadIdx.x & (threads - 1);
-  if (macro < L.nmacro)
-    for (int q = own; q < 7 * MARCH_C<STK>; q += threads) {
-      const int d = q / MARCH_C<STK>, r = q - d * MARCH_C<STK>;
-      cst[q] = __ldg(&mc[macro].mar[d][r]);
-    }
+                                            const int block, const OpFlags& fl, const SweepArgs<T>& a, T* cst,
+                                            double* partial) {
+  for (int q = threadIdx.x; q < 7 * MARCH_C<STK>; q += MARCH_BLOCK) {
+    const int d = q / MARCH_C<STK>, r = q - d * MARCH_C<STK>;
+    cst[q] = __ldg(&mc[macro].mar[d][r]);
+  }
   __syncthreads();
-  const int t = macro < L.nmacro ? block * threads + own : INT32_MAX;
+  const int t = block * MARCH_BLOCK + threadIdx.x;
   double r2 = 0.0;
   if (t < L.ncolumns[1]) {
     const int32_t col = L.columns[1][t];
@@ -544,19 +541,27 @@ struct March2 {
   }
 };
 
-// As march_block; cst: 7 MARCH2_C values.
-template <int OP, int GEN, int STK, int KB>
+// As march_block; cst: 7 MARCH2_C values, and with SHARE > 0 as many for each of the block's macros: it takes
+// macros `macro` .. with all their columns, 2^SHARE threads each.
+template <int OP, int GEN, int STK, int KB, int SHARE>
 __device__ __forceinline__ void march2_block(const LevelDev& L, const MacroConsts<float>* __restrict__ mc,
-                                             const int macro, const int block, const int threads, const OpFlags& fl,
+                                             int macro, const int block, const OpFlags& fl,
                                              const SweepArgs<float>& a, float* cst, double* partial) {
-  const int own = threadIdx.x & (threads - 1);
-  if (macro < L.nmacro)
-    for (int r = own; r < 7 * MARCH2_C<STK>; r += threads) {
-      const int d = r / MARCH2_C<STK>, w = r - d * MARCH2_C<STK>;
-      cst[r] = w < 8 ? (w < 6 ? __ldg(&mc[macro].mar[d][w]) : 0.0f) : __ldg(&mc[macro].mar[d][6 + (w - 8) / 2]);
-    }
+  constexpr int NC = 7 * MARCH2_C<STK>;
+  for (int r = threadIdx.x; r < (SHARE ? MARCH_BLOCK >> SHARE : 1) * NC; r += MARCH_BLOCK) {
+    const int m = SHARE ? macro + r / NC : macro, d = (SHARE ? r % NC : r) / MARCH2_C<STK>;
+    const int w = (SHARE ? r % NC : r) - d * MARCH2_C<STK>;
+    if (SHARE && m >= L.nmacro) break;
+    cst[r] = w < 8 ? (w < 6 ? __ldg(&mc[m].mar[d][w]) : 0.0f) : __ldg(&mc[m].mar[d][6 + (w - 8) / 2]);
+  }
   __syncthreads();
-  const int t = macro < L.nmacro ? block * threads + own : INT32_MAX;
+  int t = block * MARCH_BLOCK + threadIdx.x;
+  if constexpr (SHARE > 0) {
+    const int part = threadIdx.x >> SHARE;
+    macro += part;
+    cst += part * NC;
+    t = macro < L.nmacro ? threadIdx.x & ((1 << SHARE) - 1) : INT32_MAX;
+  }
   double r2 = 0.0;
   if (t < L.ncolumns[0]) {
     const int32_t col = L.columns[0][t];
@@ -621,19 +626,20 @@ __device__ __forceinline__ void march2_block(const LevelDev& L, const MacroConst
 
 // ---------------------------------------------------------------------------
 // A whole sweep in one launch: blocks of the macro interiors with the skeleton's blocks spread evenly
-// between them.  The skeleton rows wait for memory most of the time (strided faces) and the interiors
-// for the arithmetic pipes, so they run well side by side; as two launches on two streams they did
-// not, since either one's blocks fill the registers of every SM.
+// between them.  One launch for latency's sake: on small levels it is one wave, where two launches on two
+// streams followed one another, since either one's blocks fill the registers of every SM.  On large levels
+// the parts add up all the same (FP32 apply on 257^3 nodes: interiors alone 330 us, rows alone 66, together
+// 390): a row block waits for memory most of the time, in a slot that a march block could use.
 // ---------------------------------------------------------------------------
-template <typename T, int OP, int GEN, int STK, int KB>
+template <typename T, int OP, int GEN, int STK, int KB, int SHARE = 0>
 __global__ void __launch_bounds__(MARCH_BLOCK, sizeof(T) == 4 ? 4 : 2)
     k_sweep(const LevelDev L, const MacroConsts<T>* __restrict__ mc, const OpFlags fl, const SweepArgs<T> a,
-            const int per_macro, const int threads, const int rows) {
+            const int per_macro, const int rows) {
   constexpr int NC = 7 * (sizeof(T) == 4 ? MARCH2_C<STK> : MARCH_C<STK>);
   __shared__ union U {
     RowScratch<T, false> rows;
     float4 align;
-    T cst[MARCH_BLOCK / 32 * NC];
+    T cst[(SHARE ? MARCH_BLOCK >> SHARE : 1) * NC];
     __device__ U() {}
   } sh;
   // row blocks among the first b blocks: b rows / blocks
@@ -644,15 +650,13 @@ __global__ void __launch_bounds__(MARCH_BLOCK, sizeof(T) == 4 ? 4 : 2)
     rows_block<T, OP, STK, false>(L, mc, fl, a, (int)r0, sh.rows, a.partial);
     return;
   }
-  // a macro's columns: per_macro blocks, or `threads` threads of one
-  const int q = (int)(b - r0), part = threadIdx.x / threads;
-  const int macro = threads < MARCH_BLOCK ? q * (MARCH_BLOCK / threads) + part : q / per_macro;
-  const int block = threads < MARCH_BLOCK ? 0 : q - macro * per_macro;
+  const int q = (int)(b - r0), macro = SHARE ? q * (MARCH_BLOCK >> SHARE) : q / per_macro;
+  const int block = SHARE ? 0 : q - macro * per_macro;
   double* partial = a.partial ? a.partial + RowBlocks<T, STK>(L).partials() + q : nullptr;
   if constexpr (sizeof(T) == 4)
-    march2_block<OP, GEN, STK, KB>(L, mc, macro, block, threads, fl, a, sh.cst + part * NC, partial);
+    march2_block<OP, GEN, STK, KB, SHARE>(L, mc, macro, block, fl, a, sh.cst, partial);
   else
-    march_block<T, OP, GEN, STK>(L, mc, macro, block, threads, fl, a, sh.cst + part * NC, partial);
+    march_block<T, OP, GEN, STK>(L, mc, macro, block, fl, a, sh.cst, partial);
 }
 
 template <typename T, int OP, int STK>
@@ -661,28 +665,35 @@ int launch(const LevelDev& L, const MacroConsts<T>* mc, const OpFlags& fl, const
   const bool gen = !(fl.physical == 1 && fl.khat_edge == 0);
   const RowBlocks<T, STK> R(L);
   const int columns = L.ncolumns[sizeof(T) == 8];
-  // Macros of few columns (8 or 4 intervals per edge) share a block: a block each left one of its warps busy
-  // (FP32 apply on 3072 macros of 4 / 8 intervals 105 / 123 us, so 71 / 98).  In FP64 only with more macros
-  // than SMs: a warp's FP64 instructions fill an SM (48 macros of 8 intervals 29 us a block each, 37 so).
-  const bool share = sizeof(T) == 4 || L.nmacro > 152;
-  const int threads = share && columns <= 32 ? 32 : share && columns <= 64 ? 64 : MARCH_BLOCK;
-  const int per = std::max(1, (columns + threads - 1) / threads), macros = MARCH_BLOCK / threads;
-  const int64_t inner = columns > 0 ? (int64_t)per * ((L.nmacro + macros - 1) / macros) : 0;
+  // Macros of up to 32 columns (4 or 8 intervals per edge) share blocks of four in FP32: a block each left one of
+  // its warps busy (apply on 3072 macros of 4 / 8 intervals 105 / 123 us, so 71 / 98).  Only with more macros
+  // than SMs (fewer blocks all run at once), and not in FP64, where a warp's instructions fill an SM and the
+  // rows are most of such a sweep (831 us against 891).  A kernel of its own, with the run-time flags and the
+  // FP32 copy of a BF16 coefficient: the general index arithmetic cost the large sweeps 4 to 7 %.
+  const bool share = sizeof(T) == 4 && L.nmacro > 152 && columns <= 32;
+  const int per = std::max(1, (columns + MARCH_BLOCK - 1) / MARCH_BLOCK);
+  const int64_t inner = columns == 0 ? 0 : share ? (L.nmacro + 3) / 4 : (int64_t)per * L.nmacro;
   if (partial_count) *partial_count = inner + R.partials();
   if (inner + R.total == 0) return 0;
   if (inner + R.total > INT32_MAX) return (int)cudaErrorInvalidValue;
   const unsigned g = (unsigned)(inner + R.total);
+  if constexpr (sizeof(T) == 4) {
+    if (share) {
+      k_sweep<T, OP, 1, STK, 0, 5><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, R.total);
+      return (int)cudaGetLastError();
+    }
+  }
   // a kernel with the variant and khat rule folded in (FP64: 1.77 against 1.94 ms for a residual on
   // 129^3 nodes), but for FP32 Stokes, where the run-time flags do not show
   if constexpr (sizeof(T) == 4 && STK) {
-    k_sweep<T, OP, 1, STK, 0><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, threads, R.total);
+    k_sweep<T, OP, 1, STK, 0><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, R.total);
   } else {
     if (gen)
-      k_sweep<T, OP, 1, STK, 0><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, threads, R.total);
+      k_sweep<T, OP, 1, STK, 0><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, R.total);
     else if (sizeof(T) == 4 && a.k16)
-      k_sweep<T, OP, 0, STK, (sizeof(T) == 4)><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, threads, R.total);
+      k_sweep<T, OP, 0, STK, (sizeof(T) == 4)><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, R.total);
     else
-      k_sweep<T, OP, 0, STK, 0><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, threads, R.total);
+      k_sweep<T, OP, 0, STK, 0><<<g, MARCH_BLOCK, 0, s>>>(L, mc, fl, a, per, R.total);
   }
   return (int)cudaGetLastError();
 }

@@ -283,7 +283,7 @@ void smooth(hhg_ctx* c, int l, int steps, const T* f, T* x) {
       a.out = oth;
       a.omega = c->mg.omega;
       CK(launch_rows<T>(L.dev, consts_dev<T>(L), OP_JACOBI, c->flags, a, c->stream, 0, nullptr));
-      CK(launch_copy_entries<T>(L.dev.nskel_entries, L.dev.skel_entries, 3, L.entries, oth, x, c->stream));
+      CK(launch_copy_entries<T>((int64_t)L.skel_entries.size(), L.d_skel_entries.as<int64_t>(), 3, L.entries, oth, x, c->stream));
       CK(launch_gs<T>(L.dev, consts_dev<T>(L), c->flags, f, kptr<T>(L), x, c->stream));
     }
   } else {

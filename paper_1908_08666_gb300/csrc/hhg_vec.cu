@@ -82,12 +82,16 @@ __global__ void k_prolong_add(const LevelDev Lf, const LevelDev Lc, const T* __r
     a[q] = __ldg(c + ca + q * Ec);
     b[q] = __ldg(c + cb + q * Ec);
   }
-  // the mean and its sum as one fma (halving is exact): FP64 additions, not the loads, bound the FP64 form
+  // FP64: the mean and its sum as one fma (halving is exact): its additions, not the loads, bound that form
   // (129^3 nodes 57 us with three operations per value, 37 with two)
   const bool edge = pX | pY | pZ;
-  const T w = edge ? (T)0.5 : (T)1;
 #pragma unroll
-  for (int q = 0; q < COMPS; ++q) f[q * Ef] = fma(w, edge ? a[q] + b[q] : a[q], v[q]);
+  for (int q = 0; q < COMPS; ++q) {
+    if constexpr (sizeof(T) == 8)
+      f[q * Ef] = fma(edge ? (T)0.5 : (T)1, edge ? a[q] + b[q] : a[q], v[q]);
+    else
+      f[q * Ef] = v[q] + (edge ? (T)0.5 * (a[q] + b[q]) : a[q]);
+  }
 }
 
 // coarse macro-interior points: rc(p) = rf(2p) + 1/2 sum_d rf(2p + d)
