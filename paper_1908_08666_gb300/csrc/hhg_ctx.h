@@ -518,6 +518,12 @@ inline OpFlags sweep_flags(hhg_ctx* c, const LevelHost& L, bool pairs) {
   return f;
 }
 
+// The FP32 diagonal on large macros is taken from the point kernels, a launch per macro of at least as many
+// blocks: it needs only the coefficient, so the arithmetic that the march saves does not count, and the march
+// writes in worse order (cube of 129^3 / 257^3 nodes 31 / 207 us, so 27 / 175; two macros of 128 intervals per
+// edge 14 and 11).
+constexpr int DIAG_POINT_BLOCKS = 1000;
+
 // One operator sweep on a level.  By default one launch (k_sweep).  Else (the nodal and stored
 // variants, interior kernels chosen by hand) the macro-interior
 // rows on `stream` (all macros in one launch, or one launch per macro, every second one on aux[1]
@@ -533,7 +539,8 @@ void sweep(hhg_ctx* c, int level, OpKind op, SweepArgs<T> a, double* norm2) {
   if (std::is_same<T, float>::value && c->coeff_bf16) a.k16 = L.d_k16.as<uint16_t>();
   if (norm2) a.partial = c->scratch.as<double>();
   int64_t np = 0;
-  const OpFlags fl = sweep_flags(c, L, std::is_same<T, float>::value);
+  OpFlags fl = sweep_flags(c, L, std::is_same<T, float>::value);
+  if (op == OP_DIAG && std::is_same<T, float>::value && L.dev.ntiles_pair >= DIAG_POINT_BLOCKS) fl.whole = 0;
   if (fl.whole) {
     std::array<cudaEvent_t, 2> pi{};
     if (c->prof) {

@@ -637,7 +637,7 @@ __global__ void __launch_bounds__(MARCH_BLOCK, sizeof(T) == 4 ? 4 : 2)
             const int per_macro, const int rows) {
   constexpr int NC = 7 * (sizeof(T) == 4 ? MARCH2_C<STK> : MARCH_C<STK>);
   __shared__ union U {
-    RowScratch<T, false> rows;
+    RowScratch<T> rows;
     float4 align;
     T cst[(SHARE ? MARCH_BLOCK >> SHARE : 1) * NC];
     __device__ U() {}
@@ -647,7 +647,7 @@ __global__ void __launch_bounds__(MARCH_BLOCK, sizeof(T) == 4 ? 4 : 2)
   const uint32_t r0 = (uint32_t)((uint64_t)b * (uint32_t)rows / gridDim.x);
   const uint32_t r1 = (uint32_t)((uint64_t)(b + 1) * (uint32_t)rows / gridDim.x);
   if (r1 != r0) {
-    rows_block<T, OP, STK, false>(L, mc, fl, a, (int)r0, sh.rows, a.partial);
+    rows_block<T, OP, STK>(L, mc, fl, a, (int)r0, sh.rows, a.partial);
     return;
   }
   const int q = (int)(b - r0), macro = SHARE ? q * (MARCH_BLOCK >> SHARE) : q / per_macro;

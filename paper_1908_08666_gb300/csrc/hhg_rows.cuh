@@ -1,6 +1,6 @@
 // Rows of nodes on the macro skeleton (faces, edges and vertices of the macro mesh, Sec. 2.2 of
-// arXiv 1908.08666): device code of the skeleton part of a sweep, run by k_rows alone and by k_sweep
-// in blocks between those of the macro interiors.
+// arXiv 1908.08666): device code of the skeleton part of a sweep, run by k_rows alone (hhg_rows_launch.cuh)
+// and by k_sweep in blocks between those of the macro interiors.
 //
 // A lane takes one incidence of a node (the node seen from one of the macros that hold it) and
 // evaluates that macro's part of the row; the parts are summed in an order that is the same for every
@@ -247,10 +247,10 @@ __device__ __forceinline__ bool prim_dir_inward(int F, int d) {
   return lattice_interior(16, prim_coord(F, 1) + dir_di(d), prim_coord(F, 2) + dir_dj(d), prim_coord(F, 3) + dir_dk(d));
 }
 
-// Which form rows inside faces and edges take.  FP32 sweeps: prim_incidence, unrolled.  FP64, and FP32 rows
-// in a launch of their own (LOOP): loop_incidence; in FP64 two warps take a side of a face block.
-template <typename T, bool LOOP>
-constexpr bool ROWS_UNROLLED = sizeof(T) == 4 && !LOOP;
+// Which form rows inside faces and edges take.  FP32: prim_incidence, unrolled.  FP64: loop_incidence, and two
+// warps take a side of a face block.
+template <typename T>
+constexpr bool ROWS_UNROLLED = sizeof(T) == 4;
 template <typename T>
 constexpr int FACE_GROUPS = sizeof(T) == 8 ? 2 : 1;
 
@@ -262,10 +262,10 @@ struct RowColumns {
 };
 
 struct NoColumns {};
-template <typename T, bool LOOP>
+template <typename T>
 struct RowScratch {
   T share[6 * ROWS_BLOCK];  // sums that warps exchange
-  std::conditional_t<ROWS_UNROLLED<T, LOOP>, NoColumns, RowColumns<T>> columns;
+  std::conditional_t<ROWS_UNROLLED<T>, NoColumns, RowColumns<T>> columns;
 };
 
 // The same sums as prim_incidence in a loop over the directions, with run-time ring indices.  FP64: a
@@ -428,9 +428,9 @@ __device__ __forceinline__ void write_row(const SweepArgs<T>& a, int64_t e, int6
 // the sums are exchanged through shared memory (added in the same order in every warp) and each side's
 // first warp writes its copies.  All threads of the launch's block call this together (b < 0: nothing
 // to do).
-template <typename T, int OP, int STK, bool LOOP>
+template <typename T, int OP, int STK>
 __device__ __forceinline__ double face_block(const LevelDev& L, const MacroConsts<T>* __restrict__ mc,
-                                             const OpFlags& fl, const SweepArgs<T>& a, int b, RowScratch<T, LOOP>& sh) {
+                                             const OpFlags& fl, const SweepArgs<T>& a, int b, RowScratch<T>& sh) {
   constexpr bool DIAG = OP == OP_JACOBI || OP == OP_CHEBY || OP == OP_DIAG;
   constexpr int G = FACE_GROUPS<T>;
   const int lane = threadIdx.x & 31, side = (threadIdx.x >> 5) & 1, group = G > 1 ? (threadIdx.x >> 6) % G : 0;
@@ -448,7 +448,7 @@ __device__ __forceinline__ double face_block(const LevelDev& L, const MacroConst
     const T* px = a.x + (int64_t)m * L.nt;
     const T* pk = a.k + (int64_t)m * L.nt;
     const int64_t E = L.entries;
-    if constexpr (!ROWS_UNROLLED<T, LOOP>) {
+    if constexpr (!ROWS_UNROLLED<T>) {
       loop_incidence<T, DIAG, STK>(L, mc[m], px, pk, fl, P.i, P.j, P.k, vel, group, G, sh.columns, s);
     } else {
       switch (side == 0 ? B.face[0] : B.face[1]) {
@@ -493,9 +493,9 @@ __device__ __forceinline__ double face_block(const LevelDev& L, const MacroConst
 
 // A block of up to 32 nodes of one macro edge: warp w takes the macros w, w + 4, ... that hold the edge,
 // the warps' sums are added in order, and each warp writes its macros' copies.
-template <typename T, int OP, int STK, bool LOOP>
+template <typename T, int OP, int STK>
 __device__ __forceinline__ double edge_block(const LevelDev& L, const MacroConsts<T>* __restrict__ mc,
-                                             const OpFlags& fl, const SweepArgs<T>& a, int b, RowScratch<T, LOOP>& sh) {
+                                             const OpFlags& fl, const SweepArgs<T>& a, int b, RowScratch<T>& sh) {
   constexpr bool DIAG = OP == OP_JACOBI || OP == OP_CHEBY || OP == OP_DIAG;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const EdgeBlock B = L.edge_blocks[STK][b];
@@ -509,7 +509,7 @@ __device__ __forceinline__ double edge_block(const LevelDev& L, const MacroConst
     const T* pk = a.k + (int64_t)S.macro * L.nt;
     const MacroConsts<T>& C = mc[S.macro];
     if (!valid) continue;
-    if constexpr (!ROWS_UNROLLED<T, LOOP>) {
+    if constexpr (!ROWS_UNROLLED<T>) {
       loop_incidence<T, DIAG, STK>(L, C, px, pk, fl, i, j, k, vel, 0, 1, sh.columns, s);
     } else {
       switch (S.edge) {
@@ -558,9 +558,9 @@ __device__ __forceinline__ double edge_block(const LevelDev& L, const MacroConst
 
 // A block of macro vertices (EvWarp): the sums of a warp by a butterfly, those of a
 // node's warps in order, and the node's threads write its copies.
-template <typename T, int OP, int STK, bool LOOP>
+template <typename T, int OP, int STK>
 __device__ __forceinline__ double ev_block(const LevelDev& L, const MacroConsts<T>* __restrict__ mc, const OpFlags& fl,
-                                           const SweepArgs<T>& a, int b, RowScratch<T, LOOP>& sh) {
+                                           const SweepArgs<T>& a, int b, RowScratch<T>& sh) {
   constexpr bool DIAG = OP == OP_JACOBI || OP == OP_CHEBY || OP == OP_DIAG;
   const EvWarp W = L.ev_warps[STK][ROWS_WARPS * b + (threadIdx.x >> 5)];
   RowSum<T> s;
@@ -639,9 +639,9 @@ struct RowBlocks {
 };
 
 // Block b of them; its partial sum of |r|^2 goes to partial[b].
-template <typename T, int OP, int STK, bool LOOP>
+template <typename T, int OP, int STK>
 __device__ __forceinline__ void rows_block(const LevelDev& L, const MacroConsts<T>* __restrict__ mc, const OpFlags& fl,
-                                           const SweepArgs<T>& a, int b, RowScratch<T, LOOP>& sh, double* partial) {
+                                           const SweepArgs<T>& a, int b, RowScratch<T>& sh, double* partial) {
   const RowBlocks<T, STK> R(L);
   const int64_t E = L.entries;
   if (b >= R.partials()) {
@@ -662,11 +662,11 @@ __device__ __forceinline__ void rows_block(const LevelDev& L, const MacroConsts<
   double r2;
   if (b >= R.ev_blocks + R.edge_blocks) {
     const int f = (b - R.ev_blocks - R.edge_blocks) * R.FACES + (R.FACES > 1 ? threadIdx.x >> 6 : 0);
-    r2 = face_block<T, OP, STK, LOOP>(L, mc, fl, a, f < R.nfaces ? f : -1, sh);
+    r2 = face_block<T, OP, STK>(L, mc, fl, a, f < R.nfaces ? f : -1, sh);
   } else if (b >= R.ev_blocks) {
-    r2 = edge_block<T, OP, STK, LOOP>(L, mc, fl, a, b - R.ev_blocks, sh);
+    r2 = edge_block<T, OP, STK>(L, mc, fl, a, b - R.ev_blocks, sh);
   } else {
-    r2 = ev_block<T, OP, STK, LOOP>(L, mc, fl, a, b, sh);
+    r2 = ev_block<T, OP, STK>(L, mc, fl, a, b, sh);
   }
   if (OP == OP_RESID && partial != nullptr) block_sum_store<T>(r2, partial + b);
 }
