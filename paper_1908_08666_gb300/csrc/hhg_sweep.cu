@@ -1033,10 +1033,9 @@ int noalloc_scratch_address(int device, double** ptr) {
   return 0;
 }
 
-// a block of rows holds at least one node, except that a vertex of more than eight macros takes several
+// a block of rows holds at least one node (a vertex of many macros takes several warps, of one block)
 int64_t noalloc_partials_needed(const LevelDev& L) {
-  const int64_t rows = (int64_t)L.nev_blocks[0] + L.nedge_blocks[0] + L.nface_blocks[0];
-  return (int64_t)L.nmacro * L.ntiles_lin + std::max((int64_t)L.nface_nodes + L.nev, rows);
+  return (int64_t)L.nmacro * L.ntiles_lin + L.nface_nodes + L.nev;
 }
 
 template <typename T>

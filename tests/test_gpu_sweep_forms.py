@@ -148,3 +148,26 @@ def test_columns_of_four_points_in_fp64():
         _sweeps(ctx, 3, B.F64, ctx.torch.float64, F64, (0, 3))
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("builder,level,problem", [(_box162, 2, {}), (_box162, 3, {}), (hi.unit_tet, 2, {}),
+                                                   (hi.skewed_pair, 4, dict(variant=B.STORED)), (hi.kuhn_cube, 7, {})],
+                         ids=["box_l2", "box_l3", "one_l2", "pair_stored", "cube_l7"])
+def test_noalloc_residual(builder, level, problem):
+    """The residual without allocation against hhg_residual, up to the largest levels that its scratch takes;
+    tolerances of test_zz_no_alloc.py."""
+    ctx = Ctx(*builder(), level, dict(nu=0.3, **problem))
+    try:
+        t = ctx.torch
+        ctx.set_k(_kfun(ctx.coords_u))
+        for dt, tdt, tol in ((B.F64, t.float64, 1e-12), (B.F32, t.float32, FP32_C)):
+            x = ctx.to_lib(hi.node_noise(ctx.coords_u, seed=3), tdt, 3)
+            f = ctx.to_lib(hi.node_noise(ctx.coords_u, seed=4), tdt, 3)
+            want, got = t.empty_like(x), t.full_like(x, float("nan"))
+            n_want = B.hhg_residual(ctx.h, level, dt, f, x, want, want_norm=True)
+            n_got = B.hhg_residual_noalloc(ctx.h, level, dt, f, x, got)
+            t.cuda.synchronize()
+            _close(got, want, 3, tol)
+            assert abs(n_got - n_want) <= (1e-12 if dt == B.F64 else 1e-5) * n_want
+    finally:
+        ctx.close()
