@@ -593,8 +593,8 @@ hhg_status hhg_profile(hhg_ctx* ctx, int enable, double* ms_host, int64_t* launc
  * memory; 3 the point kernels, all macros in one launch (each block copies its macro's stencil to
  * shared memory); 1 a block per 30 x 4 x 4 box of lattice points that stages the box plus its
  * one-point halo in shared memory (asynchronous copies) and reads every neighbour from there.  The
- * Stokes sweeps follow the same choice (1 as 3 or 2); the colour passes of the hybrid Gauss-Seidel smoother
- * do not depend on it.  Errors: ARG for another value. */
+ * Stokes sweeps follow the same choice (1 as 2), the FP32 diagonal of large macros takes 2 for 0; the colour
+ * passes of the hybrid Gauss-Seidel smoother do not depend on it.  Errors: ARG for another value. */
 hhg_status hhg_set_interior_kernel(hhg_ctx* ctx, int kernel);
 
 /* FP32 FMA issue-rate probe, a measurement aid with no counterpart in the paper: the

@@ -325,7 +325,8 @@ def hhg_profile(ctx, enable, read=False):
 
 
 def hhg_set_interior_kernel(ctx, kernel):
-    """0: direct global loads (FP32 on point pairs, packed arithmetic), 1: shared-memory tile."""
+    """0: the whole sweep in one launch (default); the interiors beside the skeleton rows: 1 shared-memory tiles,
+    2 a point-kernel launch per macro, 3 one launch for all macros."""
     _check(ctx, load().hhg_set_interior_kernel(ctx, int(kernel)))
 
 
@@ -432,12 +433,13 @@ def hhg_learn_num_params():
 
 
 def hhg_learn_set_conv_kernel(ctx, kernel):
-    """0: warp-level MMA convolution (default), 1: tcgen05 per tile, 2: TMA + tcgen05 pipeline."""
+    """0: tcgen05 on four voxels per row, small grids warp-level MMA (default); 1: tcgen05 per tile, 2: TMA +
+    tcgen05 pipeline."""
     _check(ctx, load().hhg_learn_set_conv_kernel(ctx, int(kernel)))
 
 
 def hhg_learn_set_conv_wait(ctx, polls):
-    """Bound (polls) of the tensor-core convolution's wait for its MMAs; negative: the default."""
+    """Bound (polls) of the waits of convolutions 0 and 1 for their MMAs; negative: the default."""
     _check(ctx, load().hhg_learn_set_conv_wait(ctx, C.c_int64(int(polls))))
 
 

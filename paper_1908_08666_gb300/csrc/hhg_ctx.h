@@ -258,10 +258,9 @@ struct hhg_ctx {
   bool coeff_bf16 = false;     // the coefficient was given in BF16 (k16 holds it on every level)
   std::unique_ptr<LearnState> learn;
   OpFlags flags{1, 0, 0};
-  // macro-interior kernel choice (hhg_set_interior_kernel): 0 automatic, 1 shared-memory tile,
-  // 2 one launch per macro, 3 all macros in one launch
+  // sweep kernel (hhg_set_interior_kernel): 0 the whole sweep in one launch, 1 shared-memory tiles, 2 point
+  // kernels per macro, 3 point kernels over all macros
   int interior_kernel = 0;
-  int sm_count = 0;  // SMs of the device (read on first use)
   int strain_degree = 1;  // least-squares strain-rate fit on the skeleton (hhg_set_strain_fit)
   DevMem scratch;   // reduction partials
   DevMem scalar;    // device scalars
@@ -495,26 +494,14 @@ const T* stored_stencil(hhg_ctx* c, LevelHost& L) {
   return S.as<T>();
 }
 
-// The operator flags of a sweep on level L, with the launch shape of its macro-interior part:
-// all macros in one launch when chosen (interior kernel 3) or, automatically, when the mesh has
-// several macros and one macro's launch (FP32 point pairs or one point per thread) fills
-// fewer than two waves of four 128-thread blocks per SM.
-inline OpFlags sweep_flags(hhg_ctx* c, const LevelHost& L, bool pairs) {
+// The operator flags of a sweep with its launch shape (hhg_set_interior_kernel): the whole sweep in one launch
+// (0), the interiors of all macros in one launch (3) or a launch per macro (1, 2, and the nodal and stored
+// variants).
+inline OpFlags sweep_flags(hhg_ctx* c) {
   OpFlags f = c->flags;
-  f.batch = 0;
-  if (f.stored || f.nodal || f.tile || c->interior_kernel == 2) return f;
-  if (c->interior_kernel == 0) {
-    f.whole = 1;
-    return f;
-  }
-  if (c->interior_kernel == 3) {
-    f.batch = 1;
-    return f;
-  }
-  if (L.dev.nmacro < 2) return f;
-  if (c->sm_count == 0) CK(cudaDeviceGetAttribute(&c->sm_count, cudaDevAttrMultiProcessorCount, c->device));
-  const int per_macro = pairs ? L.dev.ntiles_pair : L.dev.ntiles_lin;
-  f.batch = per_macro < 2 * 4 * c->sm_count;
+  const bool per_macro = f.stored || f.nodal || f.tile || c->interior_kernel == 2;
+  f.whole = !per_macro && c->interior_kernel == 0;
+  f.batch = !per_macro && c->interior_kernel == 3;
   return f;
 }
 
@@ -539,7 +526,7 @@ void sweep(hhg_ctx* c, int level, OpKind op, SweepArgs<T> a, double* norm2) {
   if (std::is_same<T, float>::value && c->coeff_bf16) a.k16 = L.d_k16.as<uint16_t>();
   if (norm2) a.partial = c->scratch.as<double>();
   int64_t np = 0;
-  OpFlags fl = sweep_flags(c, L, std::is_same<T, float>::value);
+  OpFlags fl = sweep_flags(c);
   if (op == OP_DIAG && std::is_same<T, float>::value && L.dev.ntiles_pair >= DIAG_POINT_BLOCKS) fl.whole = 0;
   if (fl.whole) {
     std::array<cudaEvent_t, 2> pi{};

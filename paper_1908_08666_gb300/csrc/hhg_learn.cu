@@ -31,10 +31,6 @@ __device__ __forceinline__ uint32_t pack_pair(float lo, float hi) {
   return *reinterpret_cast<const uint32_t*>(&v);
 }
 
-__device__ __forceinline__ uint32_t pack_raw(unsigned short lo, unsigned short hi) {
-  return (uint32_t)lo | ((uint32_t)hi << 16);
-}
-
 // D += A * B, A 16x16 (row), B 16x8 (col), BF16 inputs, FP32 accumulators
 __device__ __forceinline__ void mma_bf16(float d[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0,
                                          uint32_t b1) {
@@ -590,7 +586,7 @@ __global__ void __launch_bounds__(CG_THREADS, 2)
 // stays at 81-90 us for four layers, where k_conv's grows with its blocks: forward pass, us, k_conv / this
 // kernel: 17^3 voxels (25 blocks) 57 / 81, 33^3 (162) 66 / 82, 129 x 33 x 32 (297) 73 / 90, 49^3 (338)
 // 82 / 83, 300 x 21^2 (450) 82 / 83; 5 x 160 x 165 (480) 92 / 81, 65^2 x 33 (578) 98 / 84, 65^3 (867)
-// 124 / 107.
+// 124 / 107.  (Both sides with a copy of the error flag after the pass, which took about 10 us and is gone.)
 constexpr int64_t CG_MIN_BLOCKS = 3 * 152;
 inline bool conv_tiling(GridShape s, ConvTiling& best) {
   const int64_t conv_blocks = (int64_t)((s.W + CT_X - 1) / CT_X) * ((s.H + CT_Y - 1) / CT_Y) * ((s.D + CT_Z - 1) / CT_Z) * s.B;

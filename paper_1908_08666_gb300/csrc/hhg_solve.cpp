@@ -517,7 +517,7 @@ double stokes_sweep(hhg_ctx* c, int l, OpKind op, const T* f, const T* x, T* out
   a.k = kptr<T>(L);
   if (norm) a.partial = c->scratch.as<double>();
   int64_t np = 0;
-  const OpFlags fl = sweep_flags(c, L, false);
+  const OpFlags fl = sweep_flags(c);
   if (fl.whole) {
     CK(launch_sweep_stokes<T>(L.dev, consts_dev<T>(L), op, fl, a, c->stream, &np));
   } else {
