@@ -996,7 +996,9 @@ def learned_bench(B, torch, dev, stream, train_level, eval_level, nseed, nrhs, i
     tf = flops / (ms * 1e-3) / 1e12
     out["conv_forward"] = {"grid": [D, H, W], "ms": round(ms, 4), "tflops": round(tf, 2), "peak_tflops": peak,
                            "frac": round(tf / peak, 4), "peak_source": src,
-                           "kernel": "k_conv_group (tcgen05.mma, four voxels per matrix row), 4 launches",
+                           "kernel": ("k_conv_group (tcgen05.mma, four voxels per matrix row), 4 launches"
+                                      if -(-W // 32) * -(-H // 4) * -(-D // 4) > 456 else
+                                      "k_conv (mma.sync on shared-memory tiles), 4 launches"),
                            "tcgen05": {"ms": round(ms_u, 4), "tflops": round(flops / (ms_u * 1e-3) / 1e12, 2),
                                        "frac": round(flops / (ms_u * 1e-3) / 1e12 / peak, 4),
                                        "kernel": "k_conv_umma (tcgen05.mma kind::f16, TMEM accumulators)"},

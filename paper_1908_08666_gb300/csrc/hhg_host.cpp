@@ -388,8 +388,8 @@ void cast_values(const S<double>& c, S<float>& o) {
 // face types, those next to the face's edges apart.  A face block has two sides, so the nodes of a face in
 // more than two macros (the mesh need not be a manifold) go to the vertices' list, and so do faces and edges of
 // up to VERTEX_LIKE nodes: three lanes of a block's 32 were busy there.  Apply on 3072 macros of 4 intervals per
-// edge, FP32 / FP64, us: elasticity 71 / 831 with blocks, 57 / 410 so, Stokes 123 / 1276 and 82 / 592; with
-// the edges of 8 intervals (7 nodes) too, elasticity on 3072 of those 98 / 1261 and 136 / 1367.
+// edge, FP32 / FP64, us: elasticity 71 / 890 with blocks, 58 / 460 so, Stokes 123 / 1346 and 82 / 646; with
+// the edges of 8 intervals (7 nodes) too, elasticity on 3072 of those in FP32 98 and 136.
 constexpr int VERTEX_LIKE = 3;
 void build_rows(LevelHost& L) {
   const int n = L.n;

@@ -666,7 +666,8 @@ int launch(const LevelDev& L, const MacroConsts<T>* mc, const OpFlags& fl, const
   const RowBlocks<T, STK> R(L);
   const int columns = L.ncolumns[sizeof(T) == 8];
   // Macros of up to 32 columns (4 or 8 intervals per edge) share blocks of four in FP32: a block each left one of
-  // its warps busy (apply on 3072 macros of 4 / 8 intervals 105 / 123 us, so 71 / 98).  Only with more macros
+  // its warps busy (apply on 3072 macros of 4 / 8 intervals 105 / 123 us; so, and with build_rows' rule for
+  // small faces and edges, 58 / 100).  Only with more macros
   // than SMs (fewer blocks all run at once), and not in FP64, where a warp's instructions fill an SM and the
   // rows are most of such a sweep (831 us against 891).  A kernel of its own, with the run-time flags and the
   // FP32 copy of a BF16 coefficient: the general index arithmetic cost the large sweeps 4 to 7 %.
